@@ -100,7 +100,7 @@ struct Context {
     std::mutex mu;
     cudaStream_t stream = nullptr;
     int sms = 0;
-    int occ[2][2][2][2] = {};  // [wide][mode][batch][compact] blocks per SM of the round kernel
+    int occ[3][2][2][2] = {};  // [variant][mode][batch][compact] blocks per SM of the round kernel
     int occ_part = 0;       // blocks per SM of the partition-mode round kernel
     int occ_ord[2] = {};    // blocks per SM of the ordered-mode round kernel [batch]
     int occ_peel = 0;       // blocks per SM of the peeling kernel
@@ -356,7 +356,7 @@ static int run(Context &C, const Problem &pb, int mode, uint64_t seed, const gc_
 
     // scratch sized by n; work-item buffers are sized after binning
     GC_TRY(ensure(C.col0, 8 * n, "vertex state"));
-    GC_TRY(ensure(C.col1, 8 * n, "vertex state"));
+    GC_TRY(ensure(C.col1, 8 * n + kDetPad, "vertex state"));
     GC_TRY(ensure(C.items, 4 * n, "worklist"));
     GC_TRY(ensure(C.small0, 4 * n, "worklist"));
     GC_TRY(ensure(C.small1, 4 * n, "worklist"));
@@ -407,6 +407,8 @@ static int run(Context &C, const Problem &pb, int mode, uint64_t seed, const gc_
     P.seed = seed;
     P.col0 = C.col0.as<uint64_t>();
     P.col1 = C.col1.as<uint64_t>();
+    set_det_state(P, C.col0.p, C.col1.p, static_cast<size_t>(n));
+    P.ci_len = pb.nnz;
     P.small0 = C.small0.as<int32_t>();
     P.small1 = C.small1.as<int32_t>();
     P.items = C.items.as<int32_t>();
@@ -604,9 +606,12 @@ static int run(Context &C, const Problem &pb, int mode, uint64_t seed, const gc_
     const int bps_opt = opt ? opt->blocks_per_sm : 0;
     const bool wide = bps_opt == 3 || (bps_opt == 0 && 2 * static_cast<int64_t>(n_chunks) * CH >= pb.nnz &&
                                        n_chunks > 0);
+    const RoundVariant variant = mode == GC_MODE_DETERMINISTIC && n_items == 0 ? kRoundSmall
+                                 : wide                                         ? kRoundWide
+                                                                                : kRoundNarrow;
     // persistent grid: every block resident; no more blocks than the first round can use
-    int &occ = C.occ[wide ? 1 : 0][mode][pb.batch ? 1 : 0][compact ? 1 : 0];
-    if (occ == 0) GC_CUDA(round_kernel_occupancy(mode, pb.batch, compact, block, &occ, wide));
+    int &occ = C.occ[variant][mode][pb.batch ? 1 : 0][compact ? 1 : 0];
+    if (occ == 0) GC_CUDA(round_kernel_occupancy(mode, pb.batch, compact, block, &occ, variant));
     int per_sm = occ;
     if (bps_opt > 0 && bps_opt < per_sm) per_sm = bps_opt;
     grid = static_cast<int64_t>(per_sm) * C.sms;
@@ -614,7 +619,7 @@ static int run(Context &C, const Problem &pb, int mode, uint64_t seed, const gc_
     if (want < grid) grid = want;
     if (grid < 1) grid = 1;
     GC_TRY(wait_colidx(pb, s));
-    GC_CUDA(launch_rounds(P, mode, pb.batch, compact, static_cast<int>(grid), block, s, wide));
+    GC_CUDA(launch_rounds(P, mode, pb.batch, compact, static_cast<int>(grid), block, s, variant));
     if (P.core_max > 0) GC_CUDA(launch_core(P, Q, pb.batch, s));
     }
     if (timing) GC_CUDA(cudaEventRecord(C.ev[2], s));

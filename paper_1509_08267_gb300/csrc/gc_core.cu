@@ -83,7 +83,7 @@ __device__ __forceinline__ bool core_fused(int R0) { return R0 <= 63; }
 struct HandOver {
     int R0;
     unsigned nsmall, nchunks;
-    const uint64_t *colc;   // state words round R0 reads
+    DetState st;            // state round R0 reads
     const int32_t *smallc;  // vertices of degree <= T1
     const DetItem *itc;     // work items of larger vertices
 };
@@ -95,7 +95,7 @@ __device__ __forceinline__ HandOver hand_over(const RoundParams &P) {
     h.nsmall = __ldcg(cc + kCntSmall);
     h.nchunks = __ldcg(cc + kCntChunks);
     const bool odd = (h.R0 & 1) != 0;
-    h.colc = odd ? P.col0 : P.col1;
+    h.st = det_state(P, h.R0);
     h.smallc = odd ? P.small0 : P.small1;
     h.itc = reinterpret_cast<const DetItem *>(odd ? P.chunk0 : P.chunk1);
     return h;
@@ -119,21 +119,15 @@ __device__ __forceinline__ unsigned long long core_reserve(const CoreParams &Q, 
 // its degree, the pool space `off` (len entries) for its row, its color in both buffers and the
 // window of final colors found so far (`fin_src`: the round kernel's slot, or none).
 __device__ void core_init_vertex(const RoundParams &P, const CoreParams &Q, int32_t local, int32_t V, int32_t g,
-                                 const int32_t *list, int32_t len, int32_t deg, const uint64_t *colc,
+                                 const int32_t *list, int32_t len, int32_t deg, const DetState &st,
                                  const unsigned *fin_src, unsigned long long off) {
     P.items[V] = local;  // local id of V (the set-up scratch is free once the rounds run)
     unsigned *rec = core_rec(Q, local);
-    const int32_t c = color_of(__ldcg(colc + V));
+    const int32_t c = det_color(st, V);
     Q.cex[local] = c;
     Q.cex[Q.max_v + local] = c;
     Q.c8[local] = static_cast<uint8_t>(sat8(c));
     Q.c8[Q.max_v + local] = static_cast<uint8_t>(sat8(c));
-    // hash key: the state word of round R0 carries the local id in place of the priority bits (the
-    // row build then gets a neighbour's finality, color and local id in one gather and recomputes
-    // the key from the id); nothing reads those bits of a worklist vertex again, and the write-back
-    // rewrites the whole word
-    if (P.priority == GC_PRIORITY_HASH)
-        const_cast<uint64_t *>(colc)[V] = pack_state(c, static_cast<uint32_t>(local), false);
     const uint4 z = make_uint4(0, 0, 0, 0);
 #pragma unroll
     for (int w = 0; w < 32; w += 4) stcg4(rec + w, z);
@@ -168,7 +162,7 @@ __global__ void core_index_kernel(RoundParams P, CoreParams Q) {
             deg = static_cast<int32_t>(r.e - r.b);
         }
         const unsigned long long off = core_reserve(Q, in, deg, lane);
-        if (in) core_init_vertex(P, Q, static_cast<int32_t>(i), V, r.g, P.colidx + r.b, deg, deg, h.colc, nullptr, off);
+        if (in) core_init_vertex(P, Q, static_cast<int32_t>(i), V, r.g, P.colidx + r.b, deg, deg, h.st, nullptr, off);
     }
     for (int64_t base = t0 & ~int64_t{31}; base < h.nchunks; base += stride) {
         const int64_t i = base + lane;
@@ -189,7 +183,7 @@ __global__ void core_index_kernel(RoundParams P, CoreParams Q) {
         if (!first) continue;
         const int32_t local = static_cast<int32_t>(h.nsmall + b + __popc(mk & lanemask_lt()));
         const int32_t g = BATCH ? __ldg(P.vg + d.V) : 0;
-        core_init_vertex(P, Q, local, d.V, g, d.list, len, d.deg, h.colc, a + kAccFin, off);
+        core_init_vertex(P, Q, local, d.V, g, d.list, len, d.deg, h.st, a + kAccFin, off);
     }
 }
 
@@ -236,7 +230,7 @@ __global__ void __launch_bounds__(kFillThreads) core_fill_kernel(RoundParams P, 
         const bool hash_key = P.priority == GC_PRIORITY_HASH;
         const uint64_t seed = hash_key ? seed_of(P, V) : 0ull;
         const uint64_t hv = hash_key ? vertex_hash(seed, static_cast<uint32_t>(r.lv)) : 0ull;
-        const uint32_t pv = hash_key ? 0u : prio_of(__ldcg(h.colc + V));
+        const uint32_t pv = hash_key ? 0u : __ldcg(P.prio + V);
         const uint64_t off = static_cast<uint64_t>(__ldcg(rec + kCoreOffLo)) |
                              (static_cast<uint64_t>(__ldcg(rec + kCoreOffHi)) << 32);
         int32_t *dst = Q.pool + off;
@@ -244,12 +238,13 @@ __global__ void __launch_bounds__(kFillThreads) core_fill_kernel(RoundParams P, 
         __syncwarp();
         uint64_t flo = 0;
         const bool fused = core_fused(h.R0);
-        const int32_t cv = fused ? color_of(__ldcg(h.colc + V)) : -1;  // C_R0 of the vertex
+        const int32_t cv = fused ? det_color(h.st, V) : -1;  // C_R0 of the vertex
         uint64_t rlo = 0;         // fused: colors of the core neighbours (all below 64)
         unsigned conflict = 0;    // fused: a smaller-key core neighbour has the vertex's color
         for (int64_t j0 = lb; j0 < le; j0 += 32 * kFillPer) {
             int32_t ul[kFillPer];
-            uint64_t st[kFillPer];
+            int32_t U[kFillPer];
+            unsigned st[kFillPer];
 #pragma unroll
             for (int q = 0; q < kFillPer; ++q) {
                 const int64_t j = j0 + lane + 32 * q;
@@ -258,52 +253,44 @@ __global__ void __launch_bounds__(kFillThreads) core_fill_kernel(RoundParams P, 
 #pragma unroll
             for (int q = 0; q < kFillPer; ++q) {
                 const int64_t j = j0 + lane + 32 * q;
-                st[q] = kNoNeighbour;  // no neighbour (past the end, or a malformed entry)
-                if (j < le) {
-                    const int32_t U = neighbour(P, r, ul[q], j);
-                    if (U >= 0) st[q] = __ldcg(h.colc + U);
-                }
+                U[q] = j < le ? neighbour(P, r, ul[q], j) : -1;  // -1: past the end, or a malformed entry
+                st[q] = U[q] >= 0 ? load_s16(h.st.s16 + U[q]) : 0u;
             }
             int32_t loc[kFillPer];
 #pragma unroll
-            for (int q = 0; q < kFillPer; ++q) {
-                loc[q] = -1;
-                if (st[q] != kNoNeighbour && !final_of(st[q]))
-                    loc[q] = hash_key ? static_cast<int32_t>(prio_of(st[q])) : __ldcg(P.items + r.vbase + ul[q]);
-            }
+            for (int q = 0; q < kFillPer; ++q)
+                loc[q] = U[q] >= 0 && !(st[q] & kFinal) ? __ldcg(P.items + U[q]) : -1;
             uint32_t ev[kFillPer];
             unsigned keepm = 0;
 #pragma unroll
             for (int q = 0; q < kFillPer; ++q) {
                 const int64_t j = j0 + lane + 32 * q;
                 ev[q] = 0;
-                if (st[q] != kNoNeighbour) {
-                    if (final_of(st[q])) {
-                        const int32_t c = color_of(st[q]);
-                        if (static_cast<unsigned>(c) < 64u)
-                            flo |= 1ull << c;
-                        else if (static_cast<unsigned>(c) < 32u * kAccWords)
-                            atomicOr(&wfin[c >> 5], 1u << (c & 31));
-                    } else if (static_cast<unsigned>(loc[q]) < m) {
-                        keepm |= 1u << q;
-                        bool smaller;
-                        if (hash_key) {
-                            const uint64_t hu = vertex_hash(seed, static_cast<uint32_t>(ul[q]));
-                            smaller = hu < hv || (hu == hv && ul[q] < r.lv);
-                        } else {
-                            smaller = key_less_in(prio_of(st[q]), pv, static_cast<uint32_t>(ul[q]),
-                                                  static_cast<uint32_t>(r.lv), P, V);
-                        }
-                        ev[q] = static_cast<uint32_t>(loc[q]) | (smaller ? kCoreSmaller : 0u);
-                        if (fused) {
-                            const int32_t c = color_of(st[q]);
-                            rlo |= 1ull << (c & 63);
-                            conflict |= static_cast<unsigned>(smaller && c == cv);
-                        }
+                if (U[q] < 0) continue;
+                const int32_t c = det_color(h.st, U[q], st[q]);
+                if (st[q] & kFinal) {
+                    if (static_cast<unsigned>(c) < 64u)
+                        flo |= 1ull << c;
+                    else if (static_cast<unsigned>(c) < 32u * kAccWords)
+                        atomicOr(&wfin[c >> 5], 1u << (c & 31));
+                } else if (static_cast<unsigned>(loc[q]) < m) {
+                    keepm |= 1u << q;
+                    bool smaller;
+                    if (hash_key) {
+                        const uint64_t hu = vertex_hash(seed, static_cast<uint32_t>(ul[q]));
+                        smaller = hu < hv || (hu == hv && ul[q] < r.lv);
                     } else {
-                        // every vertex that is not final is on the worklist; anything else is a bug
-                        set_error(P.err, GC_ERR_INVALID_GRAPH, V, j);
+                        smaller = key_less_in(__ldcg(P.prio + U[q]), pv, static_cast<uint32_t>(ul[q]),
+                                              static_cast<uint32_t>(r.lv), P, V);
                     }
+                    ev[q] = static_cast<uint32_t>(loc[q]) | (smaller ? kCoreSmaller : 0u);
+                    if (fused) {
+                        rlo |= 1ull << (c & 63);
+                        conflict |= static_cast<unsigned>(smaller && c == cv);
+                    }
+                } else {
+                    // every vertex that is not final is on the worklist; anything else is a bug
+                    set_error(P.err, GC_ERR_INVALID_GRAPH, V, j);
                 }
             }
             // one reservation per step for the entries kept
@@ -627,7 +614,7 @@ __device__ void core_first_round(const RoundParams &P, const CoreParams &Q, int3
 template <bool BATCH>
 __device__ void core_round_warp(const RoundParams &P, const CoreParams &Q, const Shared &S, const int32_t *cex_cur,
                                 const int32_t *list, unsigned nact, int32_t m, unsigned nv, int pass,
-                                const uint64_t *col_r0, unsigned *cn, unsigned *grab, unsigned gw, unsigned nw,
+                                const DetState &st_r0, unsigned *cn, unsigned *grab, unsigned gw, unsigned nw,
                                 int lane, unsigned *win, unsigned *wfin, unsigned &st_read, unsigned &st_deg,
                                 unsigned &st_cnt) {
     PieceCursor cur;
@@ -754,7 +741,7 @@ __device__ void core_round_warp(const RoundParams &P, const CoreParams &Q, const
                             const int l = __ffs(fm) - 1;
                             nc = 32 * l + __ffs(~__shfl_sync(kFull, tw, l)) - 1;
                         } else {
-                            nc = core_mex_from<BATCH>(P, col_r0, static_cast<int32_t>(__shfl_sync(kFull, rx, kCoreGid - 32)),
+                            nc = core_mex_from<BATCH>(P, st_r0, static_cast<int32_t>(__shfl_sync(kFull, rx, kCoreGid - 32)),
                                                       cex_cur, win, lane, 32 * kAccWords);
                         }
                     }
@@ -922,7 +909,7 @@ __global__ void __launch_bounds__(kCoreThreads, 1) core_round_kernel(RoundParams
             if (pass == R0 && core_fused(R0))
                 core_first_round<BATCH>(P, Q, m, pass, cn, lane, st_read, st_deg, st_cnt);
             else
-                core_round_warp<BATCH>(P, Q, S, cex_cur, list, nact, m, nv, pass, h.colc, cn,
+                core_round_warp<BATCH>(P, Q, S, cex_cur, list, nact, m, nv, pass, h.st, cn,
                                        Q.cnt + 4 * (pass % 3) + 3, gw, nw, lane, s_win[wib], s_fin[wib], st_read,
                                        st_deg, st_cnt);
 #ifdef GC_CORE_PROFILE
@@ -943,17 +930,14 @@ __global__ void __launch_bounds__(kCoreThreads, 1) core_round_kernel(RoundParams
 // Final colors of the core into both state buffers (FINAL set), where the color count reads them.
 __global__ void core_writeback_kernel(RoundParams P, CoreParams Q) {
     if (__ldcg(P.core_go) == 0) return;
-    // the round kernel rewrote passes[0]; it recorded m and the hand-over round here
-    const int64_t m = __ldcg(Q.m + 1);
-    // the priority bits from the buffer round R0 did not read (the other one may carry local ids)
-    const uint64_t *prio_src = (__ldcg(Q.m + 3) & 1u) ? P.col1 : P.col0;
+    const int64_t m = __ldcg(Q.m + 1);  // the round kernel rewrote passes[0]; the core recorded m here
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < m;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
         const int32_t V = static_cast<int32_t>(__ldcg(core_rec(Q, i) + kCoreGid));
         const int32_t c = __ldcg(Q.cex + i);
-        const uint64_t w = pack_state(c, prio_of(__ldcg(prio_src + V)), true);
-        P.col0[V] = w;
-        P.col1[V] = w;
+        const unsigned dig = digest16(load_s16(P.s16a + V));
+        det_store(DetState{P.s16a, P.cx0}, V, c, dig, true);
+        det_store(DetState{P.s16b, P.cx1}, V, c, dig, true);
     }
 }
 

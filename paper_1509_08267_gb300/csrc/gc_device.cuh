@@ -23,6 +23,9 @@ constexpr unsigned kMergeNowItems = GC_MERGE_NOW_ITEMS;
 // (80 registers; fewer spills in the warp work-item sweep, for graphs whose entries are mostly in
 // larger vertices).
 constexpr int kNarrowBlocks = 4, kWideBlocks = 3;
+// Without work items (no larger vertex) nothing spills at 4 blocks; 5 and 6 were 3% and 13% slower on
+// the 256^3 stencil.
+constexpr int kSmallBlocks = 4;
 
 // ------------------------------------------------------------------------------------------
 // priority key: key(v) = (h(v), v), h(v) = SplitMix64 output number v of the stream `seed`
@@ -179,6 +182,53 @@ __device__ __forceinline__ bool final_of(uint64_t w) { return (w & kFinalBit) !=
 // writes visible to these weak loads.
 __device__ __forceinline__ uint64_t load_state(const uint64_t *p) {
     return __ldca(reinterpret_cast<const unsigned long long *>(p));
+}
+
+// Deterministic mode's vertex state: 16 bits per vertex and buffer, the color saturated at kSat7,
+// the priority digest, and kFinal once the vertex left the worklist for good (then both buffers hold
+// its color).  Loaded through L1 like the state words.
+constexpr unsigned kSat7 = 127u, kFinal = 1u;
+constexpr uint16_t kNobody16 = 0xfffeu;  // entry n: color 127, digest 255
+__device__ __forceinline__ unsigned color16(unsigned w) { return w >> 9; }
+__device__ __forceinline__ unsigned digest16(unsigned w) { return w >> 1 & 255u; }
+
+__device__ __forceinline__ unsigned load_s16(const uint16_t *p) {
+    return __ldca(reinterpret_cast<const unsigned short *>(p));
+}
+
+// 8 bits of the 31 priority bits, in their order (a <= b implies digest(a) <= digest(b)).  Hash key:
+// the top bits.  The other keys hold kCap - value (20 bits) over hash bits, with most values far
+// below the cap: a logarithmic code of the value (3 bits below the leading one), larger values first.
+__device__ __forceinline__ unsigned prio_digest(const RoundParams &P, uint32_t p31) {
+    if (P.priority == GC_PRIORITY_HASH) return p31 >> 23;
+    const uint32_t v = ((1u << 20) - 1u) - (p31 >> 11);
+    if (v < 8u) return 255u - v;
+    const int lead = 31 - __clz(static_cast<int>(v));  // 3..19
+    return 255u - (8u * static_cast<unsigned>(lead - 2) + ((v >> (lead - 3)) & 7u));
+}
+
+// One parity's buffers: what a round reads, or what it writes.
+struct DetState {
+    uint16_t *s16;
+    int32_t *cx;
+};
+// The state round `pass` reads (C_pass) / the state it writes (C_{pass+1}).
+__device__ __forceinline__ DetState det_state(const RoundParams &P, int pass) {
+    return (pass & 1) ? DetState{P.s16a, P.cx0} : DetState{P.s16b, P.cx1};
+}
+
+// Exact color of vertex V from its word b.
+__device__ __forceinline__ int32_t det_color(const DetState &S, int64_t V, unsigned b) {
+    const unsigned c = color16(b);
+    return c == kSat7 ? __ldcg(S.cx + V) : static_cast<int32_t>(c);
+}
+__device__ __forceinline__ int32_t det_color(const DetState &S, int64_t V) { return det_color(S, V, load_s16(S.s16 + V)); }
+
+// Color c of vertex V (priority digest `dig`) into one buffer.
+__device__ __forceinline__ void det_store(const DetState &S, int64_t V, int32_t c, unsigned dig, bool final_) {
+    const bool sat = c >= static_cast<int32_t>(kSat7);
+    if (sat) S.cx[V] = c;
+    S.s16[V] = static_cast<uint16_t>((sat ? kSat7 : static_cast<unsigned>(c)) << 9 | dig << 1 | (final_ ? kFinal : 0u));
 }
 
 // Adjacency entries are streamed without allocating in L1, leaving L1 to the state words.
@@ -428,10 +478,10 @@ __device__ __forceinline__ unsigned *core_rec(const CoreParams &Q, int64_t v) {
 }
 
 // Least color >= start absent from the neighbours of global vertex V in C_r (warp-cooperative, full
-// CSR row): a final neighbour's color from its state word, a core neighbour's from cex.  Used when
+// CSR row): a final neighbour's color from its state, a core neighbour's from cex.  Used when
 // the 512-color window of a vertex is full.
 template <bool BATCH>
-__device__ int32_t core_mex_from(const RoundParams &P, const uint64_t *col_r0, int32_t V, const int32_t *cex_cur,
+__device__ int32_t core_mex_from(const RoundParams &P, const DetState &st_r0, int32_t V, const int32_t *cex_cur,
                                  unsigned *win, int lane, int32_t start) {
     const Row r = load_row<BATCH>(P, V);
     for (int32_t base = start;; base += 32 * kAccWords) {
@@ -440,8 +490,9 @@ __device__ int32_t core_mex_from(const RoundParams &P, const uint64_t *col_r0, i
         for (int64_t j = r.b + lane; j < r.e; j += 32) {
             const int32_t ul = __ldg(P.colidx + j);
             if (static_cast<uint32_t>(ul) >= static_cast<uint32_t>(r.ng)) continue;
-            const uint64_t st = __ldcg(col_r0 + r.vbase + ul);
-            const int32_t c = (final_of(st) ? color_of(st) : __ldcg(cex_cur + __ldcg(P.items + r.vbase + ul))) - base;
+            const int64_t U = static_cast<int64_t>(r.vbase) + ul;
+            const unsigned b = load_s16(st_r0.s16 + U);
+            const int32_t c = ((b & kFinal) ? det_color(st_r0, U, b) : __ldcg(cex_cur + __ldcg(P.items + U))) - base;
             if (static_cast<unsigned>(c) < 32u * kAccWords) atomicOr(&win[c >> 5], 1u << (c & 31));
         }
         __syncwarp();

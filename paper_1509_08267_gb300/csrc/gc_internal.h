@@ -91,10 +91,22 @@ struct RoundParams {
     uint64_t seed;
     const uint64_t *g_seed;  // [G] per-graph priority seeds (the server); nullptr: `seed` for every graph
 
-    // Vertex state words: low 32 bits = color (int32, -1 = uncolored), high 32 bits = the high half
-    // of the vertex's priority hash, so one gather gives a neighbour's color and priority.
-    uint64_t *col0;  // deterministic: read in odd rounds, written in even ones; in-place: the live array
-    uint64_t *col1;  // deterministic: written in odd rounds
+    // In-place and ordered modes: vertex state words, low 32 bits = color (int32, -1 = uncolored), high
+    // 32 bits = FINAL and the vertex's priority bits, so one gather gives a neighbour's color and
+    // priority.  (Partition mode: colors now, and as the round began.)
+    uint64_t *col0;
+    uint64_t *col1;
+    // Deterministic mode (set_det_state): 16 bits per vertex and buffer -- color (saturated at 127) << 9
+    // | priority digest (8 bits, prio_digest) << 1 | FINAL -- which is all that nearly every adjacency
+    // entry needs of its neighbour, so the gathered array is a quarter of the state words' size, and
+    // one subtraction tells a neighbour of equal color and smaller digest.  Entry n stands for no
+    // neighbour (color 127, digest 255).  The exact color of a saturated one is in cx0 / cx1 (written
+    // only then); prio holds the 31 priority bits, read when colors and digests are equal.
+    uint16_t *s16a;  // read in odd rounds, written in even ones (like cx0)
+    uint16_t *s16b;  // written in odd rounds (like cx1)
+    int32_t *cx0, *cx1;
+    uint32_t *prio;
+    int64_t ci_len;  // entries of colidx that may be read (16-byte loads stay inside them)
     int32_t *small0, *small1;  // thread-per-vertex worklists (two parities)
     int4 *chunk0, *chunk1;     // warp work items, kItemBytes each (two parities)
     int32_t *mid0, *mid1;      // ordered mode: medium-degree ready vertices (two parities)
@@ -140,6 +152,17 @@ struct RoundParams {
     unsigned long long *ecnt;  // [3] entries in the lists of each counter set's worklist (core_max > 0)
     int32_t *core_go;          // set to 1 by the round kernel when it hands over
 };
+
+// Places the deterministic mode's vertex state in two buffers: the exact colors of both parities in
+// the first (8 n bytes), the priority bits and both 16-bit arrays in the second (8 n + kDetPad bytes).
+constexpr size_t kDetPad = 64;
+inline void set_det_state(RoundParams &P, void *buf0, void *buf1, size_t n) {
+    P.cx0 = static_cast<int32_t *>(buf0);
+    P.cx1 = P.cx0 + n;
+    P.prio = static_cast<uint32_t *>(buf1);
+    P.s16a = reinterpret_cast<uint16_t *>(P.prio + n);
+    P.s16b = P.s16a + n + 1;
+}
 
 // Core phase (gc_core.cu).  Once the worklist is small, its vertices get local ids 0..m-1 (the core)
 // and their rows are rebuilt as lists of the local ids of neighbours still on the worklist, the
@@ -220,15 +243,17 @@ cudaError_t launch_expand(const RoundParams &P, int mode, bool batch, bool compa
                           cudaStream_t s);
 // compact (deterministic mode only): larger vertices sweep packed lists of the neighbours that can
 // still change instead of their whole rows.
-// wide: the round-kernel variant compiled for 3 resident blocks per SM (80 registers a thread)
-// instead of 4 (64): for graphs whose adjacency entries are mostly in larger vertices.
+// Round-kernel variants: kRoundWide is compiled for 3 resident blocks per SM (80 registers a thread),
+// for graphs whose adjacency entries are mostly in larger vertices; kRoundNarrow for 4 (64); kRoundSmall
+// (deterministic mode, no larger vertex) has no work-item code.
+enum RoundVariant { kRoundNarrow = 0, kRoundWide = 1, kRoundSmall = 2 };
 cudaError_t launch_rounds(const RoundParams &P, int mode, bool batch, bool compact, int grid, int block,
-                          cudaStream_t s, bool wide = false);
+                          cudaStream_t s, RoundVariant v = kRoundNarrow);
 cudaError_t round_kernel_occupancy(int mode, bool batch, bool compact, int block, int *blocks_per_sm,
-                                   bool wide = false);
+                                   RoundVariant v = kRoundNarrow);
 // Distinct colors and largest color per graph over vertices [v_begin, v_end) (graphs g_begin..g_end-1).
-// `colors_sel` != NULL: read colors from col1 when *colors_sel is odd (the deterministic buffer
-// that the last round wrote), else from col0.  `out` != NULL receives the colors of
+// `colors_sel` != NULL: deterministic mode's state, the buffer that round *colors_sel wrote (s16b / cx1
+// when it is odd, else s16a / cx0); NULL: the state words col0.  `out` != NULL receives the colors of
 // [v_begin, v_end) (out[0] is vertex v_begin) unless err[0] != 0.
 cudaError_t launch_count_colors(const RoundParams &P, bool batch, const int32_t *colors_sel, int32_t v_begin,
                                 int32_t v_end, int32_t g_begin, int32_t g_end, unsigned *bitmap, int32_t *gmax,

@@ -151,23 +151,13 @@ __device__ __forceinline__ void load4(const int32_t *colidx, bool vec, int64_t j
     }
 }
 
-// The state word a neighbour (local id ul) has when round 1 of the deterministic mode reads it with
-// the hash priority: color 0 (C_1), not final (only isolated vertices are, and they are nobody's
-// neighbour) and the top 31 bits of its hash: recomputed from the id instead of gathered.
-__device__ __forceinline__ uint64_t round1_state(uint64_t seed, int32_t ul) {
-    return pack_state(0, static_cast<uint32_t>(vertex_hash(seed, static_cast<uint32_t>(ul)) >> 33), false);
-}
-
-// Per-thread sweep of a short row (degree <= T1 <= 127): window [0, 128) in two 64-bit masks (the
-// least free color is at most deg(v)) and conflict flag.  Four entries per step from the aligned
-// group of four that holds the row's first entry; the next step's entries are loaded before the
-// current step's gathers are consumed.  `need` (colors 0..r-1 of round r, or 0): the sweep stops
-// once the vertex loses and mask0 holds all of them (its next color is then r).  Returns the end of
-// the entries read.
+// Per-thread sweep of a short row (degree <= T1 <= 127; in-place mode): window [0, 128) in two
+// 64-bit masks (the least free color is at most deg(v)) and conflict flag.  Four entries per step from
+// the aligned group of four that holds the row's first entry; the next step's entries are loaded
+// before the current step's gathers are consumed.
 template <bool BATCH, bool WINDOW, bool CONFLICT>
-__device__ __forceinline__ int64_t sweep_small(const RoundParams &P, const Row &r, const uint64_t *colc, int32_t cv,
-                                               uint32_t pv, uint64_t &mask0, uint64_t &mask1, bool &lose,
-                                               bool r1 = false, uint64_t r1seed = 0, uint64_t need = 0) {
+__device__ __forceinline__ void sweep_small(const RoundParams &P, const Row &r, const uint64_t *colc, int32_t cv,
+                                            uint32_t pv, uint64_t &mask0, uint64_t &mask1, bool &lose) {
     constexpr int kT = 4;  // entries per step
     const bool vec = (reinterpret_cast<uintptr_t>(P.colidx) & 15u) == 0;
     int64_t j0 = vec ? (r.b & ~int64_t{3}) : r.b;
@@ -180,7 +170,7 @@ __device__ __forceinline__ int64_t sweep_small(const RoundParams &P, const Row &
             w[q] = kNoNeighbour;
             if (j0 + q >= r.b && j0 + q < r.e) {
                 const int32_t U = neighbour(P, r, ul[q], j0 + q);
-                if (U >= 0) w[q] = r1 ? round1_state(r1seed, ul[q]) : load_state(colc + U);
+                if (U >= 0) w[q] = load_state(colc + U);
             }
         }
         const bool more = j0 + kT < r.e;
@@ -199,13 +189,11 @@ __device__ __forceinline__ int64_t sweep_small(const RoundParams &P, const Row &
                                                          static_cast<uint32_t>(r.lv), P, r.vbase + r.lv);
             }
         }
-        if (need && lose && (mask0 & need) == need) return min(j0 + kT, r.e);
         if (more) {
 #pragma unroll
             for (int q = 0; q < kT; ++q) ul[q] = un[q];
         }
     }
-    return r.e;
 }
 
 // Least color absent from a two-mask window [0, 128) (never full for degree <= 127).
@@ -256,103 +244,335 @@ __device__ __forceinline__ bool merge_item(unsigned *a, int nch, int lane, unsig
 // deterministic mode
 
 // Writes a vertex's state for the next round.  A vertex that did not lose is final: its color will
-// not change again, so the FINAL bit goes into both buffers (the color and priority bits are the
-// ones already there, so a concurrent reader of the current buffer sees the same color either way).
-__device__ __forceinline__ void det_write(const uint64_t *colc, uint64_t *coln, int32_t V, bool lose, int32_t cv,
-                                          int32_t nc, uint32_t pv) {
-    if (lose) {
-        coln[V] = pack_state(nc, pv, false);
-    } else {
-        const uint64_t w = pack_state(cv, pv, true);
-        coln[V] = w;
-        const_cast<uint64_t *>(colc)[V] = w;
+// not change again, so it is marked FINAL in both buffers (the color is the one already there, so a
+// concurrent reader of the current buffer sees the same color either way).
+__device__ __forceinline__ void det_write(const DetState &cur, const DetState &next, int32_t V, bool lose, int32_t cv,
+                                          int32_t nc, unsigned dig) {
+    det_store(next, V, nc, dig, !lose);
+    if (!lose) det_store(cur, V, cv, dig, true);
+}
+
+// Least color >= start absent from the row's neighbours (warp-cooperative; mex <= deg(v) bounds it).
+template <bool BATCH>
+__device__ int32_t det_mex_from(const RoundParams &P, const DetState &S, const Row &r, unsigned *win, int lane,
+                                int32_t start) {
+    for (int32_t base = start;; base += 32 * kAccWords) {
+        if (lane < kAccWords) win[lane] = 0;
+        __syncwarp();
+        for (int64_t j = r.b + lane; j < r.e; j += 32) {
+            const int32_t ul = __ldg(P.colidx + j);
+            if (static_cast<uint32_t>(ul) >= static_cast<uint32_t>(r.ng)) continue;
+            const int32_t c = det_color(S, r.vbase + ul) - base;
+            if (static_cast<unsigned>(c) < 32u * kAccWords) atomicOr(&win[c >> 5], 1u << (c & 31));
+        }
+        __syncwarp();
+        int32_t res = -1;
+#pragma unroll 1
+        for (int w = 0; w < kAccWords; ++w) {
+            const unsigned x = win[w];
+            if (~x) {
+                res = base + 32 * w + __ffs(~x) - 1;
+                break;
+            }
+        }
+        __syncwarp();
+        if (res >= 0) return res;
     }
 }
 
-// One vertex of degree <= T1 (one thread): did it lose in this round; writes its next state.
+// Does a neighbour (local id ul, global id U) of equal color have the smaller key?  pv: the
+// vertex's priority bits, lv its local id, V its global id.
+__device__ __forceinline__ bool det_smaller(const RoundParams &P, int32_t U, int32_t ul, uint32_t pv, int32_t lv,
+                                            int32_t V) {
+    return key_less_in(__ldca(P.prio + U), pv, static_cast<uint32_t>(ul), static_cast<uint32_t>(lv), P, V);
+}
+
+// Eight entries from p (the row's aligned group; slots [lo, hi) of it belong to the row): one 32-byte
+// load when the array is 32-byte aligned (align 2), two 16-byte ones when it is 16-byte aligned (1),
+// if all eight lie inside the array (`inside`); else the row's own one by one.
+__device__ __forceinline__ void load_oct(const int32_t *p, int align, bool inside, int32_t lo, int32_t hi,
+                                         int32_t (&u)[8]) {
+    if (align != 0 && inside) {
+        if (align == 2) {
+            asm("ld.global.nc.L1::no_allocate.v8.s32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7])
+                : "l"(p));
+        } else {
+            const int4 x = load_entry4(p), y = load_entry4(p + 4);
+            u[0] = x.x;
+            u[1] = x.y;
+            u[2] = x.z;
+            u[3] = x.w;
+            u[4] = y.x;
+            u[5] = y.y;
+            u[6] = y.z;
+            u[7] = y.w;
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) u[q] = q >= lo && q < hi ? load_entry(p + q) : 0;
+    }
+}
+
+// 1 << c for c in 0..31, else 0 (PTX shifts clamp).
+__device__ __forceinline__ uint32_t bit_or_none(uint32_t c) {
+    uint32_t r;
+    asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(1u), "r"(c));
+    return r;
+}
+
+// Reports the malformed entries among the first `cnt` of a row.
+__device__ __noinline__ void det_small_check(const RoundParams &P, const Row &r, int32_t cnt) {
+    for (int64_t j = r.b; j < r.b + cnt; ++j) neighbour(P, r, load_entry(P.colidx + j), j);
+}
+
+// A neighbour of equal color has the vertex's digest (a vertex that is its own neighbour always gets
+// here before it can win), or the color is 127, which a saturated word may not be: whether vertex V
+// lost, by the exact colors and the full keys.  A warp per vertex (about one row in 200 of a mesh
+// needs it; resolved by its own thread, entry after entry, it held up the other 31 rows and the
+// round's barrier: 12.5 ms against 10.3 on the 256^3 stencil).
 template <bool BATCH>
-__device__ __forceinline__ bool det_small(const RoundParams &P, const uint64_t *colc, uint64_t *coln, int32_t V,
-                                          int32_t &deg, int32_t &nread, bool r1, uint64_t need) {
+__device__ __noinline__ bool det_small_exact(const RoundParams &P, const DetState &S, int32_t V, int lane) {
     const Row r = load_row<BATCH>(P, V);
-    deg = static_cast<int32_t>(r.e - r.b);
-    const uint64_t self = load_state(colc + V);
-    const int32_t cv = color_of(self);
-    const uint32_t pv = prio_of(self);
-    uint64_t mask0 = 0, mask1 = 0;
+    const int32_t cv = det_color(S, V);
+    const uint32_t pv = __ldg(P.prio + V);
     bool lose = false;
-    nread = static_cast<int32_t>(
-        sweep_small<BATCH, true, true>(P, r, colc, cv, pv, mask0, mask1, lose, r1, r1 ? seed_of(P, V) : 0, need) -
-        r.b);
-    det_write(colc, coln, V, lose, cv, lose ? first_free_128(mask0, mask1) : cv, pv);
+    for (int64_t j = r.b + lane; j < r.e; j += 32) {
+        const int32_t ul = load_entry(P.colidx + j);
+        const int32_t U = neighbour(P, r, ul, j);
+        if (U >= 0 && det_color(S, U) == cv) lose |= det_smaller(P, U, ul, pv, r.lv, V);
+    }
+    return __any_sync(kFull, lose);
+}
+
+// The row of a vertex of degree <= T1 <= 127, one thread: eight entries a step from the aligned
+// group of eight that holds the row's first entry (a whole 32-byte sector per load), the next step's
+// entries loaded before the current step's eight gathers are consumed.  W: words of the color window
+// m (every color of round `pass` is below `pass`: one word up to round 32, two up to 64, else four;
+// the least free color is at most the degree).  self: the vertex's own state word.  A neighbour's
+// word decides the conflict by its digest; equal digests are looked up.  Slots past the row's ends
+// and malformed entries read entry n of the state; their number tells that an entry was malformed.
+// need: as det_sweep_item.
+// Returns 1 if the vertex lost, 0 if not, 2 if its exact colors and keys have to tell; nread:
+// entries read.
+//
+// What bounds it: L1 wavefronts (65% busy on a 160^3 stencil; DRAM 38%): a warp's 32 rows lie in 32
+// places, so a row load costs 32 cache-line lookups whatever its width, and whole-sector loads make
+// the fewest of them.  A least-of-differences instead of a compare per entry and clamped shifts
+// instead of 64-bit windows keep the step at about nine instructions an entry.  256^3 stencil, whole
+// coloring: 8.5 ms, against 16.0 with 16-byte loads, 8-byte state gathers and a key test per entry of
+// equal color; 4,096 graphs of 100..4,000 vertices: 5.4 against 7.4.  (Groups of 4 or 8 lanes per
+// row, rows in shared memory: 19.4 ms, three times the instructions.)
+template <int W>
+__device__ __forceinline__ int det_small_row(const RoundParams &P, const DetState &S, const Row &r, unsigned self,
+                                              uint64_t need, uint32_t (&m)[W], int32_t &nread) {
+    const uintptr_t addr = reinterpret_cast<uintptr_t>(P.colidx);
+    const int align = (addr & 31u) == 0 ? 2 : (addr & 15u) == 0 ? 1 : 0;
+    const uint16_t *state = S.s16 + r.vbase;
+    const int32_t nobody = P.n - r.vbase;
+    const unsigned cv = color16(self), dig = digest16(self);
+#pragma unroll
+    for (int w = 0; w < W; ++w) m[w] = 0u;
+    // the least (neighbour's word - own color << 9): below 2 dig for a neighbour of equal color and
+    // smaller digest, and 2 dig or 2 dig + 1 if the digests tie
+    unsigned least = ~0u;
+    // slots of the groups from the one that holds the row's first entry: the row is [lo, hi)
+    const int32_t lo0 = static_cast<int32_t>(r.b & 7), deg = static_cast<int32_t>(r.e - r.b);
+    const int32_t *p = P.colidx + (r.b - lo0);
+    const int32_t room = static_cast<int32_t>(min(P.ci_len - (r.b - lo0), int64_t{1} << 20));
+    int32_t hi = lo0 + deg, j = 8;  // j: slots loaded
+    int none = -lo0;                // slots that named no neighbour, less those before the row
+    int32_t u[8];
+    load_oct(p, align, room >= 8, lo0, hi, u);
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+        if (q < lo0) u[q] = -1;
+    for (;;) {
+        if (hi < 8) {
+#pragma unroll
+            for (int q = 1; q < 8; ++q)
+                if (q >= hi) u[q] = -1;
+            none -= 8 - hi;
+        }
+        unsigned x[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const bool ok = static_cast<uint32_t>(u[q]) < static_cast<uint32_t>(r.ng);
+            if (!ok) ++none;
+            x[q] = load_s16(state + (ok ? u[q] : nobody));
+        }
+        const bool more = hi > 8;
+        if (more) load_oct(p + 8, align, room >= j + 8, 0, hi - 8, u);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            least = min(least, x[q] - (cv << 9));
+            const unsigned c = color16(x[q]);
+#pragma unroll
+            for (int w = 0; w < W; ++w) m[w] |= bit_or_none(c - 32u * w);
+        }
+        if (!more) break;
+        if (need && W <= 2 && least < 2u * dig) {
+            const uint64_t seen = W == 1 ? m[0] : static_cast<uint64_t>(m[W - 1]) << 32 | m[0];
+            if ((seen & need) == need) {
+                if (none != 0) det_small_check(P, r, j - lo0);
+                nread = j - lo0;
+                return 1;
+            }
+        }
+        p += 8;
+        j += 8;
+        hi -= 8;
+    }
+    nread = deg;
+    if (none != 0) det_small_check(P, r, deg);
+    if ((W == 4 && cv == kSat7) || least >> 1 == dig) return 2;
+    return least < 2u * dig ? 1 : 0;
+}
+
+// Least color absent from a window of W words; 32 W when all are there.
+template <int W>
+__device__ __forceinline__ int32_t first_free_words(const uint32_t (&m)[W]) {
+    int32_t c = 32 * W;
+#pragma unroll
+    for (int w = W - 1; w >= 0; --w)
+        if (~m[w]) c = 32 * w + __ffs(static_cast<int>(~m[w])) - 1;
+    return c;
+}
+
+// One vertex of degree <= T1 per lane (lanes with `in`): did it lose in this round; writes its next
+// state (warp-uniform call).
+template <bool BATCH>
+__device__ __forceinline__ bool det_small(const RoundParams &P, const DetState &cur, const DetState &next, bool in,
+                                          int32_t V, int pass, uint64_t need, int lane, int32_t &deg, int32_t &nread) {
+    int state = 0;
+    int32_t nc = 0;
+    unsigned self = 0;
+    if (in) {
+        const Row r = load_row<BATCH>(P, V);
+        deg = static_cast<int32_t>(r.e - r.b);
+        self = load_s16(cur.s16 + V);
+        if (pass <= 32) {
+            uint32_t m[1];
+            state = det_small_row<1>(P, cur, r, self, need, m, nread);
+            nc = first_free_words<1>(m);
+        } else if (pass <= 64) {
+            uint32_t m[2];
+            state = det_small_row<2>(P, cur, r, self, need, m, nread);
+            nc = first_free_words<2>(m);
+        } else {
+            uint32_t m[4];
+            state = det_small_row<4>(P, cur, r, self, 0, m, nread);
+            // at most the degree (color 127 is in the window also for the slots past the row's ends)
+            nc = min(first_free_words<4>(m), deg);
+        }
+    }
+    for (unsigned open = __ballot_sync(kFull, state == 2); open; open &= open - 1u) {
+        const int l = __ffs(static_cast<int>(open)) - 1;
+        const bool lost = det_small_exact<BATCH>(P, cur, __shfl_sync(kFull, V, l), lane);
+        if (lane == l) state = lost ? 1 : 0;
+    }
+    const bool lose = state == 1;
+    if (in) {
+        const int32_t cv = static_cast<int32_t>(color16(self));  // exact: a color is at most the degree
+        det_write(cur, next, V, lose, cv, lose ? nc : cv, digest16(self));
+    }
     return lose;
 }
 
-
-// Sweep of entries [lb, le) of a larger vertex's list with one warp, kStep entries per step (the
-// first step's entries are already in ul; the next step's are loaded before the current step's
-// gathers are consumed).  WINDOW: every neighbour's color goes to the round window (lo: colors
-// 0..63 per lane, win: 64..511 shared by the warp).  CONFLICT: a neighbour with the same color and
-// a smaller key sets `lose`.  DROP: a neighbour found final is also recorded in the window of final
-// neighbours (flo / wfin) and dropped; the entries still active are counted (survivors, lane 0) and, when
-// `dst` is set, copied to dst at positions from *newlen (atomically when `shared_len`, else lane 0's
-// running count `written`).  `need` (colors 0..r-1 of round r, or 0; never with dst): the sweep
-// stops once some lane has the conflict and the warp's window with `fin64` (final colors 0..63
-// known before) holds all of them -- the vertex's next color is then r; the entries not read count
-// as survivors.  Returns the end of the entries read.
-template <bool DROP, bool WINDOW = true, bool CONFLICT = true>
-__device__ __forceinline__ int64_t sweep_item(const RoundParams &P, const Row &r, const uint64_t *colc,
-                                              const int32_t *list, int64_t lb, int64_t le, int32_t (&ul)[kPer],
-                                              int32_t *dst, unsigned *newlen, bool shared_len, int lane, int32_t cv,
-                                              uint32_t pv, uint64_t &lo, unsigned *win, uint64_t &flo, unsigned *wfin,
-                                              bool &lose, unsigned &survivors, unsigned &written, bool r1 = false,
-                                              uint64_t r1seed = 0, uint64_t need = 0, uint64_t fin64 = 0) {
-    int32_t un[kPer];
-    uint64_t w[kPer];
-    for (int64_t j0 = lb; j0 < le; j0 += kStep) {
-        unsigned keepm = 0;  // DROP: bit q, entry q of this lane stays on the list
+// Sweep of entries [lb, le) of a larger vertex's list with one warp, four entries per lane and step
+// (kStep entries; 16-byte loads from the aligned group that holds the first entry; the next step's
+// entries are loaded before the current step's gathers are consumed).  Every neighbour's color goes
+// to the round window (lo0, lo1: colors 0..63 per lane, win: 64..511 shared by the warp); a neighbour
+// with the same color and a smaller key sets `lose` (their digests decide, or the full keys when those tie).  DROP: a
+// neighbour found final is also recorded in the window of final neighbours (f0, f1 / wfin) and dropped;
+// the entries still active are counted (survivors, lane 0) and, when `dst` is set, copied to dst at
+// positions from *newlen (atomically when `shared_len`, else lane 0's running count `written`).
+// `need` (colors 0..r-1 of round r, or 0; never with dst): the sweep stops once the vertex lost and
+// the warp's window with `fin64` (final colors 0..63 known before) holds all of them -- the vertex's
+// next color is then r; the entries not read count as survivors.
+// Returns the end of the entries read; `lose` is the same in every lane.
+__device__ __forceinline__ void item_quad(const int32_t *list, int32_t j, int32_t lb, int32_t le, int32_t (&u)[4],
+                                          unsigned &valid) {
+    valid = 0;
+    if (j >= lb && j + 4 <= le) {
+        const int4 v = __ldcg(reinterpret_cast<const int4 *>(list + j));
+        u[0] = v.x;
+        u[1] = v.y;
+        u[2] = v.z;
+        u[3] = v.w;
+        valid = 15u;
+    } else {
 #pragma unroll
-        for (int q = 0; q < kPer; ++q) {
-            const int64_t j = j0 + lane + 32 * q;
-            w[q] = kNoNeighbour;
-            if (j < le) {
-                const int32_t U = neighbour(P, r, ul[q], j);
-                if (U >= 0) w[q] = r1 ? round1_state(r1seed, ul[q]) : load_state(colc + U);
+        for (int q = 0; q < 4; ++q) {
+            u[q] = 0;
+            if (j + q >= lb && j + q < le) {
+                u[q] = __ldcg(list + j + q);
+                valid |= 1u << q;
+            }
+        }
+    }
+}
+
+template <bool DROP>
+__device__ __forceinline__ int32_t det_sweep_item(const RoundParams &P, const DetState &S, int32_t V, int32_t vbase,
+                                                  int32_t ng, const int32_t *list, int32_t j0, int32_t lb, int32_t le,
+                                                  int32_t (&u)[4], unsigned valid, int32_t *dst, unsigned *newlen,
+                                                  bool shared_len, int lane, int32_t cv, unsigned dig, unsigned &lo0,
+                                                  unsigned &lo1, unsigned *win, unsigned &f0, unsigned &f1,
+                                                  unsigned *wfin, bool &lose, unsigned &survivors, unsigned &written,
+                                                  uint64_t need, uint64_t fin64) {
+    const int32_t lv = V - vbase;
+    for (;; j0 += kStep) {
+        int32_t un[4];
+        unsigned vn = 0;
+        unsigned b[4];
+        // this step's gathers: `valid` keeps the entries that name a neighbour
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            b[q] = 0u;
+            if ((valid >> q) & 1u) {
+                if (static_cast<uint32_t>(u[q]) < static_cast<uint32_t>(ng) && u[q] != lv) {
+                    b[q] = load_s16(S.s16 + vbase + u[q]);
+                } else {
+                    set_error(P.err, GC_ERR_INVALID_GRAPH, V, j0 + 4 * lane + q);
+                    valid &= ~(1u << q);
+                }
             }
         }
         const bool more = j0 + kStep < le;
-        if (more) {
+        if (more) item_quad(list, j0 + kStep + 4 * lane, lb, le, un, vn);
+        unsigned keepm = valid, tie = 0;
+        bool mine = lose;
 #pragma unroll
-            for (int q = 0; q < kPer; ++q) {
-                const int64_t j = j0 + kStep + lane + 32 * q;
-                un[q] = j < le ? __ldcg(list + j) : 0;
+        for (int q = 0; q < 4; ++q) {
+            if (!((valid >> q) & 1u)) continue;
+            const bool fin = DROP && (b[q] & kFinal);
+            int32_t c = static_cast<int32_t>(color16(b[q]));
+            if (c == static_cast<int32_t>(kSat7)) c = __ldcg(S.cx + vbase + u[q]);
+            if (c < 32) {
+                lo0 |= 1u << c;
+                if (fin) f0 |= 1u << c;
+            } else if (c < 64) {
+                lo1 |= 1u << (c - 32);
+                if (fin) f1 |= 1u << (c - 32);
+            } else if (c < 32 * kAccWords) {
+                atomicOr(&win[c >> 5], 1u << (c & 31));
+                if (fin) atomicOr(&wfin[c >> 5], 1u << (c & 31));
             }
+            // the smaller digest is the smaller key; equal digests are looked up
+            if (c == cv) {
+                mine |= digest16(b[q]) < dig;
+                tie |= static_cast<unsigned>(digest16(b[q]) == dig) << q;
+            }
+            if (fin) keepm &= ~(1u << q);
         }
-#pragma unroll
-        for (int q = 0; q < kPer; ++q) {
-            const int32_t c = color_of(w[q]);
-            const bool fin = DROP && j0 + lane + 32 * q < le && final_of(w[q]);
-            if constexpr (WINDOW) {
-                if (static_cast<unsigned>(c) < 64u) {
-                    lo |= 1ull << c;
-                    if (fin) flo |= 1ull << c;
-                } else if (static_cast<unsigned>(c) < 32u * kAccWords) {
-                    atomicOr(&win[c >> 5], 1u << (c & 31));
-                    if (fin) atomicOr(&wfin[c >> 5], 1u << (c & 31));
-                }
-            } else if (fin) {
-                if (static_cast<unsigned>(c) < 64u)
-                    flo |= 1ull << c;
-                else if (static_cast<unsigned>(c) < 32u * kAccWords)
-                    atomicOr(&wfin[c >> 5], 1u << (c & 31));
-            }
-            if constexpr (CONFLICT) {
-                if (c == cv && !lose) lose = key_less_in(prio_of(w[q]), pv, static_cast<uint32_t>(ul[q]),
-                                                         static_cast<uint32_t>(r.lv), P, r.vbase + r.lv);
-            }
-            if constexpr (DROP) {
-                if (j0 + lane + 32 * q < le && !fin) keepm |= 1u << q;
-            }
+        while (tie != 0u && !mine) {
+            const int q = __ffs(static_cast<int>(tie)) - 1;
+            tie &= tie - 1u;
+            const int32_t ul = q == 0 ? u[0] : q == 1 ? u[1] : q == 2 ? u[2] : u[3];
+            mine = det_smaller(P, vbase + ul, ul, __ldg(P.prio + V), lv, V);
         }
+        lose = __any_sync(kFull, mine);
         if constexpr (DROP) {
             // entries still active: counted, and in a rewrite round copied with one reservation per step
             const unsigned kept = __reduce_add_sync(kFull, static_cast<unsigned>(__popc(keepm)));
@@ -369,30 +589,29 @@ __device__ __forceinline__ int64_t sweep_item(const RoundParams &P, const Row &r
                 }
                 pos = __shfl_sync(kFull, pos, 0);
 #pragma unroll
-                for (int q = 0; q < kPer; ++q) {
+                for (int q = 0; q < 4; ++q) {
                     const bool keep = (keepm >> q) & 1u;
                     const unsigned km = __ballot_sync(kFull, keep);
-                    if (keep) dst[pos + __popc(km & lanemask_lt())] = ul[q];
+                    if (keep) dst[pos + __popc(km & lanemask_lt())] = u[q];
                     pos += __popc(km);
                 }
             }
         }
-        if (need && __any_sync(kFull, lose)) {
-            const uint64_t wl = (static_cast<uint64_t>(__reduce_or_sync(kFull, static_cast<unsigned>(lo >> 32))) << 32 |
-                                 __reduce_or_sync(kFull, static_cast<unsigned>(lo))) |
+        if (need && lose) {
+            const uint64_t wl = (static_cast<uint64_t>(__reduce_or_sync(kFull, lo1)) << 32 |
+                                 __reduce_or_sync(kFull, lo0)) |
                                 fin64;
             if ((wl & need) == need) {
-                const int64_t jend = min(le, j0 + kStep);
+                const int32_t jend = min(le, j0 + kStep);
                 if (DROP && lane == 0) survivors += static_cast<unsigned>(le - jend);
                 return jend;
             }
         }
-        if (more) {
+        if (!more) return le;
+        valid = vn;
 #pragma unroll
-            for (int q = 0; q < kPer; ++q) ul[q] = un[q];
-        }
+        for (int q = 0; q < 4; ++q) u[q] = un[q];
     }
-    return le;
 }
 
 // Appends the next round's items of the vertices that lost in lanes with items_l > 0 (one
@@ -440,7 +659,7 @@ __device__ __forceinline__ void append_items(DetItem *next, unsigned *cnt_next, 
 // `fin`; d = any item of the vertex): reads the merged slot, takes the least free color if the
 // vertex lost, writes its state, clears the slot's round part and appends its next items.
 template <bool BATCH, bool COMPACT>
-__device__ __forceinline__ void det_finish(const RoundParams &P, const uint64_t *colc, uint64_t *coln, bool fin,
+__device__ __forceinline__ void det_finish(const RoundParams &P, const DetState &S, const DetState &N, bool fin,
                                            const DetItem &d, unsigned *win, DetItem *next, unsigned *cnt_next,
                                            int pass, int lane, unsigned items_now, unsigned warps,
                                            unsigned &st_deg, unsigned &st_cnt, unsigned long long &st_ent) {
@@ -450,9 +669,12 @@ __device__ __forceinline__ void det_finish(const RoundParams &P, const uint64_t 
     unsigned *a = P.acc + static_cast<size_t>(slot) * kAccStride;
     uint4 st = make_uint4(0, 0, 0, 0), m0 = st, m1 = st;
     uint4 w[kAccWords / 4];
-    uint64_t self = 0;
+    int32_t cv = 0;
+    unsigned dig = 0;
     if (fin) {
-        self = load_state(colc + V);
+        const unsigned self = load_s16(S.s16 + V);
+        cv = det_color(S, V, self);
+        dig = digest16(self);
         st = ldcg4(a + kAccFlag);  // flag, item count, survivors, new length
         if (COMPACT) {
             m0 = ldcg4(a + kAccSrc);    // src, len, (unused), offset lo
@@ -472,8 +694,6 @@ __device__ __forceinline__ void det_finish(const RoundParams &P, const uint64_t 
     }
     const bool lose = fin && st.x != 0u;
     const bool pick = lose;
-    const int32_t cv = color_of(self);
-    const uint32_t pv = prio_of(self);
     int32_t nc = cv;
     if (pick) {
         nc = -1;
@@ -487,11 +707,11 @@ __device__ __forceinline__ void det_finish(const RoundParams &P, const uint64_t 
         const int l = __ffs(need) - 1;
         need &= need - 1;
         Row rl = load_row<BATCH>(P, __shfl_sync(kFull, V, l));
-        const int32_t x = mex_from<BATCH>(P, colc, rl, win, lane, 32 * kAccWords);
+        const int32_t x = det_mex_from<BATCH>(P, S, rl, win, lane, 32 * kAccWords);
         if (lane == l) nc = x;
     }
     if (fin) {
-        det_write(colc, coln, V, lose, cv, nc, pv);
+        det_write(S, N, V, lose, cv, nc, dig);
         st_deg += static_cast<unsigned>(deg);
         st_cnt += 1;
         const uint4 z = make_uint4(0, 0, 0, 0);
@@ -535,29 +755,22 @@ __device__ __forceinline__ void det_finish(const RoundParams &P, const uint64_t 
 // another), or the item that completes the slot's count finishes it at once (`merge_now`: sparse
 // rounds, where the extra barrier would cost more than the wait).
 template <bool BATCH, bool COMPACT>
-__device__ void det_item(const RoundParams &P, const uint64_t *colc, uint64_t *coln, const DetItem &d,
+__device__ void det_item(const RoundParams &P, const DetState &S, const DetState &N, const DetItem &d,
                          unsigned *win, unsigned *wfin, unsigned *snap, DetItem *next, unsigned *cnt_next, int pass,
                          int lane, unsigned items_now, unsigned warps, bool merge_now, unsigned &st_deg,
-                         unsigned &st_cnt, unsigned &st_read, bool r1, unsigned long long &st_ent, uint64_t need) {
+                         unsigned &st_cnt, unsigned &st_read, unsigned long long &st_ent, uint64_t need) {
     const int32_t V = d.V;
     const uint32_t slot = d.slotf & kItemSlot;
     const bool multi = (d.slotf & kItemMulti) != 0;
     unsigned *a = P.acc + static_cast<size_t>(slot) * kAccStride;
-    Row r;
-    r.b = 0;
-    r.e = 0;
-    r.vbase = d.vbase;
-    r.ng = d.ng;
-    r.lv = V - d.vbase;
-    r.g = 0;
-    // the first step's entries, the vertex's state and its slot: one round trip
-    int32_t ul[kPer];
-#pragma unroll
-    for (int q = 0; q < kPer; ++q) {
-        const int64_t j = static_cast<int64_t>(d.lb) + lane + 32 * q;
-        ul[q] = j < d.le ? __ldcg(d.list + j) : 0;
-    }
-    const uint64_t self = load_state(colc + V);
+    // the first step's entries (from the aligned group of four that holds the first), the vertex's
+    // state and its slot: one round trip
+    const int32_t j0 = d.lb - static_cast<int32_t>(reinterpret_cast<uintptr_t>(d.list + d.lb) >> 2 & 3u);
+    int32_t u[4];
+    unsigned valid;
+    item_quad(d.list, j0 + 4 * lane, d.lb, d.le, u, valid);
+    const unsigned self = load_s16(S.s16 + V);
+    const unsigned dig = digest16(self);
     const unsigned x = multi ? __ldcg(a + lane) : 0u;
     const unsigned sm = COMPACT ? __ldcg(a + 32 + lane) : 0u;
     if (lane < kAccWords) {
@@ -568,8 +781,7 @@ __device__ void det_item(const RoundParams &P, const uint64_t *colc, uint64_t *c
             snap[kAccWords + lane] = sm;
         }
     }
-    const int32_t cv = color_of(self);
-    const uint32_t pv = prio_of(self);
+    const int32_t cv = det_color(S, V, self);
     const int64_t deg = d.deg;
     int32_t *dst = nullptr;
     unsigned src = 0, len = 0;
@@ -582,23 +794,21 @@ __device__ void det_item(const RoundParams &P, const uint64_t *colc, uint64_t *c
         if (d.slotf & kItemRewrite) dst = P.lists + off + (src == 1 ? deg : 0);
     }
     __syncwarp();
-    uint64_t lo = 0, flo = 0;
+    unsigned lo0 = 0, lo1 = 0, f0 = 0, f1 = 0;
     bool lose = false;
     unsigned survivors = 0, written = 0;
     // final colors 0..63 already in the slot (lanes 0 and 1 hold them)
     const uint64_t fin64 = COMPACT ? (static_cast<uint64_t>(__shfl_sync(kFull, sm, 1)) << 32 | __shfl_sync(kFull, sm, 0))
                                    : 0ull;
-    const int64_t jend = sweep_item<COMPACT, true, true>(P, r, colc, d.list, d.lb, d.le, ul, dst, a + kAccNewLen, multi,
-                                                         lane, cv, pv, lo, win, flo, wfin, lose, survivors, written,
-                                                         r1, r1 ? seed_of(P, V) : 0, dst ? 0ull : need, fin64);
+    const int32_t jend = det_sweep_item<COMPACT>(P, S, V, d.vbase, d.ng, d.list, j0, d.lb, d.le, u, valid, dst,
+                                                 a + kAccNewLen, multi, lane, cv, dig, lo0, lo1, win, f0, f1, wfin,
+                                                 lose, survivors, written, dst ? 0ull : need, fin64);
     if (lane == 0) st_read += static_cast<unsigned>(jend - d.lb);
-    lose = __any_sync(kFull, lose);
-    unsigned lo0 = __reduce_or_sync(kFull, static_cast<unsigned>(lo));
-    unsigned lo1 = __reduce_or_sync(kFull, static_cast<unsigned>(lo >> 32));
-    unsigned f0 = 0, f1 = 0;
+    lo0 = __reduce_or_sync(kFull, lo0);
+    lo1 = __reduce_or_sync(kFull, lo1);
     if constexpr (COMPACT) {
-        f0 = __reduce_or_sync(kFull, static_cast<unsigned>(flo));
-        f1 = __reduce_or_sync(kFull, static_cast<unsigned>(flo >> 32));
+        f0 = __reduce_or_sync(kFull, f0);
+        f1 = __reduce_or_sync(kFull, f1);
     }
     __syncwarp();
     if (multi) {
@@ -618,7 +828,7 @@ __device__ void det_item(const RoundParams &P, const uint64_t *colc, uint64_t *c
         if (lane == 0) done = atom_add_acq_rel(a + kAccDone, 1u);
         done = __shfl_sync(kFull, done, 0);
         if (done != static_cast<unsigned>(d.nitems - 1)) return;
-        det_finish<BATCH, COMPACT>(P, colc, coln, lane == 0, d, win, next, cnt_next, pass, lane, items_now, warps,
+        det_finish<BATCH, COMPACT>(P, S, N, lane == 0, d, win, next, cnt_next, pass, lane, items_now, warps,
                                    st_deg, st_cnt, st_ent);
         return;
     }
@@ -640,9 +850,9 @@ __device__ void det_item(const RoundParams &P, const uint64_t *colc, uint64_t *c
     int32_t nc = cv;
     if (lose) {
         nc = first_free(lo0, lo1, win);
-        if (nc < 0) nc = mex_from<BATCH>(P, colc, load_row<BATCH>(P, V), win, lane, 32 * kAccWords);
+        if (nc < 0) nc = det_mex_from<BATCH>(P, S, load_row<BATCH>(P, V), win, lane, 32 * kAccWords);
     }
-    if (lane == 0) det_write(colc, coln, V, lose, cv, nc, pv);
+    if (lane == 0) det_write(S, N, V, lose, cv, nc, dig);
     if (!lose) return;
     if constexpr (BATCH) {
         if (lane == 0) note_graph_round(P, __ldg(P.vg + V), pass + 1);
@@ -753,6 +963,98 @@ __device__ void ip_chunk_conflict(const RoundParams &P, const uint64_t *col, int
 // the round window.
 
 constexpr int kAccDone2 = 20;  // in-place compact: phase-2 work items finished
+
+// Sweep of entries [lb, le) of a larger vertex's list with one warp, kStep entries per step (the
+// first step's entries are already in ul; the next step's are loaded before the current step's
+// gathers are consumed).  WINDOW: every neighbour's color goes to the round window (lo: colors
+// 0..63 per lane, win: 64..511 shared by the warp).  CONFLICT: a neighbour with the same color and
+// a smaller key sets `lose`.  DROP: a neighbour found final is also recorded in the window of final
+// neighbours (flo / wfin) and dropped; the entries still active are counted (survivors, lane 0) and, when
+// `dst` is set, copied to dst at positions from *newlen (atomically when `shared_len`, else lane 0's
+// running count `written`).
+template <bool DROP, bool WINDOW, bool CONFLICT>
+__device__ __forceinline__ void sweep_item(const RoundParams &P, const Row &r, const uint64_t *colc,
+                                           const int32_t *list, int64_t lb, int64_t le, int32_t (&ul)[kPer],
+                                           int32_t *dst, unsigned *newlen, bool shared_len, int lane, int32_t cv,
+                                           uint32_t pv, uint64_t &lo, unsigned *win, uint64_t &flo, unsigned *wfin,
+                                           bool &lose, unsigned &survivors, unsigned &written) {
+    int32_t un[kPer];
+    uint64_t w[kPer];
+    for (int64_t j0 = lb; j0 < le; j0 += kStep) {
+        unsigned keepm = 0;  // DROP: bit q, entry q of this lane stays on the list
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) {
+            const int64_t j = j0 + lane + 32 * q;
+            w[q] = kNoNeighbour;
+            if (j < le) {
+                const int32_t U = neighbour(P, r, ul[q], j);
+                if (U >= 0) w[q] = load_state(colc + U);
+            }
+        }
+        const bool more = j0 + kStep < le;
+        if (more) {
+#pragma unroll
+            for (int q = 0; q < kPer; ++q) {
+                const int64_t j = j0 + kStep + lane + 32 * q;
+                un[q] = j < le ? __ldcg(list + j) : 0;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) {
+            const int32_t c = color_of(w[q]);
+            const bool fin = DROP && j0 + lane + 32 * q < le && final_of(w[q]);
+            if constexpr (WINDOW) {
+                if (static_cast<unsigned>(c) < 64u) {
+                    lo |= 1ull << c;
+                    if (fin) flo |= 1ull << c;
+                } else if (static_cast<unsigned>(c) < 32u * kAccWords) {
+                    atomicOr(&win[c >> 5], 1u << (c & 31));
+                    if (fin) atomicOr(&wfin[c >> 5], 1u << (c & 31));
+                }
+            } else if (fin) {
+                if (static_cast<unsigned>(c) < 64u)
+                    flo |= 1ull << c;
+                else if (static_cast<unsigned>(c) < 32u * kAccWords)
+                    atomicOr(&wfin[c >> 5], 1u << (c & 31));
+            }
+            if constexpr (CONFLICT) {
+                if (c == cv && !lose) lose = key_less_in(prio_of(w[q]), pv, static_cast<uint32_t>(ul[q]),
+                                                         static_cast<uint32_t>(r.lv), P, r.vbase + r.lv);
+            }
+            if constexpr (DROP) {
+                if (j0 + lane + 32 * q < le && !fin) keepm |= 1u << q;
+            }
+        }
+        if constexpr (DROP) {
+            // entries still active: counted, and in a rewrite round copied with one reservation per step
+            const unsigned kept = __reduce_add_sync(kFull, static_cast<unsigned>(__popc(keepm)));
+            if (lane == 0) survivors += kept;
+            if (dst && kept) {
+                unsigned pos = 0;
+                if (lane == 0) {
+                    if (shared_len) {
+                        pos = atomicAdd(newlen, kept);
+                    } else {
+                        pos = written;
+                        written += kept;
+                    }
+                }
+                pos = __shfl_sync(kFull, pos, 0);
+#pragma unroll
+                for (int q = 0; q < kPer; ++q) {
+                    const bool keep = (keepm >> q) & 1u;
+                    const unsigned km = __ballot_sync(kFull, keep);
+                    if (keep) dst[pos + __popc(km & lanemask_lt())] = ul[q];
+                    pos += __popc(km);
+                }
+            }
+        }
+        if (more) {
+#pragma unroll
+            for (int q = 0; q < kPer; ++q) ul[q] = un[q];
+        }
+    }
+}
 
 // Phase 1 work item: First Fit over the live colors of the list's neighbours and the window of
 // final neighbours.
@@ -926,15 +1228,40 @@ __device__ void ipc_item_conflict(const RoundParams &P, uint64_t *col, const Det
 // kernels
 
 
+// The losers of a warp's small rows wait in shared memory and are appended kPend - 32 or more at a
+// time: one reservation per 32-row chunk put 0.5M same-address atomics into a heavy round of 16M rows.
+constexpr unsigned kPend = 160;
+
+__device__ __forceinline__ void pend_flush(const int32_t *buf, unsigned &npend, int32_t *list, unsigned *counter,
+                                           int lane) {
+    if (npend == 0u) return;
+    unsigned base = 0;
+    if (lane == 0) base = atomicAdd(counter, npend);
+    base = __shfl_sync(kFull, base, 0);
+    __syncwarp();
+    for (unsigned i = lane; i < npend; i += 32u) list[base + i] = buf[i];
+    __syncwarp();
+    npend = 0;
+}
+
+__device__ __forceinline__ void pend_append(bool take, int32_t V, int32_t *buf, unsigned &npend, int32_t *list,
+                                            unsigned *counter, int lane) {
+    const unsigned m = __ballot_sync(kFull, take);
+    if (take) buf[npend + __popc(m & lanemask_lt())] = V;
+    npend += static_cast<unsigned>(__popc(m));
+    if (npend > kPend - 32u) pend_flush(buf, npend, list, counter, lane);
+}
+
 // Deterministic rounds.  Phase A: the work items of larger vertices, then one thread per vertex of
 // degree <= T1.  Phase B (only in rounds where some vertex has several items, after a grid barrier):
 // those vertices are finished from their merged slots, one lane each.
-template <bool BATCH, bool COMPACT, int MINB>
+template <bool BATCH, bool COMPACT, bool ITEMS, int MINB>
 __global__ void __launch_bounds__(kBlock, MINB) det_round_kernel(RoundParams P) {
     __shared__ unsigned s_win[kMaxWarps][kAccWords];
     // per warp: the window of final neighbours found by the current item, then the item's snapshots
     // of its slot's round window and final window
     __shared__ unsigned s_aux[kMaxWarps][3 * kAccWords];
+    __shared__ int32_t s_pend[kMaxWarps][kPend];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int nw = gridDim.x * (blockDim.x >> 5);
     const int gw = blockIdx.x * (blockDim.x >> 5) + wib;
@@ -966,13 +1293,10 @@ __global__ void __launch_bounds__(kBlock, MINB) det_round_kernel(RoundParams P) 
         if (blockIdx.x == 0 && threadIdx.x < kCnt) P.cnt[kCnt * ((pass + 2) % 3) + threadIdx.x] = 0u;
         if (P.ecnt && blockIdx.x == 0 && threadIdx.x == 0) P.ecnt[(pass + 2) % 3] = 0ull;
         const bool odd = (pass & 1) != 0;
-        const uint64_t *colc = odd ? P.col0 : P.col1;
-        uint64_t *coln = odd ? P.col1 : P.col0;
+        const DetState S = det_state(P, pass), N = det_state(P, pass + 1);
         const int32_t *smallc = odd ? P.small0 : P.small1;
         int32_t *smalln = odd ? P.small1 : P.small0;
         const DetItem *itc = reinterpret_cast<const DetItem *>(odd ? P.chunk0 : P.chunk1);
-        // round 1 with the hash key: every neighbour's state is known without reading it
-        const bool r1 = pass == 1 && P.priority == GC_PRIORITY_HASH;
         // the colors a neighbour can have in this round (0..pass-1), for the early stop of a sweep
         const uint64_t need = P.early_exit && pass <= 64 ? (~0ull >> (64 - pass)) : 0ull;
         DetItem *itn = reinterpret_cast<DetItem *>(odd ? P.chunk1 : P.chunk0);
@@ -982,23 +1306,22 @@ __global__ void __launch_bounds__(kBlock, MINB) det_round_kernel(RoundParams P) 
         // the current one runs), then one thread per small vertex
         // sparse rounds (at most kMergeNowItems items per warp) finish several-item vertices in phase A
         const bool merge_now = nchunks <= kMergeNowItems * static_cast<unsigned>(nw);
-        if (static_cast<unsigned>(gw) < nchunks) {
+        if (ITEMS && static_cast<unsigned>(gw) < nchunks) {
             uint32_t w = item_word(itc, gw, lane);
             for (unsigned i = gw; i < nchunks; i += nw) {
                 const DetItem d = item_of(w);
                 if (i + nw < nchunks) w = item_word(itc, i + nw, lane);
-                det_item<BATCH, COMPACT>(P, colc, coln, d, win, wfin, snap, itn, cn, pass, lane, nchunks,
-                                         static_cast<unsigned>(nw), merge_now, st_deg, st_cnt, st_read, r1, st_ent,
-                                         need);
+                det_item<BATCH, COMPACT>(P, S, N, d, win, wfin, snap, itn, cn, pass, lane, nchunks,
+                                         static_cast<unsigned>(nw), merge_now, st_deg, st_cnt, st_read, st_ent, need);
             }
         }
+        unsigned npend = 0;  // losers in the warp's buffer
         for (unsigned base = static_cast<unsigned>(gw) * 32u; base < nsmall; base += static_cast<unsigned>(nw) * 32u) {
             const unsigned i = base + lane;
-            bool lose = false;
-            int32_t V = 0, deg = 0, nread = 0;
+            const int32_t V = i < nsmall ? __ldcg(smallc + i) : 0;
+            int32_t deg = 0, nread = 0;
+            const bool lose = det_small<BATCH>(P, S, N, i < nsmall, V, pass, need, lane, deg, nread);
             if (i < nsmall) {
-                V = __ldcg(smallc + i);
-                lose = det_small<BATCH>(P, colc, coln, V, deg, nread, r1, need);
                 st_deg += static_cast<unsigned>(deg);
                 st_read += static_cast<unsigned>(nread);
                 st_cnt += 1;
@@ -1006,11 +1329,12 @@ __global__ void __launch_bounds__(kBlock, MINB) det_round_kernel(RoundParams P) 
                     if (lose) note_graph_round(P, __ldg(P.vg + V), pass + 1);
                 }
             }
-            warp_append(lose, V, smalln, cn + kCntSmall, lane);
+            pend_append(lose, V, s_pend[wib], npend, smalln, cn + kCntSmall, lane);
             if (lose) st_ent += static_cast<unsigned long long>(deg);
         }
+        pend_flush(s_pend[wib], npend, smalln, cn + kCntSmall, lane);
         // phase B
-        if (nmulti != 0u && !merge_now) {
+        if (ITEMS && nmulti != 0u && !merge_now) {
             if (!grid_sync(P.bar, bar_target, P.err, P.spin_ns)) break;
             for (unsigned base = static_cast<unsigned>(gw) * 32u; base < nchunks;
                  base += static_cast<unsigned>(nw) * 32u) {
@@ -1021,7 +1345,7 @@ __global__ void __launch_bounds__(kBlock, MINB) det_round_kernel(RoundParams P) 
                     d = item_lane(itc + i);
                     fin = (d.slotf & kItemMulti) != 0u && d.lb == 0;
                 }
-                det_finish<BATCH, COMPACT>(P, colc, coln, fin, d, win, itn, cn, pass, lane, nchunks,
+                det_finish<BATCH, COMPACT>(P, S, N, fin, d, win, itn, cn, pass, lane, nchunks,
                                            static_cast<unsigned>(nw), st_deg, st_cnt, st_ent);
             }
         }
@@ -1237,6 +1561,10 @@ __global__ void __launch_bounds__(256) setup_kernel(RoundParams P, int32_t v_beg
     }
     const int64_t count = static_cast<int64_t>(v_end) - v_begin;
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+    if (MODE == GC_MODE_DETERMINISTIC && blockIdx.x == 0 && threadIdx.x == 0) {
+        P.s16a[P.n] = kNobody16;
+        P.s16b[P.n] = kNobody16;
+    }
     unsigned long long st_ent = 0;  // list entries of the round's worklist (rows of its vertices)
     unsigned long long st_list = 0;  // compact mode: list-pool entries of the larger vertices
     unsigned st_chunks = 0;          // work items of the larger vertices
@@ -1267,8 +1595,10 @@ __global__ void __launch_bounds__(256) setup_kernel(RoundParams P, int32_t v_beg
             // an isolated vertex takes color 0 in round 1 and never changes: it is final from the start
             if (MODE == GC_MODE_DETERMINISTIC) {
                 // C_1 = 0 everywhere: round 1's First Fit sees no colored neighbour
-                P.col0[V] = pack_state(0, pv, d == 0);
-                P.col1[V] = pack_state(0, pv, d == 0);
+                const uint16_t w = static_cast<uint16_t>(prio_digest(P, pv) << 1 | (d == 0 ? kFinal : 0u));
+                P.s16a[V] = w;
+                P.s16b[V] = w;
+                P.prio[V] = pv;
             } else {
                 P.col0[V] = pack_state(d == 0 ? 0 : -1, pv, d == 0);
             }
@@ -2280,14 +2610,15 @@ __global__ void __launch_bounds__(256) count_mark_kernel(RoundParams P, const in
         if (threadIdx.x == 0) s_max = -1;
         __syncthreads();
     }
-    const uint64_t *state = (colors_sel && (*colors_sel & 1)) ? P.col1 : P.col0;
+    const bool det = colors_sel != nullptr;  // deterministic mode's byte state
+    const DetState S = det ? det_state(P, *colors_sel + 1) : DetState{nullptr, nullptr};
     const bool copy = out != nullptr && P.err[0] == 0;
     const int64_t count = static_cast<int64_t>(v_end) - v_begin;
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
     int32_t tmax = -1;
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < count; i += stride) {
         const int32_t V = static_cast<int32_t>(v_begin + i);
-        const int32_t c = color_of(__ldcg(state + V));
+        const int32_t c = det ? det_color(S, V) : color_of(__ldcg(P.col0 + V));
         if (copy) out[i] = c;
         if (c < 0) continue;
         if (!BATCH && c < 32 * kMarkWords) {
@@ -2550,10 +2881,10 @@ template <int MINB>
 static const void *round_kernel_variant(int mode, bool batch, bool compact) {
     if (mode == GC_MODE_DETERMINISTIC) {
         if (batch)
-            return compact ? reinterpret_cast<const void *>(&det_round_kernel<true, true, MINB>)
-                           : reinterpret_cast<const void *>(&det_round_kernel<true, false, MINB>);
-        return compact ? reinterpret_cast<const void *>(&det_round_kernel<false, true, MINB>)
-                       : reinterpret_cast<const void *>(&det_round_kernel<false, false, MINB>);
+            return compact ? reinterpret_cast<const void *>(&det_round_kernel<true, true, true, MINB>)
+                           : reinterpret_cast<const void *>(&det_round_kernel<true, false, true, MINB>);
+        return compact ? reinterpret_cast<const void *>(&det_round_kernel<false, true, true, MINB>)
+                       : reinterpret_cast<const void *>(&det_round_kernel<false, false, true, MINB>);
     }
     if (batch)
         return compact ? reinterpret_cast<const void *>(&ip_round_kernel<true, true, MINB>)
@@ -2562,26 +2893,33 @@ static const void *round_kernel_variant(int mode, bool batch, bool compact) {
                    : reinterpret_cast<const void *>(&ip_round_kernel<false, false, MINB>);
 }
 
-static const void *round_kernel_fn(int mode, bool batch, bool compact, bool wide) {
-    return wide ? round_kernel_variant<kWideBlocks>(mode, batch, compact)
-                : round_kernel_variant<kNarrowBlocks>(mode, batch, compact);
+static const void *round_kernel_fn(int mode, bool batch, bool compact, RoundVariant v) {
+    if (v == kRoundSmall && mode == GC_MODE_DETERMINISTIC) {
+        if (batch)
+            return compact ? reinterpret_cast<const void *>(&det_round_kernel<true, true, false, kSmallBlocks>)
+                           : reinterpret_cast<const void *>(&det_round_kernel<true, false, false, kSmallBlocks>);
+        return compact ? reinterpret_cast<const void *>(&det_round_kernel<false, true, false, kSmallBlocks>)
+                       : reinterpret_cast<const void *>(&det_round_kernel<false, false, false, kSmallBlocks>);
+    }
+    return v == kRoundWide ? round_kernel_variant<kWideBlocks>(mode, batch, compact)
+                           : round_kernel_variant<kNarrowBlocks>(mode, batch, compact);
 }
 
-cudaError_t round_kernel_occupancy(int mode, bool batch, bool compact, int block, int *blocks_per_sm, bool wide) {
+cudaError_t round_kernel_occupancy(int mode, bool batch, bool compact, int block, int *blocks_per_sm, RoundVariant v) {
     if (block != kBlock) return cudaErrorInvalidValue;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, round_kernel_fn(mode, batch, compact, wide),
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, round_kernel_fn(mode, batch, compact, v),
                                                          block, 0);
 }
 
 cudaError_t launch_rounds(const RoundParams &P, int mode, bool batch, bool compact, int grid, int block,
-                          cudaStream_t s, bool wide) {
+                          cudaStream_t s, RoundVariant v) {
     if (block != kBlock) return cudaErrorInvalidValue;
     // the grid barrier counts this launch's arrivals from zero
     cudaError_t e = cudaMemsetAsync(&P.bar->count, 0, sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
     RoundParams arg = P;
     void *args[] = {&arg};
-    return cudaLaunchCooperativeKernel(round_kernel_fn(mode, batch, compact, wide), dim3(grid), dim3(block), args, 0,
+    return cudaLaunchCooperativeKernel(round_kernel_fn(mode, batch, compact, v), dim3(grid), dim3(block), args, 0,
                                        s);
 }
 

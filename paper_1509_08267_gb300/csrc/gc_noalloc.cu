@@ -43,7 +43,7 @@ constexpr size_t align256(size_t x) { return (x + 255) & ~size_t{255}; }
 constexpr size_t kOffCtl = 0;
 constexpr size_t kOffCol0 = align256(kOffCtl + sizeof(NaCtl));
 constexpr size_t kOffCol1 = align256(kOffCol0 + 8 * size_t{kNaMaxVertices});
-constexpr size_t kOffSmall0 = align256(kOffCol1 + 8 * size_t{kNaMaxVertices});
+constexpr size_t kOffSmall0 = align256(kOffCol1 + 8 * size_t{kNaMaxVertices} + kDetPad);
 constexpr size_t kOffSmall1 = align256(kOffSmall0 + 4 * size_t{kNaMaxVertices});
 constexpr size_t kOffItems = align256(kOffSmall1 + 4 * size_t{kNaMaxVertices});
 constexpr size_t kOffChunk0 = align256(kOffItems + 4 * size_t{kNaMaxVertices});
@@ -151,8 +151,8 @@ extern "C" int gc_color_noalloc(int32_t n, const int32_t *rowptr, const int32_t 
     P.rowptr = rowptr;
     P.colidx = nnz > 0 ? colidx : rowptr;  // never dereferenced when there are no entries
     P.seed = seed;
-    P.col0 = reinterpret_cast<uint64_t *>(base + kOffCol0);
-    P.col1 = reinterpret_cast<uint64_t *>(base + kOffCol1);
+    set_det_state(P, base + kOffCol0, base + kOffCol1, static_cast<size_t>(n));
+    P.ci_len = nnz;
     P.small0 = reinterpret_cast<int32_t *>(base + kOffSmall0);
     P.small1 = reinterpret_cast<int32_t *>(base + kOffSmall1);
     P.items = reinterpret_cast<int32_t *>(base + kOffItems);

@@ -218,7 +218,7 @@ int engine_create(gc_server *s, Engine &E, int mode) {
         DevBuf *b;
         size_t bytes;
     } plan[] = {
-        {&E.rowptr, 4 * (V + Sz)}, {&E.colidx, 4 * static_cast<size_t>(E.PE)}, {&E.col0, 8 * V}, {&E.col1, 8 * V},
+        {&E.rowptr, 4 * (V + Sz)}, {&E.colidx, 4 * static_cast<size_t>(E.PE)}, {&E.col0, 8 * V}, {&E.col1, 8 * V + kDetPad},
         {&E.outbuf, 4 * V}, {&E.small0, 4 * V}, {&E.small1, 4 * V}, {&E.items, 4 * V}, {&E.vg, 4 * V},
         {&E.chunk0, kItemBytes * static_cast<size_t>(E.PC)}, {&E.chunk1, kItemBytes * static_cast<size_t>(E.PC)},
         {&E.acc, 4 * kAccStride * slots}, {&E.lists, E.compact ? 8 * static_cast<size_t>(E.PE) : 0},
@@ -278,6 +278,8 @@ RoundParams params(gc_server *s, Engine &E, int32_t rounds = kRoundsWhileQueued)
     P.g_seed = E.gseed.as<uint64_t>();  // every request has its own seed
     P.col0 = E.col0.as<uint64_t>();
     P.col1 = E.col1.as<uint64_t>();
+    set_det_state(P, E.col0.p, E.col1.p, static_cast<size_t>(E.PV));
+    P.ci_len = E.PE;
     P.small0 = E.small0.as<int32_t>();
     P.small1 = E.small1.as<int32_t>();
     P.chunk0 = E.chunk0.as<int4>();

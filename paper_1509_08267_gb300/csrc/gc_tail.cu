@@ -175,7 +175,6 @@ __global__ void __launch_bounds__(kTailThreads, 1) tail_kernel(RoundParams P, Co
 
     // keys (priority bits, hash, local id), sorted ascending: the tail ids
     const bool hash_key = P.priority == GC_PRIORITY_HASH;
-    const uint64_t *prio_src = (R0 & 1) ? P.col1 : P.col0;  // the state words round R0 did not read
     int32_t p2 = 1;
     while (p2 < k) p2 <<= 1;
     for (int32_t j = threadIdx.x; j < p2; j += kTailThreads) {
@@ -183,7 +182,7 @@ __global__ void __launch_bounds__(kTailThreads, 1) tail_kernel(RoundParams P, Co
             const int32_t V = static_cast<int32_t>(__ldcg(core_rec(Q, kid[j]) + kCoreGid));
             const Row r = load_row<BATCH>(P, V);
             const uint64_t h = vertex_hash(seed_of(P, V), static_cast<uint32_t>(r.lv));
-            const uint32_t p31 = hash_key ? static_cast<uint32_t>(h >> 33) : prio_of(__ldcg(prio_src + V));
+            const uint32_t p31 = hash_key ? static_cast<uint32_t>(h >> 33) : __ldcg(P.prio + V);
             key1[j] = static_cast<uint64_t>(p31) << 32 | (h >> 32);
             key2[j] = (h << 32) | static_cast<uint32_t>(r.lv);
         } else {
@@ -285,7 +284,7 @@ __global__ void __launch_bounds__(kTailThreads, 1) tail_kernel(RoundParams P, Co
     cluster_sync();  // every block built before any block writes into another's colors
     TAIL_BUILD(6);
 
-    const uint64_t *col_r0 = (R0 & 1) ? P.col0 : P.col1;  // the state words round R0 read
+    const DetState st_r0 = det_state(P, R0);  // the state round R0 read
     const int32_t wk = ((k + 1023) >> 10) << 5;  // the row words that can hold bits: a multiple of 32
     unsigned *win = s_win[wib];
     unsigned *pw = &s_pw[0][threadIdx.x];  // word w of this lane's window: pw[w * kTailThreads]
@@ -378,7 +377,7 @@ __global__ void __launch_bounds__(kTailThreads, 1) tail_kernel(RoundParams P, Co
                     const int l = __ffs(static_cast<int>(fm)) - 1;
                     nc = 32 * l + __ffs(static_cast<int>(~__shfl_sync(kFull, ww, l))) - 1;
                 } else {
-                    nc = core_mex_from<BATCH>(P, col_r0, s_gid[o], cex_cur, win, lane, 32 * kAccWords);
+                    nc = core_mex_from<BATCH>(P, st_r0, s_gid[o], cex_cur, win, lane, 32 * kAccWords);
                 }
             }
             TAIL_CLK(pc_merge);
