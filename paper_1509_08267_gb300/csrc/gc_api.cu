@@ -87,7 +87,7 @@ struct Ctl {
     unsigned long long ecnt[3];  // list entries of each counter set's worklist (core hand-over)
     unsigned long long core_bump;
     int32_t core_go, pad3;
-    alignas(16) unsigned core_cnt[12];  // three sets of four, each read with one 16-byte load
+    alignas(16) unsigned core_cnt[3 * kCoreCnt];  // each set's first four read with one 16-byte load
     unsigned core_m[4];
     unsigned tail_ctl[4];  // tail phase: handed over, first round
     GridBar bar;
@@ -560,9 +560,10 @@ static int run(Context &C, const Problem &pb, int mode, uint64_t seed, const gc_
             GC_TRY(ensure(C.core_c8, 2 * Mp, "core colors"));
             GC_TRY(ensure(C.core_fbits, 4 * (Mp / 32 + 1), "core final bits"));
             GC_TRY(ensure(C.core_items, 16 * static_cast<size_t>(Q.max_pieces), "core pieces"));
-            GC_TRY(ensure(C.core_active, 2 * 4 * static_cast<size_t>(Q.max_pieces), "core active pieces"));
+            GC_TRY(ensure(C.core_active, 6 * 4 * Mp, "core worklists"));
             GC_TRY(ensure(C.core_log, 2 * 8 * Mp, "core change log"));
-            GC_TRY(ensure(C.core_pool, 4 * static_cast<size_t>(E) + 16, "core rows"));  // + prefetch slack
+            // rows start at multiples of four entries; + prefetch slack
+            GC_TRY(ensure(C.core_pool, 4 * (static_cast<size_t>(E) + 4 * Mp) + 16, "core rows"));
             Q.rec = C.core_rec.as<unsigned>();
             Q.cex = C.core_cex.as<int32_t>();
             Q.c8 = C.core_c8.as<uint8_t>();

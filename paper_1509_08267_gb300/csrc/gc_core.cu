@@ -22,14 +22,13 @@
 //
 // Work decomposition.  Each row is cut once into pieces of at most kCorePiece entries (an empty row
 // into one empty piece); a piece compacts itself in place (it drops neighbours found final once the
-// worklist has lost half of its vertices since the piece last did).  Each round's list of
-// active pieces (the pieces of its worklist vertices) is dealt to the warps round-robin.  A round
-// is: refresh the shared colors of the vertices the previous round finished (its change log); every
-// warp sweeps its pieces (the next piece's first entries and record words are loaded while the
-// current one is consumed), and the warp that holds a vertex's last piece finishes the vertex (at
-// once when it has one piece; else after the pieces' windows and flags have met in the vertex's
-// record): least free color or FINAL, C_{r+1} written, the vertex batched per warp into the change
-// log and, if it lost, its pieces into the next round's list; one grid barrier.
+// worklist has lost half of its vertices since the piece last did).  A round: refresh the shared colors
+// of the vertices the previous round finished (its change log); the vertices of several pieces are dealt
+// to the blocks, whose warps take their pieces one after another from a queue in shared memory and
+// merge the windows there; the pieces of the others are dealt to the warps of the whole grid.  The
+// warp that holds a vertex's last piece finishes the vertex: least free color or FINAL, and the vertex
+// into a per-warp batch whose results (C_{r+1}, change log, the losers' lists) are written 32 at a time;
+// one grid barrier.
 //
 // Kernels: core_index_kernel (local ids, records, initial colors), core_fill_kernel (the rows),
 // core_round_kernel (one persistent cooperative launch with one block per SM running the rounds
@@ -50,7 +49,7 @@ namespace {
 constexpr int kCoreThreads = GC_CORE_THREADS;  // one block per SM: every block holds all m colors
 constexpr int kCoreWarps = kCoreThreads / 32;
 #ifndef GC_CORE_PER
-#define GC_CORE_PER 8
+#define GC_CORE_PER 4
 #endif
 constexpr int kCorePer = GC_CORE_PER;  // entries per lane per step of a piece
 constexpr int kCoreStep = 32 * kCorePer;
@@ -101,10 +100,11 @@ __device__ __forceinline__ HandOver hand_over(const RoundParams &P) {
     return h;
 }
 
-// Pool space for the rows of a warp's vertices (lanes with `take`, len entries each): one
-// reservation per warp (one counter shared by the whole grid: an atomic per vertex would queue).
+// Pool space for the rows of a warp's vertices (lanes with `take`, len entries each, rounded up to
+// a multiple of four: rows are read 16 bytes at a time): one reservation per warp (one counter shared
+// by the whole grid: an atomic per vertex would queue).
 __device__ __forceinline__ unsigned long long core_reserve(const CoreParams &Q, bool take, int32_t len, int lane) {
-    unsigned long long x = take ? static_cast<unsigned long long>(len) : 0ull, incl = x;
+    unsigned long long x = take ? static_cast<unsigned long long>((len + 3) & ~3) : 0ull, incl = x;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const unsigned long long y = __shfl_up_sync(kFull, incl, o);
@@ -378,13 +378,13 @@ __device__ __forceinline__ void prefetch_piece(const CoreParams &Q, int32_t off,
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"(bytes) : "memory");
 }
 
-// The round's active pieces a warp takes, in batches of up to 32 (one per lane).  In a round with
-// few pieces they are dealt statically: entries gw, gw + nw, gw + 2 nw, ... of the round's list of
-// pieces (the pieces of its worklist vertices; every piece in the first round).  In a round with many
-// (at least kGrabMin per warp) each batch is taken from the round's grab counter, in chunks that
-// shrink with what is left (guided self-scheduling: the pieces differ in size up to kCorePiece
-// entries, and a warp that drew large ones would otherwise hold the whole grid at the barrier).
-// Pieces without entries are taken too: they count towards their vertex's pieces done.
+// The one-piece vertices' pieces a warp takes, in batches of up to 32 (one per lane).  In a round with
+// few pieces they are dealt statically: entries gw, gw + nw, gw + 2 nw, ... of the round's list.  In a
+// round with many (at least kGrabMin per warp) each batch is taken from the round's grab counter, in
+// chunks of at most kGrabMost that shrink with what is left (guided self-scheduling: the pieces differ
+// in size, and a warp that drew large ones would otherwise hold the whole grid at the barrier).  Pieces
+// without entries are taken too: their vertex wins.
+constexpr unsigned kGrabMost = 8;
 constexpr unsigned kGrabMin = 4;
 struct PieceCursor {
     unsigned base;  // static: first list position of the current batch; dynamic: last grab's start
@@ -399,7 +399,7 @@ __device__ __forceinline__ void cursor_fill(PieceCursor &c, const CoreParams &Q,
     c.d = make_int4(0, 0, 0, 0);
     c.idx = 0;
     if (in) {
-        c.idx = list ? static_cast<unsigned>(__ldcg(list + i)) : i;
+        c.idx = static_cast<unsigned>(__ldcg(list + i));
         c.d = __ldcg(Q.pieces + c.idx);
     }
     c.act = __ballot_sync(kFull, in);
@@ -419,7 +419,7 @@ __device__ __forceinline__ bool cursor_load(PieceCursor &c, const CoreParams &Q,
     }
     const unsigned left = nact > c.base ? nact - c.base : 0u;
     unsigned chunk = left / (2u * nw);
-    chunk = chunk < 1u ? 1u : (chunk > 32u ? 32u : chunk);
+    chunk = chunk < 1u ? 1u : (chunk > kGrabMost ? kGrabMost : chunk);
     unsigned b = 0;
     if (lane == 0) b = atomicAdd(c.grab, chunk);
     b = __shfl_sync(kFull, b, 0);
@@ -447,112 +447,134 @@ __device__ __forceinline__ bool cursor_next(PieceCursor &c, const CoreParams &Q,
     return true;
 }
 
-// Entries j0 + lane + 32 q of a piece; slots past its end read the piece's own vertex (its color is
-// the vertex's own, which a loser's window holds already -- the neighbour it lost to has it -- and
-// which a winner never uses; without the key bit it is no conflict).
+// The colors around a piece's vertex, one byte per 8-bit color: a lane marks a neighbour's color with a
+// plain byte store (no atomic, no shift), whatever the other lanes store next to it.
+constexpr int kSeen = 256;
+
+// Entries j0 + 128 h + 4 lane + {0..3} of a piece (16-byte loads: pieces start at multiples of four).  Slots past its end hold entries it held once, or read the piece's own vertex:
+// a color around the vertex, or its own, which a loser's window holds already -- the neighbour it lost
+// to has it -- and which a winner never uses; neither is a conflict (a neighbour dropped as FINAL never
+// has the vertex's color, the vertex itself comes without the key bit).
 __device__ __forceinline__ void load_piece_step(const CoreParams &Q, const Piece &p, int32_t j0, int lane,
                                                 int32_t (&e)[kCorePer]) {
 #pragma unroll
-    for (int q = 0; q < kCorePer; ++q) {
-        const int32_t j = j0 + lane + 32 * q;
-        e[q] = j < p.cnt ? __ldcg(Q.pool + p.off + j) : p.v;
+    for (int h = 0; h < kCorePer / 4; ++h) {
+        const int32_t j = j0 + 128 * h + 4 * lane;
+        int4 x = make_int4(p.v, p.v, p.v, p.v);
+        if (j < p.cnt) x = __ldcg(reinterpret_cast<const int4 *>(Q.pool + p.off + j));
+        e[4 * h] = x.x;
+        e[4 * h + 1] = x.y;
+        e[4 * h + 2] = x.z;
+        e[4 * h + 3] = x.w;
     }
 }
 
-// One step of a piece: every slot's neighbour color into the round window (colors below 128 in
-// two per-lane registers, the warp's shared window up to 512) and the conflict flag (an entry with
-// the key bit whose neighbour has the vertex's color: tgt = cv | kCoreSmaller, never matched when cv
-// is saturated).  COMPACT: also the FINAL neighbours' colors into the final window, and the slots
-// kept (entries before `nvalid`, the entries of the step inside the piece, that are not FINAL).
-// Saturated 8-bit colors (255) are looked up exactly in cex.
+// One step of a piece: every slot's neighbour color marked in `seen`, and the conflict flag (an
+// entry with the key bit whose neighbour has the vertex's color: tgt = cv | kCoreSmaller, never matched
+// when cv is saturated).  COMPACT: also the FINAL neighbours' colors into the final window (flo: 0..63,
+// wfin above), and the slots kept (entries before `nvalid`, the entries of the step inside the piece,
+// that are not FINAL or whose color is saturated).  A saturated color (255) marks its byte; its
+// neighbours are looked up exactly when the piece ends.
 template <bool COMPACT>
-__device__ __forceinline__ void consume_step(const Shared &S, const int32_t (&e)[kCorePer], uint32_t tgt, int32_t cv,
-                                             const int32_t *cex_cur, uint64_t &lo, uint64_t &mid, uint64_t &flo,
-                                             unsigned *win, unsigned *wfin, unsigned &conflict, int32_t nvalid,
-                                             int lane, unsigned &keepm) {
+__device__ __forceinline__ void consume_step(const Shared &S, const int32_t (&e)[kCorePer], uint32_t tgt,
+                                             uint64_t &flo, uint8_t *seen, unsigned *wfin, bool &conflict,
+                                             int32_t nvalid, int lane, unsigned &keepm) {
     unsigned cs[kCorePer];
 #pragma unroll
     for (int q = 0; q < kCorePer; ++q) cs[q] = S.color8(static_cast<uint32_t>(e[q]) & ~kCoreSmaller);
-    unsigned sat = 0;
+    if constexpr (COMPACT) {
 #pragma unroll
-    for (int q = 0; q < kCorePer; ++q) {
-        const unsigned c = cs[q];
-        const uint64_t b = 1ull << (c & 63u);
-        if (c < 64u) {
-            lo |= b;
-        } else if (c < 128u) {
-            mid |= b;
-        } else if (c < kSat8) {
-            atomicOr(&win[c >> 5], 1u << (c & 31));
-        }
-        conflict |= static_cast<unsigned>(((static_cast<uint32_t>(e[q]) & kCoreSmaller) | c) == tgt);
-        sat |= static_cast<unsigned>(c == kSat8) << q;
-        if constexpr (COMPACT) {
-            const uint32_t id = static_cast<uint32_t>(e[q]) & ~kCoreSmaller;
-            const unsigned fin = S.final_bit(id);
+        for (int q = 0; q < kCorePer; ++q) {
+            const unsigned fin = S.final_bit(static_cast<uint32_t>(e[q]) & ~kCoreSmaller);
+            const unsigned c = cs[q];
             if (fin && c < kSat8) {
                 if (c < 64u)
-                    flo |= b;
+                    flo |= 1ull << c;
                 else
                     atomicOr(&wfin[c >> 5], 1u << (c & 31));
             }
-            keepm |= static_cast<unsigned>(!fin && lane + 32 * q < nvalid) << q;
+            keepm |= static_cast<unsigned>((!fin || c == kSat8) && 128 * (q >> 2) + 4 * lane + (q & 3) < nvalid) << q;
         }
     }
-    if (sat) {
-        // rare: colors of 255 and more, exactly
-#pragma unroll 1
-        for (int q = 0; q < kCorePer; ++q) {
-            if (!((sat >> q) & 1u)) continue;
-            const uint32_t id = static_cast<uint32_t>(e[q]) & ~kCoreSmaller;
-            const int32_t c = __ldcg(cex_cur + id);
-            if (static_cast<unsigned>(c) < 32u * kAccWords) {
-                atomicOr(&win[c >> 5], 1u << (c & 31));
-                if (COMPACT && S.final_bit(id)) atomicOr(&wfin[c >> 5], 1u << (c & 31));
-            }
-            if (e[q] < 0 && c == cv) conflict = 1u;
-        }
+#pragma unroll
+    for (int q = 0; q < kCorePer; ++q) {
+        conflict |= ((static_cast<uint32_t>(e[q]) & kCoreSmaller) | cs[q]) == tgt;
+        seen[cs[q]] = 1;
     }
 }
 
-// Vertices a warp finished that are not yet in the round's lists: lane k holds the k-th as
-// v | 8-bit color << 18 | kPendLose (v < 2^18: the core never has more vertices), and its range of
-// pieces.
-constexpr unsigned kPendLose = 1u << 26;
-
-// The round's output for the vertices a warp finished: a change-log entry each (C_{r+1} and the
-// FINAL flag), the losers' count and the losers' pieces (the next round's piece list); one
-// reservation per list.
-__device__ __forceinline__ void flush_pending(unsigned pend, unsigned pend_pb, unsigned pend_np, unsigned npend,
-                                              unsigned *cn, uint2 *log_next, int32_t *act_next, int lane) {
-    const bool act = static_cast<unsigned>(lane) < npend;
-    const unsigned v = pend & 0x3ffffu;
-    const bool lose = act && (pend & kPendLose) != 0u;
-    const unsigned pb = lose ? pend_pb : 0u, npc = lose ? pend_np : 0u;
-    const unsigned lm = __ballot_sync(kFull, lose);
-    unsigned incl = npc;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned y = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o) incl += y;
+// Rare (rounds past 255): the `cnt` entries of a piece with saturated neighbours looked at again for
+// exactly those: lane w returns word w of the window of their colors (255..511); the conflict.
+__device__ __noinline__ unsigned saturated_piece(const CoreParams &Q, const Shared &S, const Piece &p, int32_t cnt,
+                                                 const int32_t *cex_cur, int32_t cv, int lane, bool &conflict) {
+    unsigned word = 0;
+    for (int32_t j0 = 0; j0 < cnt; j0 += 32) {
+        const int32_t j = j0 + lane;
+        int32_t c = -1;
+        if (j < cnt) {
+            const uint32_t e = static_cast<uint32_t>(__ldcg(Q.pool + p.off + j)), id = e & ~kCoreSmaller;
+            if (S.color8(id) == kSat8) {
+                c = __ldcg(cex_cur + id);
+                if (e & kCoreSmaller) conflict |= c == cv;
+            }
+        }
+        for (unsigned open = __ballot_sync(kFull, c >= 0 && c < 32 * kAccWords); open; open &= open - 1u) {
+            const int32_t x = __shfl_sync(kFull, c, __ffs(static_cast<int>(open)) - 1);
+            if (lane == (x >> 5)) word |= 1u << (x & 31);
+        }
     }
-    const unsigned total = __shfl_sync(kFull, incl, 31);
-    unsigned lb = 0, ab = 0;
+    return word;
+}
+
+// The vertices a warp finished that are not yet in the round's lists: lane k holds the k-th (v |
+// kPendLose; the core never has 2^18 vertices), its C_{r+1}, its first piece and how many it has.
+constexpr unsigned kPendLose = 1u << 31;
+struct Pending {
+    unsigned v;
+    int32_t color;
+    unsigned piece, count;
+};
+
+// The lists of round `pass`'s worklist vertices: the pieces of those with one (counter word 2); first
+// piece and number of pieces of those with several (word 4).
+__device__ __forceinline__ int32_t *active_ones(const CoreParams &Q, int pass) {
+    return Q.active + static_cast<size_t>(pass & 1) * Q.max_v;
+}
+__device__ __forceinline__ int2 *active_many(const CoreParams &Q, int pass) {
+    return reinterpret_cast<int2 *>(Q.active + (2 + 2 * static_cast<size_t>(pass & 1)) * Q.max_v);
+}
+
+// The output of round `pass` for the vertices a warp finished, a lane each: C_{r+1} into the other color
+// buffers, a winner's FINAL bit, a change-log entry, the losers' count and the next round's lists; one
+// reservation per list.
+__device__ __forceinline__ void flush_pending(const CoreParams &Q, const Pending &pd, unsigned npend, unsigned *cn,
+                                              int pass, int lane) {
+    const size_t nxt = static_cast<size_t>((pass & 1) ^ 1);
+    const bool act = static_cast<unsigned>(lane) < npend;
+    const unsigned v = pd.v & ~kPendLose;
+    const bool lose = act && (pd.v & kPendLose) != 0u, many = pd.count > 1u;
+    const unsigned m1 = __ballot_sync(kFull, lose && !many), m2 = __ballot_sync(kFull, lose && many);
+    unsigned lb = 0, b1 = 0, b2 = 0;
     if (lane == 0) {
         lb = atomicAdd(cn, npend);
-        if (lm) atomicAdd(cn + 1, static_cast<unsigned>(__popc(lm)));
-        if (total) ab = atomicAdd(cn + 2, total);
+        if (m1 | m2) atomicAdd(cn + 1, static_cast<unsigned>(__popc(m1) + __popc(m2)));
+        if (m1) b1 = atomicAdd(cn + 2, static_cast<unsigned>(__popc(m1)));
+        if (m2) b2 = atomicAdd(cn + 4, static_cast<unsigned>(__popc(m2)));
+    }
+    const unsigned n8 = sat8(pd.color);
+    if (act) {
+        Q.cex[nxt * Q.max_v + v] = pd.color;
+        Q.c8[nxt * Q.max_v + v] = static_cast<uint8_t>(n8);
+        if (!lose) atomicOr(Q.fbits + (v >> 5), 1u << (v & 31));  // final for good: one bitmap
     }
     lb = __shfl_sync(kFull, lb, 0);
-    ab = __shfl_sync(kFull, ab, 0);
-    if (act) log_next[lb + lane] = make_uint2(v, ((pend >> 18) & 0xffu) | (lose ? 0u : 0x100u));
-    // the losers' pieces, written by the whole warp one vertex at a time
-    for (unsigned pm = __ballot_sync(kFull, npc > 0u); pm; pm &= pm - 1u) {
-        const int l = __ffs(pm) - 1;
-        const unsigned b0 = __shfl_sync(kFull, pb, l), k0 = __shfl_sync(kFull, npc, l);
-        const unsigned at = ab + __shfl_sync(kFull, incl, l) - k0;
-        for (unsigned k = lane; k < k0; k += 32) act_next[at + k] = static_cast<int32_t>(b0 + k);
-    }
+    b1 = __shfl_sync(kFull, b1, 0);
+    b2 = __shfl_sync(kFull, b2, 0);
+    if (act) Q.log[nxt * Q.max_v + lb + lane] = make_uint2(v, n8 | (lose ? 0u : 0x100u));
+    if (lose && !many) active_ones(Q, pass + 1)[b1 + __popc(m1 & lanemask_lt())] = static_cast<int32_t>(pd.piece);
+    if (lose && many)
+        active_many(Q, pass + 1)[b2 + __popc(m2 & lanemask_lt())] =
+            make_int2(static_cast<int32_t>(pd.piece), static_cast<int32_t>(pd.count));
 }
 
 // The first core round when the fill computed it (core_fused): a lane per vertex finishes it from
@@ -562,13 +584,13 @@ __device__ __forceinline__ void flush_pending(unsigned pend, unsigned pend_pb, u
 template <bool BATCH>
 __device__ void core_first_round(const RoundParams &P, const CoreParams &Q, int32_t m, int pass, unsigned *cn,
                                  int lane, unsigned &st_read, unsigned &st_deg, unsigned &st_cnt) {
-    const size_t cur = static_cast<size_t>(pass & 1), nxt = cur ^ 1u;
+    const size_t cur = static_cast<size_t>(pass & 1);
     const unsigned stride = gridDim.x * blockDim.x;
     for (unsigned base = (blockIdx.x * blockDim.x + threadIdx.x) & ~31u; base < static_cast<unsigned>(m);
          base += stride) {
         const unsigned v = base + lane;
         const bool in = v < static_cast<unsigned>(m);
-        unsigned pend = 0, pend_pb = 0, pend_np = 0;
+        Pending pd{0, 0, 0, 1};
         if (in) {
             unsigned *rec = core_rec(Q, v);
             const uint4 w = ldcg4(rec);
@@ -577,10 +599,6 @@ __device__ void core_first_round(const RoundParams &P, const CoreParams &Q, int3
             const int32_t cv = __ldcg(Q.cex + cur * Q.max_v + v);
             const uint64_t win = static_cast<uint64_t>(w.x | f.x) | (static_cast<uint64_t>(w.y | f.y) << 32);
             const int32_t nc = lose ? __ffsll(static_cast<long long>(~win)) - 1 : cv;
-            const unsigned n8 = sat8(nc);
-            Q.cex[nxt * Q.max_v + v] = nc;
-            Q.c8[nxt * Q.max_v + v] = static_cast<uint8_t>(n8);
-            if (!lose) atomicOr(Q.fbits + (v >> 5), 1u << (v & 31));
             const uint4 z = make_uint4(0, 0, 0, 0);
 #pragma unroll
             for (int c = 0; c < 20; c += 4) stcg4(rec + c, z);
@@ -591,55 +609,88 @@ __device__ void core_first_round(const RoundParams &P, const CoreParams &Q, int3
             if constexpr (BATCH) {
                 if (lose) note_graph_round(P, static_cast<int32_t>(__ldcg(rec + kCoreG)), pass + 1);
             }
-            pend = v | (n8 << 18) | (lose ? kPendLose : 0u);
-            pend_pb = __ldcg(rec + kCorePcBeg);
-            pend_np = __ldcg(rec + kCorePcEnd) - pend_pb;
+            pd.color = nc;
+            pd.piece = __ldcg(rec + kCorePcBeg);
+            pd.count = __ldcg(rec + kCorePcEnd) - pd.piece;
+            pd.v = v | (lose ? kPendLose : 0u);
         }
         const unsigned npend = static_cast<unsigned>(__popc(__ballot_sync(kFull, in)));
-        flush_pending(pend, pend_pb, pend_np, npend, cn, Q.log + nxt * Q.max_v, Q.active + nxt * Q.max_pieces, lane);
+        flush_pending(Q, pd, npend, cn, pass, lane);
     }
 }
 
-// One round for one warp: every active piece it owns, as one stream of steps (the next step's
-// entries, possibly the next piece's first ones and its record words, are loaded before the current
-// step is consumed).  For each piece: the round window (all neighbour colors), the conflict flag (a
-// smaller-key neighbour with the vertex's color) and, when the piece compacts, the window of final
-// colors of the neighbours it drops.  The vertex is finished by the warp that holds its last
-// piece: at once for a vertex with one piece; else every piece ORs its windows and flag into the
-// vertex's record and counts itself done, and the warp that completes the count reads the merged
-// record.  Finishing: a loser takes the least color absent from the round window and the final
-// window (its full row is rescanned past 512 colors), a winner becomes FINAL; C_{r+1} goes into the
-// other color buffers (a winner's FINAL bit into the bitmap) and the vertex into the warp's pending
-// batch for the change log and the next round's lists.
-template <bool BATCH>
-__device__ void core_round_warp(const RoundParams &P, const CoreParams &Q, const Shared &S, const int32_t *cex_cur,
-                                const int32_t *list, unsigned nact, int32_t m, unsigned nv, int pass,
-                                const DetState &st_r0, unsigned *cn, unsigned *grab, unsigned gw, unsigned nw,
-                                int lane, unsigned *win, unsigned *wfin, unsigned &st_read, unsigned &st_deg,
-                                unsigned &st_cnt) {
-    PieceCursor cur;
-    cur.act = 0;
-    cur.grab = nact >= kGrabMin * nw ? grab : nullptr;
-    cur.base = cur.grab ? 0u : gw;
-    const size_t nxt = static_cast<size_t>((pass & 1) ^ 1);
-    if (!cursor_load(cur, Q, list, nact, nw, lane)) return;
+// The vertices of several pieces a block takes at a time, in shared memory: their first piece, the
+// running count of pieces, the round window and conflict flag their pieces meet in and the pieces
+// done.  (Merged in the vertices' records in global memory, every piece waited for an acquire-release
+// atomic and the pieces had to be 4,096 entries long, so that a warp that drew several of a hub's
+// pieces held up the grid: blocks finished a heavy round between 90 and 140 us.)
+constexpr int kMany = 64;
+struct ManyShared {
+    unsigned first[kMany];
+    unsigned before[kMany + 1];  // pieces of the vertices before
+    unsigned win[kMany][kAccWords];
+    unsigned lost[kMany];
+    unsigned done[kMany];
+    unsigned next;  // the queue: pieces taken
+};
+
+// One round for one warp: pieces as one stream of steps (the next step's entries, possibly the next
+// piece's first ones and its record words, are loaded before the current step is consumed).  For each
+// piece: the round window (all neighbour colors), the conflict flag (a smaller-key neighbour with the
+// vertex's color) and, when the piece compacts, the window of final colors of the neighbours it drops.
+// MANY: the block's vertices of several pieces (M); each piece ORs its window and flag into the
+// vertex's slot and counts itself done, and the warp that completes the count finishes the vertex.
+// Else the one-piece vertices, each finished at once.  Finishing: a loser takes the least color absent
+// from the round window and the final window (its full row is rescanned past 512 colors), a winner
+// becomes FINAL; the vertex joins the warp's pending batch (flush_pending).
+//
+// What bounds it: issue slots and the latency of a piece's descriptor and entries.  A slot is about
+// seven instructions (a byte load, a byte store, the conflict test; with 64-bit register windows it
+// was 25), a piece adds about two hundred (its descriptor, windows and the finish), and pieces average
+// 350 entries on a power-law graph: a round of 64M entries over 135k vertices takes 110-140 us, 200
+// with the register windows.  R-MAT-22 18.05 -> 15.9 ms with four entries per lane and step (eight:
+// the same there, 1-5% slower on smaller graphs), 2,048-entry pieces (1,024: 6% slower, 4,096: 1%
+// faster there, 3% slower on smaller graphs) and 24 warps (32: 2-6% slower).
+template <bool BATCH, bool MANY>
+__device__ void core_stream(const RoundParams &P, const CoreParams &Q, const Shared &S, const int32_t *cex_cur,
+                            PieceCursor &cur, const int32_t *list, unsigned nact, unsigned nv, int pass,
+                            const DetState &st_r0, unsigned *cn, unsigned nw, int lane, uint8_t *seen, unsigned *wfin,
+                            ManyShared &M, int nmv, Pending &pd, unsigned &npend, unsigned &st_read, unsigned &st_deg,
+                            unsigned &st_cnt) {
+    // the next piece of this warp: its slot (MANY) or 0
+    auto next = [&](Piece &out, unsigned &idx, int &slot) -> bool {
+        if constexpr (MANY) {
+            unsigned q = 0;
+            if (lane == 0) q = atomicAdd(&M.next, 1u);
+            q = __shfl_sync(kFull, q, 0);
+            if (q >= M.before[nmv]) return false;
+            const unsigned lo = __ballot_sync(kFull, lane < nmv && M.before[min(lane + 1, nmv)] <= q);
+            const unsigned hi = __ballot_sync(kFull, lane + 32 < nmv && M.before[min(lane + 33, nmv)] <= q);
+            slot = __popc(lo) + __popc(hi);
+            idx = M.first[slot] + q - M.before[slot];
+            const int4 d = __ldcg(Q.pieces + idx);
+            out = Piece{d.x, d.y, d.z, d.w};
+            return true;
+        } else {
+            slot = 0;
+            return cursor_next(cur, Q, list, nact, nw, lane, out, idx);
+        }
+    };
+    if constexpr (!MANY) {
+        if (!cursor_load(cur, Q, list, nact, nw, lane)) return;
+    }
     Piece p;
     unsigned pidx = 0;
-    if (!cursor_next(cur, Q, list, nact, nw, lane, p, pidx)) return;
+    int slot = 0;
+    if (!next(p, pidx, slot)) return;
     int32_t e[kCorePer];
     load_piece_step(Q, p, 0, lane, e);
     // words 32..63 of the piece's vertex record: final window, row fields, piece range
     unsigned rx = __ldcg(core_rec(Q, p.v) + 32 + lane);
-    unsigned pend = 0, pend_pb = 0, pend_np = 0, npend = 0;
+    const int words = min(kSeen / 32, ((pass - 1) >> 5) + 1);  // colors of this round are below `pass`
     for (;;) {
-        // a piece starts: its windows, own color and compaction mode
-        if (lane < kAccWords) {
-            win[lane] = 0u;
-            wfin[lane] = 0u;
-        }
-        __syncwarp();
+        // a piece starts: its own color and compaction mode
         const unsigned own8 = S.color8(static_cast<uint32_t>(p.v));  // own color (never final on the worklist)
-        const int32_t cv = own8 == kSat8 ? __ldcg(cex_cur + p.v) : static_cast<int32_t>(own8);
         // the conflict test's target: the key bit and the vertex's 8-bit color (never matched when it
         // is saturated; those are compared exactly)
         const uint32_t tgt = kCoreSmaller | (own8 == kSat8 ? 0x1000u : own8);
@@ -647,31 +698,32 @@ __device__ void core_round_warp(const RoundParams &P, const CoreParams &Q, const
         // since the piece last did (its `flags` field records that worklist size): more often costs
         // more in writes than it saves in reads (a quarter: 1% slower on R-MAT-22; never: 25%)
         const bool compact = 2ull * nv < static_cast<unsigned long long>(static_cast<unsigned>(p.flags));
-        uint64_t lo = 0, mid = 0, flo = 0;
-        unsigned conflict = 0;
+        uint64_t flo = 0;
+        bool conflict = false;
         unsigned kept_total = 0;  // entries kept so far (the compaction position)
+        if (compact) {
+            if (lane < kAccWords) wfin[lane] = 0u;
+            __syncwarp();
+        }
         int32_t j0 = 0;
         for (;;) {
             // what comes next: this piece's next step or the next active piece's first step
             Piece pn = p;
             unsigned pnidx = pidx;
+            int slotn = slot;
             int32_t jn = j0 + kCoreStep;
             bool more = jn < p.cnt;
             unsigned rxn = rx;
             if (!more) {
-                more = cursor_next(cur, Q, list, nact, nw, lane, pn, pnidx);
+                more = next(pn, pnidx, slotn);
                 jn = 0;
                 if (more) rxn = __ldcg(core_rec(Q, pn.v) + 32 + lane);
             }
             int32_t en[kCorePer];
             if (more) load_piece_step(Q, pn, jn, lane, en);
             unsigned keepm = 0;
-            if (compact)
-                consume_step<true>(S, e, tgt, cv, cex_cur, lo, mid, flo, win, wfin, conflict, p.cnt - j0, lane, keepm);
-            else
-                consume_step<false>(S, e, tgt, cv, cex_cur, lo, mid, flo, win, wfin, conflict, p.cnt - j0, lane, keepm);
-            const unsigned kept = compact ? __reduce_add_sync(kFull, static_cast<unsigned>(__popc(keepm))) : 0u;
-            if (compact && kept) {
+            if (compact) {
+                consume_step<true>(S, e, tgt, flo, seen, wfin, conflict, p.cnt - j0, lane, keepm);
                 // in place: the positions written never pass the ones already read
                 unsigned pos = kept_total;
 #pragma unroll
@@ -681,105 +733,106 @@ __device__ void core_round_warp(const RoundParams &P, const CoreParams &Q, const
                     if (keep) Q.pool[p.off + pos + __popc(km & lanemask_lt())] = e[q];
                     pos += __popc(km);
                 }
+                kept_total = pos;
+            } else {
+                consume_step<false>(S, e, tgt, flo, seen, wfin, conflict, 0, lane, keepm);
             }
-            kept_total += kept;
             const bool piece_done = jn == 0 || !more;
             if (piece_done) {
-                const bool lose_p = __any_sync(kFull, conflict != 0u);
-                const unsigned lo0 = __reduce_or_sync(kFull, static_cast<unsigned>(lo));
-                const unsigned lo1 = __reduce_or_sync(kFull, static_cast<unsigned>(lo >> 32));
-                const unsigned lo2 = __reduce_or_sync(kFull, static_cast<unsigned>(mid));
-                const unsigned lo3 = __reduce_or_sync(kFull, static_cast<unsigned>(mid >> 32));
-                const unsigned f0 = __reduce_or_sync(kFull, static_cast<unsigned>(flo));
-                const unsigned f1 = __reduce_or_sync(kFull, static_cast<unsigned>(flo >> 32));
                 __syncwarp();
-                unsigned *rec = core_rec(Q, p.v);
-                // lanes 0..15: this piece's round window and final window; the final window as the
-                // record held it when the piece started
-                const unsigned rw = lane == 0 ? lo0 : lane == 1 ? lo1 : lane == 2 ? lo2 : lane == 3 ? lo3
-                                  : (lane < kAccWords ? win[lane] : 0u);
-                const unsigned fw = lane == 0 ? f0 : lane == 1 ? f1 : (lane < kAccWords ? wfin[lane] : 0u);
-                const unsigned fold = lane < kAccWords ? rx : 0u;
-                const unsigned npc = __shfl_sync(kFull, rx, kCorePcEnd - 32) - __shfl_sync(kFull, rx, kCorePcBeg - 32);
-                if (lane == 0) {
-                    st_read += static_cast<unsigned>(p.cnt);
-                    if (compact)
+                // lanes 0..15: word `lane` of this piece's round window, of its final window, and of the
+                // final window as the record held it when the piece started
+                unsigned rw = 0, fw = 0;
+                for (int w = 0; w < words; ++w) {
+                    const unsigned b = __ballot_sync(kFull, seen[32 * w + lane] != 0);
+                    if (lane == w) rw = b;
+                }
+                __syncwarp();
+                *reinterpret_cast<uint2 *>(seen + 8 * lane) = make_uint2(0u, 0u);
+                if (compact) {
+                    const unsigned f0 = __reduce_or_sync(kFull, static_cast<unsigned>(flo));
+                    const unsigned f1 = __reduce_or_sync(kFull, static_cast<unsigned>(flo >> 32));
+                    fw = lane == 0 ? f0 : lane == 1 ? f1 : (lane < kAccWords ? wfin[lane] : 0u);
+                    if (lane == 0)
                         reinterpret_cast<int2 *>(Q.pieces + pidx)[1] =
                             make_int2(static_cast<int32_t>(kept_total), static_cast<int32_t>(nv));
                 }
-                bool lose = lose_p, finish = true;
-                unsigned tw = 0;  // lanes 0..15: colors 32 lane .. 32 lane + 31 around the vertex
-                if (npc <= 1u) {
-                    if (lane < kAccWords && (fw & ~fold)) rec[kAccFin + lane] = fold | fw;
-                    tw = rw | fw | fold;
-                } else {
-                    if (lane < kAccWords && rw) atomicOr(rec + lane, rw);
-                    if (lane < kAccWords && (fw & ~fold)) atomicOr(rec + kAccFin + lane, fw);
-                    if (lane == 0 && lose_p) atomicOr(rec + kCoreFlag, 1u);
-                    // the piece that completes the count (release: its merges first; acquire: the others')
-                    __syncwarp();
-                    unsigned done = 0;
-                    if (lane == 0) done = atom_add_acq_rel(rec + kCoreDone, 1u);
-                    done = __shfl_sync(kFull, done, 0);
-                    finish = done == npc - 1u;
-                    if (finish) {
-                        __syncwarp();
-                        const unsigned x = __ldcg(rec + lane);  // window (lanes 0..15), flag (lane 16)
-                        const unsigned fx = lane < kAccWords ? __ldcg(rec + kAccFin + lane) : 0u;
-                        lose = __shfl_sync(kFull, x, kCoreFlag) != 0u;
-                        tw = lane < kAccWords ? (x | fx) : 0u;
-                        __syncwarp();
-                        if (lane <= kCoreDone) rec[lane] = 0u;  // the round part, for the next round
+                if (pass > static_cast<int>(kSat8)) {
+                    const bool sat = __shfl_sync(kFull, rw, kSeen / 32 - 1) >> 31;
+                    if (lane == kSeen / 32 - 1) rw &= 0x7fffffffu;
+                    if (sat) {
+                        const int32_t cv = __ldcg(cex_cur + p.v);
+                        rw |= saturated_piece(Q, S, p, compact ? static_cast<int32_t>(kept_total) : p.cnt, cex_cur,
+                                              cv, lane, conflict);
                     }
                 }
+                bool lose = __any_sync(kFull, conflict), finish = true;
+                const unsigned fold = lane < kAccWords ? rx : 0u;
+                if (lane == 0) st_read += static_cast<unsigned>(p.cnt);
+                unsigned tw = rw | fold;  // lanes 0..15: colors 32 lane .. 32 lane + 31 around the vertex
+                unsigned *rec = core_rec(Q, p.v);
+                if constexpr (MANY) {
+                    // into the vertex's slot; the dropped neighbours' colors (part of this round's window,
+                    // too) into its record for the rounds to come
+                    if (fw & ~fold) atomicOr(rec + kAccFin + lane, fw);
+                    if (rw) atomicOr(&M.win[slot][lane], rw);
+                    if (lane == 0 && lose) M.lost[slot] = 1u;
+                    __threadfence_block();
+                    __syncwarp();
+                    unsigned done = 0;
+                    if (lane == 0) done = atomicAdd(&M.done[slot], 1u);
+                    done = __shfl_sync(kFull, done, 0);
+                    finish = done == M.before[slot + 1] - M.before[slot] - 1u;
+                    if (finish) {
+                        __threadfence_block();
+                        tw = lane < kAccWords ? (*const_cast<volatile unsigned *>(&M.win[slot][lane]) | fold) : 0u;
+                        lose = *const_cast<volatile unsigned *>(&M.lost[slot]) != 0u;
+                    }
+                } else {
+                    if (fw & ~fold) rec[kAccFin + lane] = fold | fw;
+                }
                 if (finish) {
-                    const int32_t v = p.v;
-                    int32_t nc = cv;
+                    int32_t nc;
                     if (lose) {
                         const unsigned fm = __ballot_sync(kFull, lane < kAccWords && ~tw != 0u);
                         if (fm) {
                             const int l = __ffs(fm) - 1;
                             nc = 32 * l + __ffs(~__shfl_sync(kFull, tw, l)) - 1;
                         } else {
+                            // (the warp's `seen` bytes, cleared above, hold the rescan's window)
+                            __syncwarp();
                             nc = core_mex_from<BATCH>(P, st_r0, static_cast<int32_t>(__shfl_sync(kFull, rx, kCoreGid - 32)),
-                                                      cex_cur, win, lane, 32 * kAccWords);
+                                                      cex_cur, reinterpret_cast<unsigned *>(seen), lane, 32 * kAccWords);
+                            *reinterpret_cast<uint2 *>(seen + 8 * lane) = make_uint2(0u, 0u);
                         }
+                    } else {  // a winner keeps its color
+                        nc = own8 == kSat8 ? __ldcg(cex_cur + p.v) : static_cast<int32_t>(own8);
                     }
-                    const unsigned deg = __shfl_sync(kFull, rx, kCoreDeg - 32);
-                    const unsigned n8 = sat8(nc);
-                    if (lane == 0) {
-                        Q.cex[nxt * Q.max_v + v] = nc;
-                        Q.c8[nxt * Q.max_v + v] = static_cast<uint8_t>(n8);
-                        if (!lose) atomicOr(Q.fbits + (v >> 5), 1u << (v & 31));  // final for good: one bitmap
-                        st_deg += deg;
-                        st_cnt += 1;
+                    if (P.stats) {
+                        const unsigned deg = __shfl_sync(kFull, rx, kCoreDeg - 32);
+                        if (lane == 0) {
+                            st_deg += deg;
+                            st_cnt += 1;
+                        }
                     }
                     if constexpr (BATCH) {
                         const unsigned g = __shfl_sync(kFull, rx, kCoreG - 32);
                         if (lane == 0 && lose) note_graph_round(P, static_cast<int32_t>(g), pass + 1);
                     }
-                    const unsigned pb = __shfl_sync(kFull, rx, kCorePcBeg - 32);
-                    if (static_cast<unsigned>(lane) == npend) {
-                        pend = static_cast<unsigned>(v) | (n8 << 18) | (lose ? kPendLose : 0u);
-                        pend_pb = pb;
-                        pend_np = npc;
-                    }
+                    if (static_cast<unsigned>(lane) == npend)
+                        pd = Pending{static_cast<unsigned>(p.v) | (lose ? kPendLose : 0u), nc, MANY ? M.first[slot] : pidx,
+                                     MANY ? M.before[slot + 1] - M.before[slot] : 1u};
                     if (++npend == 32u) {
-                        flush_pending(pend, pend_pb, pend_np, npend, cn, Q.log + nxt * Q.max_v,
-                                      Q.active + nxt * Q.max_pieces, lane);
+                        flush_pending(Q, pd, npend, cn, pass, lane);
                         npend = 0;
                     }
                 }
                 __syncwarp();
             }
-            if (!more) {
-                if (npend)
-                    flush_pending(pend, pend_pb, pend_np, npend, cn, Q.log + nxt * Q.max_v,
-                                  Q.active + nxt * Q.max_pieces, lane);
-                return;
-            }
+            if (!more) return;
             p = pn;
             pidx = pnidx;
+            slot = slotn;
             rx = rxn;
             j0 = jn;
 #pragma unroll
@@ -787,6 +840,60 @@ __device__ void core_round_warp(const RoundParams &P, const CoreParams &Q, const
             if (piece_done) break;
         }
     }
+}
+
+// A round: the block's share of the vertices of several pieces (every grid-th of the list, kMany at a
+// time), then the warp's share of the others.
+template <bool BATCH>
+__device__ void core_round(const RoundParams &P, const CoreParams &Q, const Shared &S, const int32_t *cex_cur,
+                           unsigned none, unsigned nmany, unsigned nv, int pass, const DetState &st_r0, unsigned *cn,
+                           unsigned *grab, unsigned gw, unsigned nw, int lane, int wib, uint8_t *seen, unsigned *wfin,
+                           ManyShared &M, unsigned &st_read, unsigned &st_deg, unsigned &st_cnt) {
+    Pending pd{0, 0, 0, 1};
+    unsigned npend = 0;
+    PieceCursor cur;
+    cur.act = 0;
+    cur.grab = none >= kGrabMin * nw ? grab : nullptr;
+    cur.base = cur.grab ? 0u : gw;
+    const int2 *many = active_many(Q, pass);
+    const unsigned mine = nmany > blockIdx.x ? (nmany - 1u - blockIdx.x) / gridDim.x + 1u : 0u;
+    for (unsigned c0 = 0; c0 < mine; c0 += kMany) {
+        const int nmv = static_cast<int>(min(mine - c0, static_cast<unsigned>(kMany)));
+        __syncthreads();  // the previous chunk's slots are done with
+        for (int i = threadIdx.x; i < nmv * kAccWords; i += blockDim.x) M.win[i / kAccWords][i % kAccWords] = 0u;
+        if (wib == 0) {
+            // two vertices a lane: their pieces and the running count
+            unsigned np[2] = {0, 0};
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int t = 2 * lane + h;
+                if (t >= nmv) continue;
+                const int2 x = __ldcg(many + blockIdx.x + (c0 + static_cast<unsigned>(t)) * gridDim.x);
+                np[h] = static_cast<unsigned>(x.y);
+                M.first[t] = static_cast<unsigned>(x.x);
+                M.lost[t] = 0u;
+                M.done[t] = 0u;
+            }
+            unsigned incl = np[0] + np[1];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned y = __shfl_up_sync(kFull, incl, o);
+                if (lane >= o) incl += y;
+            }
+            if (2 * lane < nmv) M.before[2 * lane + 1] = incl - np[1];
+            if (2 * lane + 1 < nmv) M.before[2 * lane + 2] = incl;
+            if (lane == 0) {
+                M.before[0] = 0u;
+                M.next = 0u;
+            }
+        }
+        __syncthreads();
+        core_stream<BATCH, true>(P, Q, S, cex_cur, cur, nullptr, 0u, nv, pass, st_r0, cn, nw, lane, seen, wfin, M, nmv,
+                                 pd, npend, st_read, st_deg, st_cnt);
+    }
+    core_stream<BATCH, false>(P, Q, S, cex_cur, cur, active_ones(Q, pass), none, nv, pass, st_r0, cn, nw, lane,
+                              seen, wfin, M, 0, pd, npend, st_read, st_deg, st_cnt);
+    if (npend) flush_pending(Q, pd, npend, cn, pass, lane);
 }
 
 #ifdef GC_CORE_PROFILE
@@ -804,7 +911,7 @@ __device__ unsigned long long g_core_prof[8 * 4096];
 template <bool BATCH>
 __global__ void __launch_bounds__(kCoreThreads, 1) core_round_kernel(RoundParams P, CoreParams Q) {
     extern __shared__ __align__(16) unsigned char s_dyn[];
-    __shared__ unsigned s_win[kCoreWarps][kAccWords];
+    __shared__ __align__(16) uint8_t s_seen[kCoreWarps][kSeen];
     __shared__ unsigned s_fin[kCoreWarps][kAccWords];
     if (__ldcg(P.core_go) == 0) return;
     const HandOver h = hand_over(P);
@@ -818,19 +925,23 @@ __global__ void __launch_bounds__(kCoreThreads, 1) core_round_kernel(RoundParams
         Q.m[1] = static_cast<unsigned>(m);
         Q.m[3] = static_cast<unsigned>(R0);
     }
+    __shared__ ManyShared s_many;
+    *reinterpret_cast<uint2 *>(s_seen[wib] + 8 * lane) = make_uint2(0u, 0u);
     Shared S;
     S.col = s_dyn;
     S.fin = reinterpret_cast<unsigned *>(s_dyn + Q.max_v);
     load_shared(S, Q, Q.c8 + static_cast<size_t>(R0 & 1) * Q.max_v, m);
     {
-        // the pieces of every row: consecutive pieces of a row go to consecutive warps
+        // the pieces of every row, and the first round's lists
         const unsigned stride = gridDim.x * blockDim.x;
+        unsigned *c0 = Q.cnt + kCoreCnt * (R0 % 3);
         for (unsigned base = (blockIdx.x * blockDim.x + threadIdx.x) & ~31u; base < static_cast<unsigned>(m);
              base += stride) {
             const unsigned v = base + lane;
+            const bool in = v < static_cast<unsigned>(m);
             unsigned len = 0, np = 0;
             uint64_t off = 0;
-            if (v < static_cast<unsigned>(m)) {
+            if (in) {
                 const unsigned *rec = core_rec(Q, v);
                 len = __ldcg(rec + kCoreFill);  // the row as the fill kernel wrote it
                 off = static_cast<uint64_t>(__ldcg(rec + kCoreOffLo)) |
@@ -844,30 +955,44 @@ __global__ void __launch_bounds__(kCoreThreads, 1) core_round_kernel(RoundParams
                 if (lane >= o) incl += y;
             }
             const unsigned total = __shfl_sync(kFull, incl, 31);
-            unsigned b = 0;
-            if (lane == 0 && total) b = atomicAdd(Q.m + 2, total);
-            b = __shfl_sync(kFull, b, 0);
-            if (v < static_cast<unsigned>(m)) {
-                unsigned *rec = core_rec(Q, v);
-                rec[kCorePcBeg] = b + incl - np;
-                rec[kCorePcEnd] = b + incl;
+            const unsigned m1 = __ballot_sync(kFull, in && np == 1u), m2 = __ballot_sync(kFull, in && np > 1u);
+            unsigned b = 0, b1 = 0, b2 = 0;
+            if (lane == 0) {
+                b = atomicAdd(Q.m + 2, total);
+                if (m1) b1 = atomicAdd(c0 + 2, static_cast<unsigned>(__popc(m1)));
+                if (m2) b2 = atomicAdd(c0 + 4, static_cast<unsigned>(__popc(m2)));
             }
+            b = __shfl_sync(kFull, b, 0) + incl - np;
+            b1 = __shfl_sync(kFull, b1, 0) + __popc(m1 & lanemask_lt());
+            b2 = __shfl_sync(kFull, b2, 0) + __popc(m2 & lanemask_lt());
+            if (!in) continue;
+            unsigned *rec = core_rec(Q, v);
+            rec[kCorePcBeg] = b;
+            rec[kCorePcEnd] = b + np;
+            if (np == 1u)
+                active_ones(Q, R0)[b1] = static_cast<int32_t>(b);
+            else
+                active_many(Q, R0)[b2] = make_int2(static_cast<int32_t>(b), static_cast<int32_t>(np));
             for (unsigned k = 0; k < np; ++k) {
                 const unsigned lb = k * kCorePiece;
-                Q.pieces[b + incl - np + k] =
-                    make_int4(static_cast<int32_t>(v), static_cast<int32_t>(off + lb),
-                              static_cast<int32_t>(min(len - lb, static_cast<unsigned>(kCorePiece))), m);
+                Q.pieces[b + k] = make_int4(static_cast<int32_t>(v), static_cast<int32_t>(off + lb),
+                                            static_cast<int32_t>(min(len - lb, static_cast<unsigned>(kCorePiece))), m);
             }
+            // the slots up to the next multiple of four hold the vertex itself (no conflict, and a color
+            // a loser's window holds anyway)
+            for (unsigned k = len; k & 3u; ++k) Q.pool[off + k] = static_cast<int32_t>(v);
         }
     }
     unsigned bar_target = 0;
     int pass = R0;
     if (grid_sync(P.bar, bar_target, P.err, P.spin_ns)) {
-        const unsigned npieces = __ldcg(Q.m + 2);
         for (;; ++pass) {
-            // the previous round's counts: {change-log entries, losers, pieces listed, -}
-            const uint4 cc = ldcg4(Q.cnt + 4 * (pass % 3));
-            unsigned *cn = Q.cnt + 4 * ((pass + 1) % 3);
+            // the previous round's counts: {change-log entries, losers, one-piece vertices listed, -, vertices
+            // of several pieces listed}
+            unsigned *cset = Q.cnt + kCoreCnt * (pass % 3);
+            const uint4 cc = ldcg4(cset);
+            const unsigned nmany = __ldcg(cset + 4);
+            unsigned *cn = Q.cnt + kCoreCnt * ((pass + 1) % 3);
             // |W_pass|: every core vertex in the first round, then the previous round's losers
             const unsigned nv = pass == R0 ? static_cast<unsigned>(m) : cc.y;
             if (nv == 0u) break;
@@ -885,7 +1010,7 @@ __global__ void __launch_bounds__(kCoreThreads, 1) core_round_kernel(RoundParams
                 }
                 break;
             }
-            if (blockIdx.x == 0 && threadIdx.x < 4) Q.cnt[4 * ((pass + 2) % 3) + threadIdx.x] = 0u;
+            if (blockIdx.x == 0 && threadIdx.x < kCoreCnt) Q.cnt[kCoreCnt * ((pass + 2) % 3) + threadIdx.x] = 0u;
             CORE_PROF(0, atomicMin);
 #ifdef GC_CORE_PROFILE
             if (blockIdx.x == 0 && threadIdx.x == 0 && pass - R0 < 4096) g_core_prof[8 * (pass - R0) + 7] = nv;
@@ -902,16 +1027,12 @@ __global__ void __launch_bounds__(kCoreThreads, 1) core_round_kernel(RoundParams
             __syncthreads();
             CORE_PROF(1, atomicMax);
             unsigned st_deg = 0, st_cnt = 0, st_read = 0;
-            // the round's pieces: all of them in the first round, then those the previous round listed
-            const int32_t *list = pass == R0 ? nullptr : Q.active + static_cast<size_t>(pass & 1) * Q.max_pieces;
-            const unsigned nact = pass == R0 ? npieces : cc.z;
-            // the round's grab counter: word 3 of its counter set (cleared two rounds ahead like the rest)
+            // (word 3 of the counter set is the round's grab counter)
             if (pass == R0 && core_fused(R0))
                 core_first_round<BATCH>(P, Q, m, pass, cn, lane, st_read, st_deg, st_cnt);
             else
-                core_round_warp<BATCH>(P, Q, S, cex_cur, list, nact, m, nv, pass, h.st, cn,
-                                       Q.cnt + 4 * (pass % 3) + 3, gw, nw, lane, s_win[wib], s_fin[wib], st_read,
-                                       st_deg, st_cnt);
+                core_round<BATCH>(P, Q, S, cex_cur, cc.z, nmany, nv, pass, h.st, cn, cset + 3, gw, nw, lane, wib,
+                                  s_seen[wib], s_fin[wib], s_many, st_read, st_deg, st_cnt);
 #ifdef GC_CORE_PROFILE
             __syncthreads();
             CORE_PROF(2, atomicMin);

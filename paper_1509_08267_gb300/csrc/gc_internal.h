@@ -174,8 +174,9 @@ inline void set_det_state(RoundParams &P, void *buf0, void *buf1, size_t n) {
 // active pieces hands out to the warps.
 constexpr uint32_t kCoreSmaller = 0x80000000u;
 constexpr int64_t kCoreEntries = int64_t{1} << 27;  // list entries the core phase takes at most
+constexpr int kCoreCnt = 8;  // counter words per set
 #ifndef GC_CORE_PIECE
-#define GC_CORE_PIECE 4096
+#define GC_CORE_PIECE 2048
 #endif
 constexpr int kCorePiece = GC_CORE_PIECE;
 // Per core vertex, kCoreRecWords words: [0, 16) the round's window of neighbour colors 0..511,
@@ -208,11 +209,13 @@ struct CoreParams {
     uint8_t *c8;          // [2][M] colors saturated at 255, double-buffered like cex
     unsigned *fbits;      // [M / 32 + 1] FINAL bit of every core vertex (zero at hand-over)
     int4 *pieces;         // [max_pieces] {local vertex, pool offset, entries, flags}
-    int32_t *active;      // [2][max_pieces] the pieces of each round's worklist vertices
+    int32_t *active;      // each round's worklist: [2][M] pieces of the one-piece vertices, [2][M] {first piece,
+                          // pieces} of the others
     uint2 *log;           // [2][M] {local vertex, 8-bit color | FINAL << 8} of the vertices a round finished
     int32_t *pool;        // [max_e] the rows
     unsigned long long *bump;  // pool allocation counter
-    unsigned *cnt;        // [3][4] per-round counters: vertices finished (log entries), losers, active pieces
+    unsigned *cnt;        // [3][kCoreCnt] per-round counters: vertices finished (log entries), losers, one-piece
+                          // vertices, grabs, vertices of several pieces
     unsigned *m;          // [4]: larger vertices numbered by the index kernel, m, pieces
     int32_t tail_max;     // tail phase once the worklist has at most this many vertices (0: never)
     int32_t tail_nc;      // blocks of the tail's cluster (tail_max <= kTailOwned * tail_nc)

@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(kTailThreads, 1) tail_kernel(RoundParams P, Co
     int32_t *kid = reinterpret_cast<int32_t *>(key2 + kt);
 
     // W_R1: the losers in the change log of round R1 - 1, in log order (the same in every block)
-    const uint4 cc = ldcg4(Q.cnt + 4 * (R1 % 3));
+    const uint4 cc = ldcg4(Q.cnt + kCoreCnt * (R1 % 3));
     const uint2 *log = Q.log + static_cast<size_t>(R1 & 1) * Q.max_v;
     if (threadIdx.x == 0) s_k = 0;
     __syncthreads();
