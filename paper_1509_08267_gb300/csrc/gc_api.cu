@@ -90,6 +90,8 @@ struct Ctl {
     alignas(16) unsigned core_cnt[3 * kCoreCnt];  // each set's first four read with one 16-byte load
     unsigned core_m[4];
     unsigned tail_ctl[4];  // tail phase: handed over, first round
+    unsigned small_ctl[4];  // small graphs: a batch's queued and taken graphs; a cluster's losers per round
+    unsigned long long small_left;  // vertices of the graphs that are not small
     GridBar bar;
 };
 static_assert(offsetof(Ctl, bar) % 128 == 0, "barrier alignment");
@@ -105,6 +107,9 @@ struct Context {
     int occ_ord[2] = {};    // blocks per SM of the ordered-mode round kernel [batch]
     int occ_peel = 0;       // blocks per SM of the peeling kernel
     Buf col0, col1, small0, small1, items, chunk0, chunk1, acc, lists, ctl, stats, bitmap, vg, hist;
+    Buf small_queue, small_done;  // a batch's small graphs
+    int32_t *small_result = nullptr;  // pinned host words small_one_kernel writes
+    int small_blocks = -1;  // its cluster (-1: not asked yet)
     Buf gmax, gcount, glast, g_vbase, g_n, g_ebase, g_rbase, g_m;
     Buf st_rowptr, st_colidx, st_vtx, st_edge, st_colors, st_colors_in, mid0, mid1, rank;
     Buf core_rec, core_cex, core_c8, core_fbits, core_items, core_active, core_log, core_pool;
@@ -120,7 +125,7 @@ struct Context {
         Buf *all[] = {&col0, &col1, &small0, &small1, &items, &chunk0, &chunk1, &acc, &lists, &ctl, &stats, &bitmap, &hist,
                       &vg, &gmax, &gcount, &glast, &g_vbase, &g_n, &g_ebase, &g_rbase, &g_m, &st_rowptr, &st_colidx, &st_vtx, &st_edge, &st_colors, &st_colors_in, &mid0, &mid1, &rank,
                       &core_rec, &core_cex, &core_c8, &core_fbits, &core_items, &core_active, &core_log, &core_pool,
-                      &st_cur, &st_work, &st_next, &st_lost};
+                      &st_cur, &st_work, &st_next, &st_lost, &small_queue, &small_done};
         for (Buf *b : all) b->release();
     }
 };
@@ -327,6 +332,104 @@ static int peel_levels(Context &C, Ctl *ctl, RoundParams P, int32_t T1, int32_t 
     return GC_OK;
 }
 
+// Options that leave every choice to the library and ask for nothing but the coloring (a round cap
+// and a stream aside): such calls may take the small-graph kernels.
+static bool plain_options(const gc_options *o) {
+    return !o || (o->small_max_degree == 0 && o->chunk == 0 && o->block_size == 0 && o->blocks_per_sm == 0 &&
+                  o->spin_limit_ns == 0 && o->flags == 0 && o->core_vertices == 0 && o->core_entries == 0 &&
+                  o->tail_vertices == 0);
+}
+
+static int32_t round_cap(const gc_options *o, int64_t n) {
+    return o && o->max_rounds > 0 ? o->max_rounds : static_cast<int32_t>(n < INT32_MAX ? n + 1 : INT32_MAX);
+}
+
+// A small single graph in one launch (gc_small.cu).  rowptr and colidx are device memory; colors may
+// be a host array.  *handled: the call is done (else *nnz, if not -1, has been read on the way).
+static int color_small(Context &C, int32_t n, const int32_t *rowptr, const int32_t *colidx, uint64_t seed,
+                       const gc_options *opt, gc_stats *stats, const Outputs &out, cudaStream_t s, bool *handled,
+                       int64_t *nnz) {
+    NvtxRange range("gc: small coloring");
+    *handled = false;
+    if (C.small_blocks < 0) C.small_blocks = small_one_blocks();
+    if (!C.small_result) {
+        if (cudaHostAlloc(reinterpret_cast<void **>(&C.small_result), 64, cudaHostAllocPortable | cudaHostAllocMapped) !=
+            cudaSuccess) {
+            cudaGetLastError();
+            C.small_result = nullptr;
+            return GC_OK;
+        }
+    }
+    GC_TRY(ensure(C.ctl, sizeof(Ctl), "control"));
+    GC_TRY(ensure(C.col0, 8 * static_cast<size_t>(kSmallOneVertices), "vertex state"));
+    int out_dev = 0;
+    GC_TRY(locate(out.colors, C.device, &out_dev));
+    if (!out_dev) GC_TRY(ensure(C.st_colors, 4 * static_cast<size_t>(n), "color staging"));
+    Ctl *ctl = C.ctl.as<Ctl>();
+    RoundParams P{};
+    P.n = n;
+    P.G = 1;
+    P.rowptr = rowptr;
+    P.colidx = colidx;
+    P.seed = seed;
+    P.priority = opt ? opt->priority : GC_PRIORITY_HASH;
+    const int32_t cap_rounds = round_cap(opt, n);
+    P.pass_begin = 1;
+    P.pass_end = cap_rounds < INT32_MAX ? cap_rounds + 1 : INT32_MAX;
+    P.cap_is_error = 1;
+    P.err = ctl->err;
+    SmallOne A{};
+    A.exchange = C.col0.as<uint32_t>();
+    A.cnt = ctl->small_ctl;
+    A.out = out_dev ? out.colors : C.st_colors.as<int32_t>();
+    void *mapped = nullptr;
+    GC_CUDA(cudaHostGetDevicePointer(&mapped, C.small_result, 0));
+    A.result = static_cast<int32_t *>(mapped);
+    volatile int32_t *res = C.small_result;
+    const int64_t most = kSmallOneRow * n;
+    int blocks = n <= kSmallBlockVertices ? 1 : C.small_blocks;
+    for (; blocks > 0; blocks = C.small_blocks) {
+        A.cap = (n + 7) & ~7;
+        A.max_entries = std::min(most, blocks == 1 ? kSmallBlockEntries : kSmallOneEntries);
+        GC_CUDA(launch_small_one(P, A, blocks, s));
+        GC_CUDA(cudaStreamSynchronize(s));
+        *nnz = res[1];
+        if (res[0] != 1) break;
+        if (blocks > 1 || res[1] < 0 || res[1] > std::min(most, kSmallOneEntries)) return GC_OK;
+    }
+    if (blocks <= 0) return GC_OK;
+    *handled = true;
+    if (res[0] != 0) {
+        Ctl h{};
+        for (int k = 0; k < 4; ++k) h.err[k] = res[5 + k];
+        return error_from_ctl(h);
+    }
+    if (!out_dev) {
+        GC_CUDA(cudaMemcpyAsync(out.colors, C.st_colors.p, 4 * static_cast<size_t>(n), cudaMemcpyDeviceToHost, s));
+        GC_CUDA(cudaStreamSynchronize(s));
+    }
+    const int32_t rounds = res[2] > 0 ? res[2] : 1;
+    if (out.ncolors) *out.ncolors = res[3];
+    if (out.rounds) *out.rounds = rounds;
+    if (stats) {
+        stats->rounds = rounds;
+        stats->ncolors = res[3];
+        stats->max_color = res[4];
+        stats->grid_blocks = blocks;
+        stats->block_size = 1024;
+        stats->worklist_total = 0;
+        stats->entries_scanned = 0;
+        stats->kernel_ms = 0.f;
+        stats->setup_ms = 0.f;
+    }
+    return GC_OK;
+}
+
+static bool small_candidate(int32_t n, int mode, const gc_options *opt) {
+    return mode == GC_MODE_DETERMINISTIC && n <= kSmallOneVertices && plain_options(opt) &&
+           (!opt || opt->priority == GC_PRIORITY_HASH || opt->priority == GC_PRIORITY_LARGEST_FIRST);
+}
+
 static int run(Context &C, const Problem &pb, int mode, uint64_t seed, const gc_options *opt, gc_stats *stats,
                const Outputs &out) {
     NvtxRange range(pb.batch ? "gc: batch coloring" : "gc: coloring");
@@ -348,8 +451,7 @@ static int run(Context &C, const Problem &pb, int mode, uint64_t seed, const gc_
     const int32_t priority = pb.priority_override >= 0 ? pb.priority_override : opt_priority;
     const int64_t n = pb.n;
     const int32_t G = pb.G;
-    const int32_t max_rounds =
-        (opt && opt->max_rounds > 0) ? opt->max_rounds : static_cast<int32_t>(n < INT32_MAX ? n + 1 : INT32_MAX);
+    const int32_t max_rounds = round_cap(opt, n);
     const int64_t spin_ns = (opt && opt->spin_limit_ns > 0) ? opt->spin_limit_ns : 1000000000LL;
     const int32_t stats_cap = (flags & GC_FLAG_STATS) ? (max_rounds < 65536 ? max_rounds : 65536) : 0;
     const size_t gz = static_cast<size_t>(G);
@@ -443,13 +545,25 @@ static int run(Context &C, const Problem &pb, int mode, uint64_t seed, const gc_
 
     const bool timing = (flags & GC_FLAG_TIMING) != 0;
     Ctl h{};
+    bool small = false;
     if (pb.batch) {
         GC_CUDA(launch_batch_tables(P, pb.vtx_off, pb.edge_off, C.g_vbase.as<int64_t>(), C.g_n.as<int32_t>(),
                                     C.g_ebase.as<int64_t>(), C.g_rbase.as<int64_t>(), C.g_m.as<int64_t>(), s));
+        small = mode == GC_MODE_DETERMINISTIC && plain_options(opt);
+        if (small) {
+            // the small graphs, by one block each; the rest of this call skips them
+            GC_TRY(ensure(C.small_queue, 4 * gz, "small graphs"));
+            GC_TRY(ensure(C.small_done, gz, "small graphs"));
+            P.g_done = C.small_done.as<uint8_t>();
+            const SmallBatch B{C.small_queue.as<int32_t>(), ctl->small_ctl, ctl->small_ctl + 1, &ctl->small_left,
+                               C.small_done.as<uint8_t>()};
+            GC_CUDA(launch_small_batch(P, B, pb.nnz, s));
+        }
         GC_CUDA(cudaMemcpyAsync(&h, ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
         GC_CUDA(cudaStreamSynchronize(s));
         if (h.err[0] != 0) return error_from_ctl(h);
     }
+    const bool rest = !small || h.small_left != 0;  // graphs the small-graph kernel left
     if (timing) GC_CUDA(cudaEventRecord(C.ev[0], s));
     if (priority == GC_PRIORITY_SMALLEST_LAST && mode != GC_MODE_PARTITION && n > 0) {
         GC_TRY(wait_colidx(pb, s));
@@ -520,7 +634,7 @@ static int run(Context &C, const Problem &pb, int mode, uint64_t seed, const gc_
         grid = static_cast<int64_t>(per_sm) * C.sms;
         GC_TRY(wait_colidx(pb, s));
         GC_CUDA(launch_ordered(P, pb.batch, reinterpret_cast<int32_t *>(C.col1.p), static_cast<int>(grid), block, s));
-    } else {
+    } else if (rest) {
     GC_CUDA(launch_setup(P, mode, pb.batch, 0, static_cast<int32_t>(n), -1, s));
     GC_CUDA(launch_sort_small(P, pb.batch, 0, static_cast<int32_t>(n), s));
     GC_CUDA(cudaMemcpyAsync(&h, ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
@@ -730,12 +844,15 @@ static int run(Context &C, const Problem &pb, int mode, uint64_t seed, const gc_
 }
 
 // Device views of a single graph's CSR (host arrays staged), with GC_FLAG_VALIDATE applied.
+// nnz_known: rowptr[n] if it has been read already, else -1.
 static int single_problem(Context *C, int32_t n, const int32_t *rowptr, const int32_t *colidx, const gc_options *opt,
-                          cudaStream_t s, Problem &pb) {
+                          cudaStream_t s, Problem &pb, int64_t nnz_known = -1) {
     int rp_dev = 0;
     GC_TRY(locate(rowptr, C->device, &rp_dev));
     int32_t nnz32 = 0;
-    if (rp_dev) {
+    if (nnz_known >= 0) {
+        nnz32 = static_cast<int32_t>(nnz_known);
+    } else if (rp_dev) {
         GC_CUDA(cudaMemcpyAsync(&nnz32, rowptr + n, 4, cudaMemcpyDeviceToHost, s));
         GC_CUDA(cudaStreamSynchronize(s));
     } else {
@@ -809,15 +926,32 @@ static int color_single(int32_t n, const int32_t *rowptr, const int32_t *colidx,
     }
     cudaStream_t s = (opt && opt->stream) ? static_cast<cudaStream_t>(opt->stream) : C->stream;
     Problem pb{};
+    const Outputs o{colors_out, ncolors, rounds};
+    int64_t nnz = -1;
+    bool handled = false;
+    const bool small = !colors_in && colidx && small_candidate(n, mode, opt);
+    if (small) {
+        int rp_dev = 0, ci_dev = 0;
+        GC_TRY(locate(rowptr, C->device, &rp_dev));
+        GC_TRY(locate(colidx, C->device, &ci_dev));
+        if (rp_dev && ci_dev) {
+            const int st = color_small(*C, n, rowptr, colidx, seed, opt, stats, o, s, &handled, &nnz);
+            if (handled || st != GC_OK) return st;
+        }
+    }
     UploadGuard upload{C->copy_stream};
-    GC_TRY(single_problem(C, n, rowptr, colidx, opt, s, pb));
+    GC_TRY(single_problem(C, n, rowptr, colidx, opt, s, pb, nnz));
+    if (small && nnz < 0 && pb.nnz > 0) {  // staged host arrays
+        GC_TRY(wait_colidx(pb, s));
+        const int st = color_small(*C, n, pb.rowptr, pb.colidx, seed, opt, stats, o, s, &handled, &nnz);
+        if (handled || st != GC_OK) return st;
+    }
     const void *v = nullptr;
     if (colors_in) {
         GC_TRY(device_view(colors_in, 4 * static_cast<size_t>(n), C->device, C->st_colors_in, s, &v));
         pb.prio_rank = static_cast<const int32_t *>(v);
         pb.priority_override = kPriorityRecolor;
     }
-    Outputs o{colors_out, ncolors, rounds};
     return run(*C, pb, mode, seed, opt, stats, o);
 }
 

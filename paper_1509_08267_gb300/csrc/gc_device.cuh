@@ -231,6 +231,23 @@ __device__ __forceinline__ void det_store(const DetState &S, int64_t V, int32_t 
     S.s16[V] = static_cast<uint16_t>((sat ? kSat7 : static_cast<unsigned>(c)) << 9 | dig << 1 | (final_ ? kFinal : 0u));
 }
 
+// 1 << c for c in 0..31, else 0 (PTX shifts clamp).
+__device__ __forceinline__ uint32_t bit_or_none(uint32_t c) {
+    uint32_t r;
+    asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(1u), "r"(c));
+    return r;
+}
+
+// Least color absent from a window of W words; 32 W when all are there.
+template <int W>
+__device__ __forceinline__ int32_t first_free_words(const uint32_t (&m)[W]) {
+    int32_t c = 32 * W;
+#pragma unroll
+    for (int w = W - 1; w >= 0; --w)
+        if (~m[w]) c = 32 * w + __ffs(static_cast<int>(~m[w])) - 1;
+    return c;
+}
+
 // Adjacency entries are streamed without allocating in L1, leaving L1 to the state words.
 __device__ __forceinline__ int32_t load_entry(const int32_t *p) {
     int32_t v;

@@ -106,6 +106,7 @@ struct RoundParams {
     uint16_t *s16b;  // written in odd rounds (like cx1)
     int32_t *cx0, *cx1;
     uint32_t *prio;
+    const uint8_t *g_done;  // [G] graphs the set-up skips (colored by small_batch_kernel), or nullptr
     int64_t ci_len;  // entries of colidx that may be read (16-byte loads stay inside them)
     int32_t *small0, *small1;  // thread-per-vertex worklists (two parities)
     int4 *chunk0, *chunk1;     // warp work items, kItemBytes each (two parities)
@@ -221,6 +222,35 @@ struct CoreParams {
     int32_t tail_nc;      // blocks of the tail's cluster (tail_max <= kTailOwned * tail_nc)
     unsigned *tail;       // [4]: 1 when the core handed over to the tail, the tail's first round
 };
+
+// Small graphs (gc_small.cu).  A batch's graphs of at most kSmallBatchVertices vertices and
+// kSmallBatchEntries entries are colored by one block each; a single graph of at most
+// kSmallOneVertices vertices whose rows average at most kSmallOneRow entries by one block (up to
+// kSmallBlockVertices vertices and kSmallBlockEntries entries) or one cluster (kSmallOneEntries).
+constexpr int32_t kSmallBatchVertices = 4096;
+constexpr int64_t kSmallBatchEntries = int64_t{1} << 18;
+constexpr int32_t kSmallOneVertices = 16384, kSmallBlockVertices = 2048;
+constexpr int64_t kSmallOneEntries = int64_t{1} << 19, kSmallBlockEntries = int64_t{1} << 15;
+constexpr int64_t kSmallOneRow = 64;
+struct SmallBatch {
+    int32_t *queue;            // [G] the small graphs, largest first
+    unsigned *queued, *taken;  // their number; how many blocks have taken
+    unsigned long long *left;  // vertices of the other graphs
+    uint8_t *g_done;           // [G] 1: small
+};
+struct SmallOne {
+    uint32_t *exchange;   // [2][cap] a cluster's new states
+    unsigned *cnt;        // [3] a cluster's losers per round
+    int32_t *out;         // [n] the colors (written only if nothing is wrong)
+    int32_t *result;      // [9] {0: done, 1: too large, -1: error in [5..8]; entries, last round, colors, largest}
+    int32_t cap;          // vertices the shared arrays hold (a multiple of 4)
+    int64_t max_entries;  // larger graphs are left alone
+};
+// The cluster a single graph runs as (16 or 8 blocks, 0: none).
+int small_one_blocks();
+cudaError_t launch_small_one(const RoundParams &P, const SmallOne &A, int blocks, cudaStream_t s);
+// After launch_batch_tables: picks the small graphs and colors them (nnz: the batch's entries).
+cudaError_t launch_small_batch(const RoundParams &P, const SmallBatch &B, int64_t nnz, cudaStream_t s);
 
 // Launch wrappers (gc_kernels.cu).  All return the launch's cudaError_t.
 // gc_color_batch: graph table from the offset tables, graph id per vertex, graph_last = 1 (0 if empty).

@@ -314,13 +314,6 @@ __device__ __forceinline__ void load_oct(const int32_t *p, int align, bool insid
     }
 }
 
-// 1 << c for c in 0..31, else 0 (PTX shifts clamp).
-__device__ __forceinline__ uint32_t bit_or_none(uint32_t c) {
-    uint32_t r;
-    asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(1u), "r"(c));
-    return r;
-}
-
 // Reports the malformed entries among the first `cnt` of a row.
 __device__ __noinline__ void det_small_check(const RoundParams &P, const Row &r, int32_t cnt) {
     for (int64_t j = r.b; j < r.b + cnt; ++j) neighbour(P, r, load_entry(P.colidx + j), j);
@@ -427,16 +420,6 @@ __device__ __forceinline__ int det_small_row(const RoundParams &P, const DetStat
     if (none != 0) det_small_check(P, r, deg);
     if ((W == 4 && cv == kSat7) || least >> 1 == dig) return 2;
     return least < 2u * dig ? 1 : 0;
-}
-
-// Least color absent from a window of W words; 32 W when all are there.
-template <int W>
-__device__ __forceinline__ int32_t first_free_words(const uint32_t (&m)[W]) {
-    int32_t c = 32 * W;
-#pragma unroll
-    for (int w = W - 1; w >= 0; --w)
-        if (~m[w]) c = 32 * w + __ffs(static_cast<int>(~m[w])) - 1;
-    return c;
 }
 
 // One vertex of degree <= T1 per lane (lanes with `in`): did it lose in this round; writes its next
@@ -1575,15 +1558,19 @@ __global__ void __launch_bounds__(256) setup_kernel(RoundParams P, int32_t v_beg
         int kind = 0;  // 1 = one thread, 2 = work items
         int32_t nch = 0;
         int64_t d = 0;
-        if (in) {
-            int32_t g = 0;
-            if constexpr (BATCH) {
+        int32_t g = 0;
+        bool mine = in;
+        if constexpr (BATCH) {
+            if (in) {
                 g = g_fixed;
                 if (g >= 0)
                     P.vg[V] = g;
                 else
                     g = P.vg[V];
+                mine = !P.g_done || P.g_done[g] == 0;
             }
+        }
+        if (mine) {
             int64_t b;
             int32_t lv;
             d = checked_degree<BATCH>(P, V, g, b, lv);
@@ -1708,7 +1695,7 @@ __global__ void scatter_small_kernel(RoundParams P, int32_t v_begin, int32_t v_e
             const int32_t g = BATCH ? P.vg[V] : 0;
             int64_t b;
             int32_t lv;
-            d = checked_degree<BATCH>(P, V, g, b, lv);
+            if (!BATCH || !P.g_done || P.g_done[g] == 0) d = checked_degree<BATCH>(P, V, g, b, lv);
         }
         const bool small = d > 0 && d <= P.T1;
         unsigned rank = 0;
