@@ -92,6 +92,7 @@ struct Ctl {
     unsigned tail_ctl[4];  // tail phase: handed over, first round
     unsigned small_ctl[4];  // small graphs: a batch's queued and taken graphs; a cluster's losers per round
     unsigned long long small_left;  // vertices of the graphs that are not small
+    alignas(128) unsigned ord_cnt[3 * kOrdSet];  // ordered mode and peeling
     GridBar bar;
 };
 static_assert(offsetof(Ctl, bar) % 128 == 0, "barrier alignment");
@@ -292,17 +293,15 @@ static int peel_levels(Context &C, Ctl *ctl, RoundParams P, int32_t T1, int32_t 
     GC_TRY(ensure(C.col0, 8 * n, "vertex state"));
     GC_TRY(ensure(C.col1, 8 * n, "vertex state"));
     GC_TRY(ensure(C.items, 4 * n, "worklist"));
-    GC_TRY(ensure(C.small0, 4 * n, "worklist"));
-    GC_TRY(ensure(C.small1, 4 * n, "worklist"));
-    GC_TRY(ensure(C.mid0, 4 * n, "worklist"));
-    GC_TRY(ensure(C.mid1, 4 * n, "worklist"));
+    GC_TRY(ensure(C.mid0, 32 * n, "worklist"));
+    GC_TRY(ensure(C.mid1, 32 * n, "worklist"));
     P.T1 = T1 < kOrdSmall ? T1 : kOrdSmall;
     P.CH = CH < kOrdChunk ? CH : kOrdChunk;
     P.pass_begin = 1;
-    int32_t *res = reinterpret_cast<int32_t *>(C.col1.p);
+    unsigned long long *W = C.col1.as<unsigned long long>();
     int32_t *level = C.rank.as<int32_t>();
     GC_CUDA(cudaMemsetAsync(ctl->peel, 0, sizeof(ctl->peel), s));
-    GC_CUDA(launch_peel_init(P, res, level, ctl->peel, ctl->peel + 2, s));
+    GC_CUDA(launch_peel_init(P, W, level, ctl->peel, ctl->peel + 2, s));
     Ctl h{};
     GC_CUDA(cudaMemcpyAsync(&h, ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
     GC_CUDA(cudaStreamSynchronize(s));
@@ -310,19 +309,20 @@ static int peel_levels(Context &C, Ctl *ctl, RoundParams P, int32_t T1, int32_t 
     const size_t n_items = h.peel[2];
     GC_TRY(ensure(C.chunk0, 16 * std::max<size_t>(n_items, 1), "work items"));
     GC_TRY(ensure(C.chunk1, 16 * std::max<size_t>(n_items, 1), "work items"));
-    P.small0 = C.small0.as<int32_t>();
-    P.small1 = C.small1.as<int32_t>();
-    P.mid0 = C.mid0.as<int32_t>();
-    P.mid1 = C.mid1.as<int32_t>();
+    P.ord0 = C.mid0.as<int4>();
+    P.ord1 = C.mid1.as<int4>();
+    P.ord_items = static_cast<unsigned>(n_items);
+    P.ord_cnt = ctl->ord_cnt;
     P.chunk0 = C.chunk0.as<int4>();
     P.chunk1 = C.chunk1.as<int4>();
-    GC_CUDA(cudaMemsetAsync(ctl->cnt, 0, sizeof(ctl->cnt), s));
+    GC_CUDA(cudaMemsetAsync(ctl->ord_cnt, 0, sizeof(ctl->ord_cnt), s));
     int &occ = C.occ_peel;
     if (occ == 0) GC_CUDA(peel_kernel_occupancy(256, &occ));
-    const int grid = (blocks_per_sm > 0 && blocks_per_sm < occ ? blocks_per_sm : occ) * C.sms;
+    // two blocks per SM: levels are as latency-bound as the ordered mode's rounds (three: 2% slower)
+    const int grid = (blocks_per_sm > 0 && blocks_per_sm < occ ? blocks_per_sm : std::min(occ, 2)) * C.sms;
     // the lists of vertices left by each threshold search: two scratch arrays that every mode
     // rewrites afterwards
-    GC_CUDA(launch_peel(P, res, level, ctl->peel, C.items.as<int32_t>(), C.col0.as<int32_t>(), ctl->peel + 2, grid,
+    GC_CUDA(launch_peel(P, W, level, ctl->peel, C.items.as<int32_t>(), C.col0.as<int32_t>(), ctl->peel + 2, grid,
                         256, s));
     GC_CUDA(cudaMemcpyAsync(&h, ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
     GC_CUDA(cudaStreamSynchronize(s));
@@ -601,9 +601,9 @@ static int run(Context &C, const Problem &pb, int mode, uint64_t seed, const gc_
         // vertices only
         P.deg_hist = nullptr;
         P.T1 = T1 < kOrdSmall ? T1 : kOrdSmall;
-        // a single graph's rounds are a chain of short latency-bound steps: 64-entry work items and
-        // one block per SM by default (R-MAT-22: 33.8 ms against 39.7 with 128 entries and three
-        // blocks; the grid barrier is cheaper with fewer blocks)
+        // a single graph's rounds are a chain of short latency-bound steps: 64-entry work items (32 and
+        // 128: 0-32% slower on long chains or heavy rounds) and two blocks per SM (one: 1.5% faster where
+        // a round holds a hundred vertices, 24% slower where it holds thousands)
         const int32_t ch_ord = (opt && opt->chunk) || pb.batch ? CH : kOrdSingleChunk;
         P.CH = ch_ord < kOrdChunk ? ch_ord : kOrdChunk;
         GC_CUDA(launch_setup(P, GC_MODE_INPLACE, pb.batch, 0, static_cast<int32_t>(n), -1, s));
@@ -617,23 +617,25 @@ static int run(Context &C, const Problem &pb, int mode, uint64_t seed, const gc_
         GC_TRY(ensure(C.chunk0, 16 * std::max<size_t>(n_items, 1), "work items"));
         GC_TRY(ensure(C.chunk1, 16 * std::max<size_t>(n_items, 1), "work items"));
         GC_TRY(ensure(C.acc, 4 * kOrdSlotWords * std::max<size_t>(slots, 1), "accumulators"));
-        GC_TRY(ensure(C.mid0, 4 * static_cast<size_t>(n), "worklist"));
-        GC_TRY(ensure(C.mid1, 4 * static_cast<size_t>(n), "worklist"));
+        GC_TRY(ensure(C.mid0, 32 * static_cast<size_t>(n), "worklist"));
+        GC_TRY(ensure(C.mid1, 32 * static_cast<size_t>(n), "worklist"));
         P.chunk0 = C.chunk0.as<int4>();
         P.chunk1 = C.chunk1.as<int4>();
-        P.mid0 = C.mid0.as<int32_t>();
-        P.mid1 = C.mid1.as<int32_t>();
+        P.ord0 = C.mid0.as<int4>();
+        P.ord1 = C.mid1.as<int4>();
+        P.ord_items = static_cast<unsigned>(n_items);
+        P.ord_cnt = ctl->ord_cnt;
         P.acc = C.acc.as<unsigned>();
         if (slots) GC_CUDA(cudaMemsetAsync(C.acc.p, 0, 4 * kOrdSlotWords * slots, s));
-        GC_CUDA(cudaMemsetAsync(ctl->cnt, 0, sizeof(ctl->cnt), s));
+        GC_CUDA(cudaMemsetAsync(ctl->ord_cnt, 0, sizeof(ctl->ord_cnt), s));
         if (timing) GC_CUDA(cudaEventRecord(C.ev[1], s));
         int &occ = C.occ_ord[pb.batch ? 1 : 0];
         if (occ == 0) GC_CUDA(ordered_kernel_occupancy(pb.batch, block, &occ));
-        int per_sm = pb.batch ? occ : 1;
+        int per_sm = pb.batch ? occ : std::min(occ, 2);
         if (opt && opt->blocks_per_sm > 0) per_sm = opt->blocks_per_sm < occ ? opt->blocks_per_sm : occ;
         grid = static_cast<int64_t>(per_sm) * C.sms;
         GC_TRY(wait_colidx(pb, s));
-        GC_CUDA(launch_ordered(P, pb.batch, reinterpret_cast<int32_t *>(C.col1.p), static_cast<int>(grid), block, s));
+        GC_CUDA(launch_ordered(P, pb.batch, C.col1.as<unsigned long long>(), static_cast<int>(grid), block, s));
     } else if (rest) {
     GC_CUDA(launch_setup(P, mode, pb.batch, 0, static_cast<int32_t>(n), -1, s));
     GC_CUDA(launch_sort_small(P, pb.batch, 0, static_cast<int32_t>(n), s));

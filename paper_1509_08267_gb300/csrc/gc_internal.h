@@ -53,6 +53,7 @@ constexpr int32_t kPriorityRecolor = 3;
 constexpr int kOrdChunk = 128;
 constexpr int kOrdSingleChunk = 64;  // default work-item size of the ordered mode on a single graph
 constexpr int kOrdSlotWords = 32;
+constexpr int kOrdPad = 32, kOrdSet = 4 * kOrdPad;  // words from one counter, or counter set, to the next
 
 // Worklist counters: three sets used round-robin (read / append / clear), kCnt words each.
 constexpr int kCnt = 4;
@@ -110,7 +111,10 @@ struct RoundParams {
     int64_t ci_len;  // entries of colidx that may be read (16-byte loads stay inside them)
     int32_t *small0, *small1;  // thread-per-vertex worklists (two parities)
     int4 *chunk0, *chunk1;     // warp work items, kItemBytes each (two parities)
-    int32_t *mid0, *mid1;      // ordered mode: medium-degree ready vertices (two parities)
+    int4 *ord0, *ord1;         // ordered mode: small, then medium-degree ready vertices, n each (two parities)
+    unsigned ord_items;        // ordered mode: entries chunk0 / chunk1 hold
+    unsigned *ord_cnt;         // [3][kOrdSet] its counter sets, a counter per 128 bytes: every releasing warp adds
+                               // to them, and atomics on one line queue
     int32_t *items;            // setup scratch: larger vertices found by the binning pass
     unsigned *tmp;             // [2] setup scratch counters: larger vertices, their work items
     unsigned *cnt;             // [3][kCnt] worklist counters
@@ -293,21 +297,21 @@ cudaError_t launch_count_colors(const RoundParams &P, bool batch, const int32_t 
                                 int32_t *gcount, int32_t *out, cudaStream_t s);
 // Ordered mode (GC_MODE_ORDERED): after the in-place launch_setup (every vertex with neighbours
 // uncolored) with P.T1 <= kOrdSmall and P.CH <= kOrdChunk, with the counter sets and P.acc's slots
-// zeroed, counts each vertex's smaller-key neighbours into pend[n], lists the first ready vertices
-// (small ones in small0, medium ones in mid0, work items {V, q, slot, nch} in chunk0; P.mid0/mid1
-// hold n entries each) and runs the cooperative round kernel on `grid` blocks.
+// zeroed, counts each vertex's smaller-key neighbours into its word W[n], lists the first ready
+// vertices (P.ord0 / ord1 hold 2 n entries each, chunk0 / chunk1 P.ord_items work items) and runs the
+// cooperative round kernel on `grid` blocks.
 cudaError_t ordered_kernel_occupancy(bool batch, int block, int *blocks_per_sm);
-// Smallest-last levels (single graph): launch_peel_init sets res[v] = deg(v), level[v] = 0, the two
+// Smallest-last levels (single graph): launch_peel_init sets the words W to deg(v), level[v] = 0, the two
 // threshold words kw[2] and adds the work items the lists may need (vertices past kOrdMid, P.CH
 // entries each) to *items; launch_peel (counter sets zeroed, P.T1 <= kOrdSmall, P.CH <= kOrdChunk,
 // lists as the ordered mode's; rlist0 / rlist1 int32[n] scratch with two counters rcnt) writes
 // level[v] >= 1, the number of levels to passes[0] and the degeneracy to passes[1].
-cudaError_t launch_peel_init(const RoundParams &P, int32_t *res, int32_t *level, unsigned *kw, unsigned *items,
+cudaError_t launch_peel_init(const RoundParams &P, unsigned long long *W, int32_t *level, unsigned *kw, unsigned *items,
                              cudaStream_t s);
 cudaError_t peel_kernel_occupancy(int block, int *blocks_per_sm);
-cudaError_t launch_peel(const RoundParams &P, int32_t *res, int32_t *level, unsigned *kw, int32_t *rlist0,
+cudaError_t launch_peel(const RoundParams &P, unsigned long long *W, int32_t *level, unsigned *kw, int32_t *rlist0,
                         int32_t *rlist1, unsigned *rcnt, int grid, int block, cudaStream_t s);
-cudaError_t launch_ordered(const RoundParams &P, bool batch, int32_t *pend, int grid, int block, cudaStream_t s);
+cudaError_t launch_ordered(const RoundParams &P, bool batch, unsigned long long *W, int grid, int block, cudaStream_t s);
 // Partition mode (GC_MODE_PARTITION, single graph): set-up (rows checked, colors -1, W_1 = V) and
 // the cooperative round kernel with p blocks of consecutive ids.
 cudaError_t launch_partition_init(const RoundParams &P, cudaStream_t s);

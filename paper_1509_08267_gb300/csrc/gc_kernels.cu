@@ -1969,7 +1969,10 @@ __global__ void __launch_bounds__(kBlock, kNarrowBlocks) part_round_kernel(Round
 }
 
 // ------------------------------------------------------------------------------------------
-// ordered mode: First Fit in key order without speculation.  pend[v] counts v's neighbours with a
+// ordered mode: First Fit in key order without speculation.  A vertex's word in W holds its degree (top
+// bit set: uncolored) or its color in the high half, and kOrdBias plus a count in the low half: one
+// atomic decrement also tells the degree, which says how the vertex will be listed.  The count is the
+// number of v's neighbours with a
 // smaller key that are still uncolored; a vertex whose count is 0 is ready: it takes First Fit over
 // its colored neighbours (exactly those with a smaller key) and, in the same sweep, counts itself
 // down at each uncolored neighbour (each has a larger key and waits for it).  A neighbour whose count
@@ -1984,22 +1987,63 @@ __global__ void __launch_bounds__(kBlock, kNarrowBlocks) part_round_kernel(Round
 // the whole run (its count reaches 0 once), so the small and medium lists never hold more than n
 // vertices and the item lists no more than the sum over larger v of ceil(deg(v) / P.CH) items.
 
+//
+// What bounds it: the chain of a round -- list counters, list entry, adjacency entries, neighbours'
+// words, decrements, list reservation, merge, grid barrier -- at six to seven microseconds for a hundred
+// ready vertices, of which the barrier is about two; R-MAT graphs have hundreds to thousands of rounds.
+// The list entries name the row, the decrement's result the degree, each list counter has a line of its
+// own, an item's window is merged while its decrements and listings are under way, and items are dealt
+// one per SM first: 8.0 -> 6.5 us a round (R-MAT n = 500,000, smallest-last key: 9.6 -> 8.0 ms; peeling
+// 5.5 -> 4.2).  A block of 512 threads per large vertex instead of items was slower (12.0 ms): one SM
+// takes a gather and an atomic a cycle.
+
 constexpr int kOrdPer = kOrdChunk / 32;  // entries per lane per step of a work item
 constexpr int kOrdMidLanes = 8;          // lanes per medium vertex
 constexpr int kOrdMidPer = kOrdMid / kOrdMidLanes;  // entries per lane of a medium vertex
 
-// The lists a round fills for the next one.
+// (A count only falls, by at most one per adjacency entry: the bias keeps it from borrowing from the
+// high half even if the input is not symmetric.)
+constexpr uint64_t kOrdBias = 0x80000000ull;
+constexpr uint64_t kOrdOpen = 1ull << 63;
+__device__ __forceinline__ uint64_t ord_word(int64_t deg, unsigned count) {
+    return kOrdOpen | static_cast<uint64_t>(deg) << 32 | (kOrdBias + count);
+}
+__device__ __forceinline__ bool ord_open(uint64_t w) { return (w & kOrdOpen) != 0; }
+__device__ __forceinline__ int32_t ord_degree(uint64_t w) { return static_cast<int32_t>(w >> 32 & 0x7fffffffu); }
+__device__ __forceinline__ int32_t ord_color(uint64_t w) { return ord_open(w) ? -1 : static_cast<int32_t>(w >> 32); }
+
+// The lists a round fills for the next one.  Entries name the row (single graphs; a batch looks it up),
+// so that a round starts with its entries' loads.
 struct OrdLists {
-    int32_t *small;  // vertices of degree <= P.T1           (count cnt[kCntSmall])
-    int32_t *mid;    // vertices of degree <= kOrdMid         (count cnt[kCntMulti])
-    int4 *items;     // work items {V, q, slot, nch}          (count cnt[kCntChunks]; slots cnt[kCntItems])
-    unsigned *cnt;   // the round's counter set
+    int4 *small;    // {V, first entry, degree}: degree <= P.T1    (count cnt[kCntSmall])
+    int4 *mid;      // the same: degree <= kOrdMid                  (count cnt[kCntMulti])
+    int4 *items;    // work items {V, first entry, entries | kOrdFirst, slot}, a batch's first entry counted
+                    // from the row's start                        (count cnt[kCntChunks]; slots cnt[kCntItems])
+    unsigned *cnt;  // the round's counter set
 };
+constexpr int32_t kOrdFirst = 1 << 30;  // a vertex's first item
 
 __device__ __forceinline__ OrdLists ord_lists(const RoundParams &P, int pass) {
     const bool odd = (pass & 1) != 0;
-    return OrdLists{odd ? P.small0 : P.small1, odd ? P.mid0 : P.mid1, odd ? P.chunk0 : P.chunk1,
-                    P.cnt + kCnt * (pass % 3)};
+    int4 *base = odd ? P.ord0 : P.ord1;
+    return OrdLists{base, base + P.n, odd ? P.chunk0 : P.chunk1, P.ord_cnt + kOrdSet * (pass % 3)};
+}
+
+// Row of a small or medium list entry.
+template <bool BATCH>
+__device__ __forceinline__ Row ord_row(const RoundParams &P, int4 x) {
+    if constexpr (BATCH) {
+        return load_row<true>(P, x.x);
+    } else {
+        Row r;
+        r.b = x.y;
+        r.e = x.y + x.z;
+        r.vbase = 0;
+        r.ng = P.n;
+        r.lv = x.x;
+        r.g = 0;
+        return r;
+    }
 }
 
 // Warp-wide exclusive prefix sum of x; `total` receives the sum over all lanes.
@@ -2014,61 +2058,71 @@ __device__ __forceinline__ unsigned warp_exclusive_sum(unsigned x, int lane, uns
     return incl - x;
 }
 
-// Lists the ready vertices U[k] (those with ready[k]; up to K per lane) in L, with one atomic per
-// list and warp: by degree on the small or the medium list, or as ceil(deg / P.CH) work items with
-// an accumulator slot when there are several (warp-uniform call).
+// Lists the ready vertices U[k] (those with ready[k]; up to K per lane; degree deg[k]) in L, with one
+// atomic per list and warp: by degree on the small or the medium list, or as ceil(deg / P.CH) work
+// items with an accumulator slot when there are several (warp-uniform call).  The rows' offsets are
+// loaded while the reservations are under way.
 template <bool BATCH, int K>
-__device__ void ord_list(const RoundParams &P, const bool (&ready)[K], const int32_t (&U)[K], const OrdLists &L,
-                         int lane) {
-    bool any = false;
+__device__ void ord_list(const RoundParams &P, const bool (&ready)[K], const int32_t (&U)[K], const int32_t (&deg)[K],
+                         const OrdLists &L, int lane) {
+    unsigned any = 0;  // bit k: this lane's k-th is ready
 #pragma unroll
-    for (int k = 0; k < K; ++k) any |= ready[k];
-    if (!__any_sync(kFull, any)) return;
-    unsigned nch[K];  // work items of a larger vertex; 0 for a small or medium one or none
-    uint8_t kind[K];  // 0 none, 1 small, 2 medium, 3 items
-    unsigned ns = 0, nd = 0, ni = 0, nm = 0;
+    for (int k = 0; k < K; ++k) any |= static_cast<unsigned>(ready[k]) << k;
+    const unsigned all = __reduce_or_sync(kFull, any);
+    if (all == 0u) return;
+    int32_t rb[K];     // the row's first entry (single graphs)
+    unsigned kind[K];  // 0 small, 1 medium, 2 items, 3 none
+    unsigned total = 0;            // lane c: entries for list c (0 small, 1 medium, 2 items), lane 3: slots
+    unsigned ni = 0, nm = 0;       // this lane's work items and slots
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-        nch[k] = 0;
-        kind[k] = 0;
+        kind[k] = 3;
+        rb[k] = 0;
+        if (!((all >> k) & 1u)) continue;
         if (ready[k]) {
-            const Row r = load_row<BATCH>(P, U[k]);
-            const int64_t deg = r.e - r.b;
-            kind[k] = deg <= P.T1 ? 1 : deg <= kOrdMid ? 2 : 3;
-            if (kind[k] == 3) nch[k] = static_cast<unsigned>((deg + P.CH - 1) / P.CH);
+            if (!BATCH) rb[k] = __ldg(P.rowptr + U[k]);
+            kind[k] = deg[k] <= P.T1 ? 0u : deg[k] <= kOrdMid ? 1u : 2u;
         }
-        ns += kind[k] == 1 ? 1u : 0u;
-        nd += kind[k] == 2 ? 1u : 0u;
-        ni += nch[k];
-        nm += nch[k] > 1u ? 1u : 0u;
+        const unsigned m0 = __ballot_sync(kFull, kind[k] == 0u), m1 = __ballot_sync(kFull, kind[k] == 1u);
+        if (lane < 2) total += static_cast<unsigned>(__popc(lane == 0 ? m0 : m1));
+        if (kind[k] == 2u) {
+            const unsigned nch = static_cast<unsigned>((deg[k] + P.CH - 1) / P.CH);
+            ni += nch;
+            nm += nch > 1u ? 1u : 0u;
+        }
     }
-    unsigned ts, td, ti, tm;
-    unsigned sb = warp_exclusive_sum(ns, lane, ts);
-    unsigned db = warp_exclusive_sum(nd, lane, td);
-    unsigned ib = warp_exclusive_sum(ni, lane, ti);
-    unsigned mb = warp_exclusive_sum(nm, lane, tm);
-    unsigned b0 = 0, b1 = 0, b2 = 0, b3 = 0;
-    if (lane == 0) {
-        if (ts) b0 = atomicAdd(L.cnt + kCntSmall, ts);
-        if (td) b1 = atomicAdd(L.cnt + kCntMulti, td);
-        if (ti) b2 = atomicAdd(L.cnt + kCntChunks, ti);
-        if (tm) b3 = atomicAdd(L.cnt + kCntItems, tm);
+    unsigned ib = 0, mb = 0;
+    if (__any_sync(kFull, ni != 0u)) {
+        unsigned ti, tm;
+        ib = warp_exclusive_sum(ni, lane, ti);
+        mb = warp_exclusive_sum(nm, lane, tm);
+        if (lane == 2) total = ti;
+        if (lane == 3) total = tm;
     }
-    sb += __shfl_sync(kFull, b0, 0);
-    db += __shfl_sync(kFull, b1, 0);
-    ib += __shfl_sync(kFull, b2, 0);
-    mb += __shfl_sync(kFull, b3, 0);
+    // lanes 0..3 reserve in the lists
+    const int counter = lane == 0 ? kCntSmall : lane == 1 ? kCntMulti : lane == 2 ? kCntChunks : kCntItems;
+    unsigned run = 0;
+    if (lane < 4 && total) run = atomicAdd(L.cnt + kOrdPad * counter, total);
+    ib += __shfl_sync(kFull, run, 2);
+    mb += __shfl_sync(kFull, run, 3);
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-        if (kind[k] == 1) {
-            L.small[sb++] = U[k];
-        } else if (kind[k] == 2) {
-            L.mid[db++] = U[k];
-        } else if (kind[k] == 3) {
-            const int32_t slot = nch[k] > 1u ? static_cast<int32_t>(mb++) : -1;
-            for (unsigned q = 0; q < nch[k]; ++q)
-                L.items[ib + q] = make_int4(U[k], static_cast<int32_t>(q), slot, static_cast<int32_t>(nch[k]));
-            ib += nch[k];
+        if (!((all >> k) & 1u)) continue;
+        const unsigned b = __shfl_sync(kFull, run, static_cast<int>(kind[k] & 1u));
+        const unsigned m0 = __ballot_sync(kFull, kind[k] == 0u), m1 = __ballot_sync(kFull, kind[k] == 1u);
+        if (lane < 2) run += static_cast<unsigned>(__popc(lane == 0 ? m0 : m1));
+        if (kind[k] == 0u) {
+            L.small[b + __popc(m0 & lanemask_lt())] = make_int4(U[k], rb[k], deg[k], 0);
+        } else if (kind[k] == 1u) {
+            L.mid[b + __popc(m1 & lanemask_lt())] = make_int4(U[k], rb[k], deg[k], 0);
+        } else if (kind[k] == 2u) {
+            const unsigned nch = static_cast<unsigned>((deg[k] + P.CH - 1) / P.CH);
+            const int32_t slot = nch > 1u ? static_cast<int32_t>(mb++) : -1;
+            for (unsigned q = 0; q < nch; ++q) {
+                const int32_t at = static_cast<int32_t>(q) * P.CH;
+                L.items[ib + q] = make_int4(U[k], rb[k] + at, min(P.CH, deg[k] - at) | (q == 0 ? kOrdFirst : 0), slot);
+            }
+            ib += nch;
         }
     }
 }
@@ -2076,44 +2130,83 @@ __device__ void ord_list(const RoundParams &P, const bool (&ready)[K], const int
 // Counts down the neighbours U[k] (those with take[k]): the ones whose count was `fire` before the
 // decrement are listed (warp-uniform call).  Ordered mode: pend, fire 1 (the last smaller-key
 // neighbour was colored).  Peeling: the residual degrees, fire k + 1 (the degree reached k).
-template <bool BATCH, int K>
-__device__ __forceinline__ void ord_release(const RoundParams &P, int32_t *pend, const bool (&take)[K],
-                                            const int32_t (&U)[K], const OrdLists &L, int lane,
-                                            int32_t fire = 1) {
-    bool ready[K];
+template <int K>
+__device__ __forceinline__ void ord_count_down(unsigned long long *W, const bool (&take)[K], const int32_t (&U)[K],
+                                               unsigned fire, bool (&ready)[K], int32_t (&deg)[K]) {
+    unsigned long long old[K];
 #pragma unroll
-    for (int k = 0; k < K; ++k) ready[k] = take[k] && atomicSub(pend + U[k], 1) == fire;
-    ord_list<BATCH, K>(P, ready, U, L, lane);
-}
-
-// Does neighbour u (local id lu, state word read on demand) have a smaller key than v?  With the
-// hash key both keys are recomputed from the ids (the same order as key_less: the 31 priority bits
-// are the top of the hash), so no state word is read; the other keys compare the state words.
-template <bool HASH>
-__device__ __forceinline__ bool smaller_key(const RoundParams &P, const unsigned long long *st, int32_t U,
-                                            uint32_t lu, uint32_t lv, uint64_t hv, uint32_t pv) {
-    if constexpr (HASH) {
-        const uint64_t hu = vertex_hash(P.seed, lu);
-        return hu != hv ? hu < hv : lu < lv;
-    } else {
-        return key_less(prio_of(__ldcg(st + U)), pv, lu, lv, P.seed);
+    for (int k = 0; k < K; ++k) old[k] = take[k] ? atomicAdd(W + U[k], ~0ull) : 0ull;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        ready[k] = take[k] && static_cast<uint32_t>(old[k]) == static_cast<uint32_t>(kOrdBias) + fire;
+        deg[k] = ord_degree(old[k]);
     }
 }
 
-// pend[v] for every vertex, and the first round's lists (vertices with neighbours, none of them
-// with a smaller key).  A warp takes 32 consecutive vertices, one per lane: a lane counts a row of
-// up to 32 entries itself (four entries at a time), and the warp counts the longer rows one after
-// another with all lanes; the ready vertices are listed together.  Vertices without neighbours
-// were colored by setup.
+template <bool BATCH, int K>
+__device__ __forceinline__ void ord_release(const RoundParams &P, unsigned long long *W, const bool (&take)[K],
+                                            const int32_t (&U)[K], const OrdLists &L, int lane,
+                                            unsigned fire = 1) {
+    bool ready[K];
+    int32_t deg[K];
+    ord_count_down<K>(W, take, U, fire, ready, deg);
+    ord_list<BATCH, K>(P, ready, U, deg, L, lane);
+}
+
+// The words W of every vertex, and the first round's lists (vertices with neighbours, none of them with
+// a smaller key).  A warp takes 32 consecutive vertices, one per lane: a lane counts a row of up to 32
+// entries itself (four entries at a time), the warp counts longer rows one after another with all
+// lanes, 256 entries in flight, and the rows past kCountWarp wait for the whole block (a hub's row of
+// 65,000 entries on one warp, 32 at a time, took 1.4 ms; R-MAT n = 2^20: 1.49 -> 0.27 ms).  Vertices
+// without neighbours were colored by setup.
+constexpr int kCountWarp = 4096;  // longest row one warp counts
+constexpr int kCountBig = 128;    // rows a block keeps for later at a time
+
+// Smaller-key neighbours among every `step`-th entry of row r from `from`, eight in flight.
+template <bool HASH>
+__device__ __forceinline__ unsigned ord_count_row(const RoundParams &P, const unsigned long long *st, const Row &r,
+                                                  int from, int step, uint64_t hv, uint32_t pv) {
+    unsigned c = 0;
+    for (int64_t j = r.b + from; j < r.e; j += 8 * step) {
+        int32_t u[8];
+        uint32_t p[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) u[t] = j + t * step < r.e ? load_entry(P.colidx + j + t * step) : 0;
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            const bool in = j + t * step < r.e;
+            const int32_t U = in ? neighbour(P, r, u[t], j + t * step) : -1;
+            if constexpr (HASH) {
+                const uint64_t hu = vertex_hash(P.seed, static_cast<uint32_t>(u[t]));
+                c += U >= 0 && (hu != hv ? hu < hv : u[t] < r.lv) ? 1u : 0u;
+                p[t] = 0;
+            } else {
+                p[t] = U >= 0 ? prio_of(load_state(reinterpret_cast<const uint64_t *>(st) + U)) : ~0u;
+            }
+        }
+        if constexpr (!HASH) {
+#pragma unroll
+            for (int t = 0; t < 8; ++t)
+                if (p[t] != ~0u)
+                    c += key_less(p[t], pv, static_cast<uint32_t>(u[t]), static_cast<uint32_t>(r.lv), P.seed) ? 1u : 0u;
+        }
+    }
+    return c;
+}
+
 template <bool BATCH, bool HASH>
-__global__ void ord_count_kernel(RoundParams P, int32_t *pend) {
+__global__ void __launch_bounds__(256) ord_count_kernel(RoundParams P, unsigned long long *W) {
     constexpr int64_t kLaneRow = 32;  // longest row one lane counts alone
+    __shared__ int32_t s_big[kCountBig];
+    __shared__ unsigned s_nbig, s_sum;
     const int lane = threadIdx.x & 31;
-    const int64_t nw = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5);
+    const int64_t nb = static_cast<int64_t>(gridDim.x) * blockDim.x;
     const OrdLists L = ord_lists(P, P.pass_begin);
     const unsigned long long *st = reinterpret_cast<const unsigned long long *>(P.col0);
-    for (int64_t base = (static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32;
-         base < P.n; base += nw * 32) {
+    if (threadIdx.x == 0) s_nbig = 0u;
+    __syncthreads();
+    for (int64_t block0 = static_cast<int64_t>(blockIdx.x) * blockDim.x; block0 < P.n; block0 += nb) {
+        const int64_t base = block0 + threadIdx.x - lane;
         const int32_t V = static_cast<int32_t>(base + lane);
         const bool valid = base + lane < P.n;
         Row r{};
@@ -2129,61 +2222,81 @@ __global__ void ord_count_kernel(RoundParams P, int32_t *pend) {
                 pv = prio_of(__ldcg(st + V));
         }
         unsigned c = 0;
-        if (deg > 0 && deg <= kLaneRow) {
-            for (int64_t j = r.b; j < r.e; j += 4) {
-                int32_t u[4];
-#pragma unroll
-                for (int t = 0; t < 4; ++t) u[t] = j + t < r.e ? load_entry(P.colidx + j + t) : 0;
-#pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    if (j + t >= r.e) continue;
-                    const int32_t U = neighbour(P, r, u[t], j + t);
-                    if (U >= 0 && smaller_key<HASH>(P, st, U, static_cast<uint32_t>(u[t]),
-                                                    static_cast<uint32_t>(r.lv), hv, pv))
-                        ++c;
-                }
-            }
-        }
+        bool later = false;  // counted by the block
+        if (deg > 0 && deg <= kLaneRow) c = ord_count_row<HASH>(P, st, r, 0, 1, hv, pv);
         unsigned big = __ballot_sync(kFull, deg > kLaneRow);
         while (big) {
             const int l = __ffs(big) - 1;
             big &= big - 1;
             const int32_t Vb = __shfl_sync(kFull, V, l);
             const Row rb = load_row<BATCH>(P, Vb);
-            const uint64_t hb = __shfl_sync(kFull, hv, l);
-            const uint32_t pb = __shfl_sync(kFull, pv, l);
-            unsigned cb = 0;
-            for (int64_t j = rb.b + lane; j < rb.e; j += 32) {
-                const int32_t ul = load_entry(P.colidx + j);
-                const int32_t U = neighbour(P, rb, ul, j);
-                if (U >= 0 &&
-                    smaller_key<HASH>(P, st, U, static_cast<uint32_t>(ul), static_cast<uint32_t>(rb.lv), hb, pb))
-                    ++cb;
+            if (rb.e - rb.b > kCountWarp) {
+                unsigned at = 0;
+                if (lane == 0) at = atomicAdd(&s_nbig, 1u);
+                at = __shfl_sync(kFull, at, 0);
+                if (at < kCountBig) {
+                    if (lane == 0) s_big[at] = Vb;
+                    if (lane == l) later = true;
+                    continue;
+                }
             }
+            unsigned cb = ord_count_row<HASH>(P, st, rb, lane, 32, __shfl_sync(kFull, hv, l),
+                                              __shfl_sync(kFull, pv, l));
             cb = __reduce_add_sync(kFull, cb);
             if (lane == l) c = cb;
         }
-        if (valid) pend[V] = static_cast<int32_t>(c);
-        const bool ready[1] = {valid && deg > 0 && c == 0};
-        const int32_t Vs[1] = {V};
-        ord_list<BATCH, 1>(P, ready, Vs, L, lane);
+        if (valid && !later) W[V] = ord_word(deg, c);
+        const bool ready[1] = {valid && deg > 0 && c == 0 && !later};
+        const int32_t Vs[1] = {V}, ds[1] = {static_cast<int32_t>(deg)};
+        ord_list<BATCH, 1>(P, ready, Vs, ds, L, lane);
     }
+    // the long rows, a block each
+    __syncthreads();
+    const unsigned nbig = min(s_nbig, static_cast<unsigned>(kCountBig));
+    for (unsigned i = 0; i < nbig; ++i) {
+        const int32_t V = s_big[i];
+        const Row r = load_row<BATCH>(P, V);
+        const uint64_t hv = HASH ? vertex_hash(P.seed, static_cast<uint32_t>(r.lv)) : 0ull;
+        const uint32_t pv = HASH ? 0u : prio_of(__ldcg(st + V));
+        if (threadIdx.x == 0) s_sum = 0u;
+        __syncthreads();
+        unsigned c = ord_count_row<HASH>(P, st, r, static_cast<int>(threadIdx.x), static_cast<int>(blockDim.x), hv, pv);
+        c = __reduce_add_sync(kFull, c);
+        if (lane == 0 && c) atomicAdd(&s_sum, c);
+        __syncthreads();
+        c = s_sum;
+        if (threadIdx.x == 0) W[V] = ord_word(r.e - r.b, c);
+        if (threadIdx.x < 32) {
+            const bool ready[1] = {lane == 0 && c == 0};
+            const int32_t Vs[1] = {V}, ds[1] = {static_cast<int32_t>(r.e - r.b)};
+            ord_list<BATCH, 1>(P, ready, Vs, ds, L, lane);
+        }
+        __syncthreads();
+    }
+}
+
+// A slot without a neighbour: a color past every window, not to be released.
+constexpr uint64_t kOrdNone = 0x7fffffffull << 32;
+
+// Vertex V's color, into its word (its neighbours read it from the next round on) and the state array.
+__device__ __forceinline__ void ord_paint(const RoundParams &P, unsigned long long *W, int32_t V, int32_t c) {
+    W[V] = static_cast<uint64_t>(static_cast<uint32_t>(c)) << 32 | kOrdBias;
+    P.col0[V] = pack_state(c, 0u, true);
 }
 
 // Ready vertices of degree <= P.T1 <= kOrdSmall, one per lane (lanes with `valid`; warp-uniform
 // call): every entry loaded, then every state gathered, then the least color absent (at most
 // deg(v) < 64) and the releases.
 template <bool BATCH>
-__device__ __forceinline__ void ord_small(const RoundParams &P, uint64_t *col, int32_t *pend, bool valid, int32_t V,
+__device__ __forceinline__ void ord_small(const RoundParams &P, unsigned long long *W, bool valid, int4 x,
                                           const OrdLists &L, int pass, int lane, unsigned &st_deg,
                                           unsigned &st_cnt) {
+    const int32_t V = x.x;
     Row r{};
     int32_t deg = 0;
-    uint64_t self = 0;
     if (valid) {
-        r = load_row<BATCH>(P, V);
+        r = ord_row<BATCH>(P, x);
         deg = static_cast<int32_t>(r.e - r.b);
-        self = load_state(col + V);
     }
     int32_t ul[kOrdSmall];
     uint64_t w[kOrdSmall];
@@ -2191,10 +2304,10 @@ __device__ __forceinline__ void ord_small(const RoundParams &P, uint64_t *col, i
     for (int k = 0; k < kOrdSmall; ++k) ul[k] = k < deg ? load_entry(P.colidx + r.b + k) : 0;
 #pragma unroll
     for (int k = 0; k < kOrdSmall; ++k) {
-        w[k] = kNoNeighbour;
+        w[k] = kOrdNone;
         if (k < deg) {
             const int32_t U = neighbour(P, r, ul[k], r.b + k);
-            if (U >= 0) w[k] = load_state(col + U);
+            if (U >= 0) w[k] = load_state(reinterpret_cast<const uint64_t *>(W) + U);
         }
     }
     uint64_t mask = 0;
@@ -2202,14 +2315,14 @@ __device__ __forceinline__ void ord_small(const RoundParams &P, uint64_t *col, i
     int32_t U[kOrdSmall];
 #pragma unroll
     for (int k = 0; k < kOrdSmall; ++k) {
-        const int32_t c = color_of(w[k]);
+        const int32_t c = ord_color(w[k]);
         if (c >= 0 && c < 64) mask |= 1ull << c;
         take[k] = c < 0;
         U[k] = r.vbase + ul[k];
     }
-    ord_release<BATCH, kOrdSmall>(P, pend, take, U, L, lane);
+    ord_release<BATCH, kOrdSmall>(P, W, take, U, L, lane);
     if (valid) {
-        col[V] = pack_state(__ffsll(static_cast<long long>(~mask)) - 1, prio_of(self), true);
+        ord_paint(P, W, V, __ffsll(static_cast<long long>(~mask)) - 1);
         if constexpr (BATCH) note_graph_round(P, r.g, pass);
         st_deg += static_cast<unsigned>(deg);
         st_cnt += 1;
@@ -2220,16 +2333,16 @@ __device__ __forceinline__ void ord_small(const RoundParams &P, uint64_t *col, i
 // warp-uniform call): entry gl + 8k of the row in lane gl of the group, the group's colors OR-ed
 // into one mask (the least color absent is at most deg(v) <= kOrdMid < 64).
 template <bool BATCH>
-__device__ __forceinline__ void ord_mid(const RoundParams &P, uint64_t *col, int32_t *pend, bool valid, int32_t V,
+__device__ __forceinline__ void ord_mid(const RoundParams &P, unsigned long long *W, bool valid, int4 x,
                                         const OrdLists &L, int pass, int lane, unsigned &st_deg, unsigned &st_cnt) {
+    const int32_t V = x.x;
     const int gl = lane & (kOrdMidLanes - 1);
     Row r{};
     int32_t deg = 0;
     if (valid) {
-        r = load_row<BATCH>(P, V);
+        r = ord_row<BATCH>(P, x);
         deg = static_cast<int32_t>(r.e - r.b);
     }
-    const uint64_t self = valid && gl == 0 ? load_state(col + V) : 0;
     int32_t ul[kOrdMidPer];
     uint64_t w[kOrdMidPer];
 #pragma unroll
@@ -2240,10 +2353,10 @@ __device__ __forceinline__ void ord_mid(const RoundParams &P, uint64_t *col, int
 #pragma unroll
     for (int k = 0; k < kOrdMidPer; ++k) {
         const int32_t e = gl + kOrdMidLanes * k;
-        w[k] = kNoNeighbour;
+        w[k] = kOrdNone;
         if (e < deg) {
             const int32_t U = neighbour(P, r, ul[k], r.b + e);
-            if (U >= 0) w[k] = load_state(col + U);
+            if (U >= 0) w[k] = load_state(reinterpret_cast<const uint64_t *>(W) + U);
         }
     }
     uint64_t mask = 0;
@@ -2251,83 +2364,138 @@ __device__ __forceinline__ void ord_mid(const RoundParams &P, uint64_t *col, int
     int32_t U[kOrdMidPer];
 #pragma unroll
     for (int k = 0; k < kOrdMidPer; ++k) {
-        const int32_t c = color_of(w[k]);
+        const int32_t c = ord_color(w[k]);
         if (c >= 0 && c < 64) mask |= 1ull << c;
         take[k] = c < 0;
         U[k] = r.vbase + ul[k];
     }
 #pragma unroll
     for (int o = 1; o < kOrdMidLanes; o <<= 1) mask |= __shfl_xor_sync(kFull, mask, o);
-    ord_release<BATCH, kOrdMidPer>(P, pend, take, U, L, lane);
+    ord_release<BATCH, kOrdMidPer>(P, W, take, U, L, lane);
     if (valid && gl == 0) {
-        col[V] = pack_state(__ffsll(static_cast<long long>(~mask)) - 1, prio_of(self), true);
+        ord_paint(P, W, V, __ffsll(static_cast<long long>(~mask)) - 1);
         if constexpr (BATCH) note_graph_round(P, r.g, pass);
         st_deg += static_cast<unsigned>(deg);
         st_cnt += 1;
     }
 }
 
-// One work item {V, q, slot, nch} of a larger ready vertex (one warp): entries
-// [q P.CH, (q + 1) P.CH) of its row.  Colors of colored neighbours go into the window [0, 512)
-// (0..63 in registers, the rest in win); the last of the vertex's items picks the color.
+// Least color >= start absent from the row's colored neighbours (warp-cooperative).
 template <bool BATCH>
-__device__ void ord_item(const RoundParams &P, uint64_t *col, int32_t *pend, int4 it, unsigned *win,
-                         const OrdLists &L, int pass, int lane, unsigned &st_deg, unsigned &st_cnt) {
-    const int32_t V = it.x, q = it.y, slot = it.z, nch = it.w;
-    const Row r = load_row<BATCH>(P, V);
-    const int64_t jb = r.b + static_cast<int64_t>(q) * P.CH;
-    const int64_t je = min(r.e, jb + P.CH);
+__device__ int32_t ord_mex_from(const RoundParams &P, const unsigned long long *W, const Row &r, unsigned *win, int lane,
+                                int32_t start) {
+    for (int32_t base = start;; base += 32 * kAccWords) {
+        if (lane < kAccWords) win[lane] = 0;
+        __syncwarp();
+        for (int64_t j = r.b + lane; j < r.e; j += 32) {
+            const int32_t ul = __ldg(P.colidx + j);
+            if (static_cast<uint32_t>(ul) >= static_cast<uint32_t>(r.ng)) continue;
+            const int32_t x = ord_color(__ldcg(W + r.vbase + ul));
+            if (x >= base && x - base < 32 * kAccWords) atomicOr(&win[(x - base) >> 5], 1u << ((x - base) & 31));
+        }
+        __syncwarp();
+        const unsigned w = lane < kAccWords ? win[lane] : ~0u;
+        const unsigned open = __ballot_sync(kFull, ~w != 0u);
+        if (open) {
+            const int l = __ffs(static_cast<int>(open)) - 1;
+            return base + 32 * l + __ffs(static_cast<int>(~__shfl_sync(kFull, w, l))) - 1;
+        }
+        __syncwarp();
+    }
+}
+
+// One work item of a larger ready vertex (one warp).  Colors of colored neighbours go into the window
+// [0, 512) (0..63 in registers, the rest in win); the last of the vertex's items picks the color.
+template <bool BATCH>
+__device__ void ord_item(const RoundParams &P, unsigned long long *W, int4 it, unsigned *win, const OrdLists &L,
+                         int pass, int lane, unsigned &st_deg, unsigned &st_cnt) {
+    const int32_t V = it.x, slot = it.w;
+    Row r;
+    if constexpr (BATCH) {
+        r = load_row<true>(P, V);
+    } else {
+        r.b = 0;
+        r.e = 0;
+        r.vbase = 0;
+        r.ng = P.n;
+        r.lv = V;
+        r.g = 0;
+    }
+    const int64_t jb = (BATCH ? r.b : int64_t{0}) + it.y;
+    const int64_t je = jb + (it.z & (kOrdFirst - 1));
+    const int32_t deg = ord_degree(__ldcg(W + V));
     if (lane < kAccWords) win[lane] = 0;
     __syncwarp();
+    // an item is one step (P.CH <= kOrdChunk)
     uint64_t lo = 0;
-    for (int64_t j0 = jb; j0 < je; j0 += 32 * kOrdPer) {
-        int32_t ul[kOrdPer];
-        uint64_t w[kOrdPer];
+    int32_t ul[kOrdPer];
+    uint64_t w[kOrdPer];
 #pragma unroll
-        for (int k = 0; k < kOrdPer; ++k) {
-            const int64_t j = j0 + lane + 32 * k;
-            ul[k] = j < je ? load_entry(P.colidx + j) : 0;
-        }
+    for (int k = 0; k < kOrdPer; ++k) {
+        const int64_t j = jb + lane + 32 * k;
+        ul[k] = j < je ? load_entry(P.colidx + j) : 0;
+    }
 #pragma unroll
-        for (int k = 0; k < kOrdPer; ++k) {
-            const int64_t j = j0 + lane + 32 * k;
-            w[k] = kNoNeighbour;
-            if (j < je) {
-                const int32_t U = neighbour(P, r, ul[k], j);
-                if (U >= 0) w[k] = load_state(col + U);
-            }
+    for (int k = 0; k < kOrdPer; ++k) {
+        const int64_t j = jb + lane + 32 * k;
+        w[k] = kOrdNone;
+        if (j < je) {
+            const int32_t U = neighbour(P, r, ul[k], j);
+            if (U >= 0) w[k] = load_state(reinterpret_cast<const uint64_t *>(W) + U);
         }
-        bool take[kOrdPer];
-        int32_t U[kOrdPer];
+    }
+    bool take[kOrdPer];
+    int32_t U[kOrdPer];
 #pragma unroll
-        for (int k = 0; k < kOrdPer; ++k) {
-            const int32_t c = color_of(w[k]);
-            if (c >= 0 && c < 64)
-                lo |= 1ull << c;
-            else if (c >= 64 && c < 32 * kAccWords)
-                atomicOr(&win[c >> 5], 1u << (c & 31));
-            take[k] = c < 0;
-            U[k] = r.vbase + ul[k];
-        }
-        ord_release<BATCH, kOrdPer>(P, pend, take, U, L, lane);
+    for (int k = 0; k < kOrdPer; ++k) {
+        const int32_t c = ord_color(w[k]);
+        if (c >= 0 && c < 64)
+            lo |= 1ull << c;
+        else if (c >= 64 && c < 32 * kAccWords)
+            atomicOr(&win[c >> 5], 1u << (c & 31));
+        take[k] = c < 0;
+        U[k] = r.vbase + ul[k];
     }
     unsigned lo0 = __reduce_or_sync(kFull, static_cast<unsigned>(lo));
     unsigned lo1 = __reduce_or_sync(kFull, static_cast<unsigned>(lo >> 32));
     __syncwarp();
     if (lane == 0) {
         st_deg += static_cast<unsigned>(je - jb);
-        st_cnt += q == 0 ? 1u : 0u;
+        st_cnt += (it.z & kOrdFirst) ? 1u : 0u;
     }
-    bool unused = false;
-    if (nch > 1 && !merge_item<true>(P.acc + static_cast<size_t>(slot) * kOrdSlotWords, nch, lane, lo0, lo1, win,
-                                     unused, 0u))
-        return;
+    // the window into the vertex's slot, then the decrements, then the slot's count: the merge is under
+    // way while the released vertices are listed
+    const int32_t nch = (deg + P.CH - 1) / P.CH;
+    unsigned *a = P.acc + static_cast<size_t>(slot) * kOrdSlotWords;
+    if (nch > 1) {
+        const unsigned x = lane == 0 ? lo0 : lane == 1 ? lo1 : (lane < kAccWords ? win[lane] : 0u);
+        if (x) atomicOr(a + lane, x);
+    }
+    bool ready[kOrdPer];
+    int32_t dg[kOrdPer];
+    ord_count_down<kOrdPer>(W, take, U, 1u, ready, dg);
+    unsigned done = 0;
+    if (nch > 1) {
+        __syncwarp();
+        if (lane == 0) done = atom_add_acq_rel(a + kAccDone, 1u);
+    }
+    ord_list<BATCH, kOrdPer>(P, ready, U, dg, L, lane);
+    if (nch > 1) {
+        if (__shfl_sync(kFull, done, 0) != static_cast<unsigned>(nch - 1)) return;
+        __syncwarp();
+        const unsigned x = __ldcg(a + lane);
+        lo0 = __shfl_sync(kFull, x, 0);
+        lo1 = __shfl_sync(kFull, x, 1);
+        if (lane >= 2 && lane < kAccWords) win[lane] = x;
+        __syncwarp();
+        a[lane] = 0u;  // for the slot's next vertex
+    }
     int32_t nc = first_free(lo0, lo1, win);
     // every neighbour with a larger key is still uncolored, so the whole row's colors are the
     // smaller-key neighbours' colors
-    if (nc < 0) nc = mex_from<BATCH>(P, col, r, win, lane, 32 * kAccWords);
+    if (nc < 0) nc = ord_mex_from<BATCH>(P, W, load_row<BATCH>(P, V), win, lane, 32 * kAccWords);
     if (lane == 0) {
-        col[V] = pack_state(nc, prio_of(load_state(col + V)), true);
+        ord_paint(P, W, V, nc);
         if constexpr (BATCH) note_graph_round(P, r.g, pass);
     }
     __syncwarp();
@@ -2339,11 +2507,12 @@ __device__ void ord_item(const RoundParams &P, uint64_t *col, int32_t *pend, int
 // round's lists.  When the lists run dry, a vertex still uncolored means the input was not
 // symmetric.
 template <bool BATCH>
-__global__ void __launch_bounds__(kBlock, kWideBlocks) ord_round_kernel(RoundParams P, int32_t *pend) {
+__global__ void __launch_bounds__(kBlock, BATCH ? kWideBlocks : 2) ord_round_kernel(RoundParams P, unsigned long long *W) {
     __shared__ unsigned s_win[kMaxWarps][kAccWords];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const unsigned nw = gridDim.x * (blockDim.x >> 5);
-    const unsigned gw = blockIdx.x * (blockDim.x >> 5) + wib;
+    // interleaved over the blocks: a round of a hundred items takes a hundred SMs
+    const unsigned gw = static_cast<unsigned>(wib) * gridDim.x + blockIdx.x;
     unsigned *win = s_win[wib];
     uint64_t *col = P.col0;
     if (P.stats && blockIdx.x == 0 && threadIdx.x == 0) P.stats[4 * P.stats_cap] = global_ns();
@@ -2352,8 +2521,10 @@ __global__ void __launch_bounds__(kBlock, kWideBlocks) ord_round_kernel(RoundPar
     int pass = P.pass_begin;
     for (;; ++pass) {
         const OrdLists C = ord_lists(P, pass), L = ord_lists(P, pass + 1);
-        const unsigned nsmall = __ldcg(C.cnt + kCntSmall), nmid = __ldcg(C.cnt + kCntMulti);
-        const unsigned nitems = __ldcg(C.cnt + kCntChunks);
+        const unsigned nsmall = __ldcg(C.cnt + kOrdPad * kCntSmall), nmid = __ldcg(C.cnt + kOrdPad * kCntMulti);
+        const unsigned nitems = __ldcg(C.cnt + kOrdPad * kCntChunks);
+        // this warp's first item, in the counters' round trip (not used past the list's end)
+        const int4 first = gw < P.ord_items ? __ldcg(C.items + gw) : make_int4(0, 0, 0, 0);
         if (nsmall + nmid + nitems == 0u) {
             drained = true;
             break;
@@ -2363,20 +2534,21 @@ __global__ void __launch_bounds__(kBlock, kWideBlocks) ord_round_kernel(RoundPar
                 set_error(P.err, GC_ERR_NO_CONVERGENCE, pass, 0);
             break;
         }
-        if (blockIdx.x == 0 && threadIdx.x < kCnt) P.cnt[kCnt * ((pass + 2) % 3) + threadIdx.x] = 0u;
+        if (blockIdx.x == 0 && threadIdx.x < kCnt) P.ord_cnt[kOrdSet * ((pass + 2) % 3) + kOrdPad * threadIdx.x] = 0u;
         unsigned st_deg = 0, st_cnt = 0;
         for (unsigned i = gw; i < nitems; i += nw)
-            ord_item<BATCH>(P, col, pend, __ldcg(C.items + i), win, L, pass, lane, st_deg, st_cnt);
+            ord_item<BATCH>(P, W, i == gw ? first : __ldcg(C.items + i), win, L, pass, lane, st_deg, st_cnt);
         const unsigned mid_groups = (nmid + 3u) / 4u;
         for (unsigned b = (gw + nw - nitems % nw) % nw; b < mid_groups; b += nw) {
             const unsigned i = 4u * b + static_cast<unsigned>(lane >> 3);
-            ord_mid<BATCH>(P, col, pend, i < nmid, i < nmid ? __ldcg(C.mid + i) : 0, L, pass, lane, st_deg, st_cnt);
+            ord_mid<BATCH>(P, W, i < nmid, i < nmid ? __ldcg(C.mid + i) : make_int4(0, 0, 0, 0), L, pass, lane, st_deg,
+                           st_cnt);
         }
         const unsigned skip = (nitems + mid_groups) % nw;
         for (unsigned base = ((gw + nw - skip) % nw) * 32u; base < nsmall; base += nw * 32u) {
             const unsigned i = base + lane;
-            ord_small<BATCH>(P, col, pend, i < nsmall, i < nsmall ? __ldcg(C.small + i) : 0, L, pass, lane, st_deg,
-                             st_cnt);
+            ord_small<BATCH>(P, W, i < nsmall, i < nsmall ? __ldcg(C.small + i) : make_int4(0, 0, 0, 0), L, pass, lane,
+                             st_deg, st_cnt);
         }
         if (P.stats) flush_stats(P, pass, st_deg, st_cnt, st_deg);
         if (!grid_sync(P.bar, bar_target, P.err, P.spin_ns)) break;
@@ -2404,7 +2576,7 @@ __global__ void __launch_bounds__(kBlock, kWideBlocks) ord_round_kernel(RoundPar
 // Decrements of removed vertices are harmless: their res is already <= k and never fires.
 
 // res, level and the two threshold words (the least res of a search, alternating).
-__global__ void peel_init_kernel(RoundParams P, int32_t *res, int32_t *level, unsigned *kw, unsigned *items) {
+__global__ void peel_init_kernel(RoundParams P, unsigned long long *W, int32_t *level, unsigned *kw, unsigned *items) {
     const int lane = threadIdx.x & 31;
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
     if (blockIdx.x == 0 && threadIdx.x == 0) kw[0] = kw[1] = 0x7fffffffu;
@@ -2420,7 +2592,7 @@ __global__ void peel_init_kernel(RoundParams P, int32_t *res, int32_t *level, un
                 set_error(P.err, GC_ERR_INVALID_GRAPH, static_cast<int32_t>(V), b);
                 d = 0;
             }
-            res[V] = static_cast<int32_t>(d);
+            W[V] = ord_word(d, static_cast<unsigned>(d));
             level[V] = 0;
             if (d > kOrdMid) nch = static_cast<unsigned>((d + P.CH - 1) / P.CH);
         }
@@ -2430,15 +2602,12 @@ __global__ void peel_init_kernel(RoundParams P, int32_t *res, int32_t *level, un
 }
 
 // One level for the vertices of degree <= P.T1, one per lane (lanes with `valid`).
-__device__ __forceinline__ void peel_small(const RoundParams &P, int32_t *res, int32_t *level, bool valid, int32_t V,
+__device__ __forceinline__ void peel_small(const RoundParams &P, unsigned long long *W, int32_t *level, bool valid, int4 x,
                                            int32_t k, int32_t L, const OrdLists &N, int lane) {
-    int64_t b = 0;
-    int32_t deg = 0;
-    if (valid) {
-        b = __ldg(P.rowptr + V);
-        deg = static_cast<int32_t>(__ldg(P.rowptr + V + 1) - b);
-        level[V] = L;
-    }
+    const int32_t V = x.x;
+    const int64_t b = x.y;
+    const int32_t deg = valid ? x.z : 0;
+    if (valid) level[V] = L;
     bool take[kOrdSmall];
     int32_t U[kOrdSmall];
 #pragma unroll
@@ -2447,20 +2616,17 @@ __device__ __forceinline__ void peel_small(const RoundParams &P, int32_t *res, i
         take[q] = q < deg && static_cast<uint32_t>(U[q]) < static_cast<uint32_t>(P.n) && U[q] != V;
         if (q < deg && !take[q]) set_error(P.err, GC_ERR_INVALID_GRAPH, V, b + q);
     }
-    ord_release<false, kOrdSmall>(P, res, take, U, N, lane, k + 1);
+    ord_release<false, kOrdSmall>(P, W, take, U, N, lane, static_cast<unsigned>(k) + 1u);
 }
 
 // One level for the vertices of degree in (P.T1, kOrdMid], one per 8-lane group.
-__device__ __forceinline__ void peel_mid(const RoundParams &P, int32_t *res, int32_t *level, bool valid, int32_t V,
+__device__ __forceinline__ void peel_mid(const RoundParams &P, unsigned long long *W, int32_t *level, bool valid, int4 x,
                                          int32_t k, int32_t L, const OrdLists &N, int lane) {
     const int gl = lane & (kOrdMidLanes - 1);
-    int64_t b = 0;
-    int32_t deg = 0;
-    if (valid) {
-        b = __ldg(P.rowptr + V);
-        deg = static_cast<int32_t>(__ldg(P.rowptr + V + 1) - b);
-        if (gl == 0) level[V] = L;
-    }
+    const int32_t V = x.x;
+    const int64_t b = x.y;
+    const int32_t deg = valid ? x.z : 0;
+    if (valid && gl == 0) level[V] = L;
     bool take[kOrdMidPer];
     int32_t U[kOrdMidPer];
 #pragma unroll
@@ -2470,17 +2636,15 @@ __device__ __forceinline__ void peel_mid(const RoundParams &P, int32_t *res, int
         take[q] = e < deg && static_cast<uint32_t>(U[q]) < static_cast<uint32_t>(P.n) && U[q] != V;
         if (e < deg && !take[q]) set_error(P.err, GC_ERR_INVALID_GRAPH, V, b + e);
     }
-    ord_release<false, kOrdMidPer>(P, res, take, U, N, lane, k + 1);
+    ord_release<false, kOrdMidPer>(P, W, take, U, N, lane, static_cast<unsigned>(k) + 1u);
 }
 
-// One level for a work item {V, q, slot, nch} of a larger vertex (one warp).
-__device__ __forceinline__ void peel_item(const RoundParams &P, int32_t *res, int32_t *level, int4 it, int32_t k,
+// One level for a work item of a larger vertex (one warp).
+__device__ __forceinline__ void peel_item(const RoundParams &P, unsigned long long *W, int32_t *level, int4 it, int32_t k,
                                           int32_t L, const OrdLists &N, int lane) {
-    const int32_t V = it.x, q = it.y;
-    const int64_t b = __ldg(P.rowptr + V), e = __ldg(P.rowptr + V + 1);
-    const int64_t jb = b + static_cast<int64_t>(q) * P.CH;
-    const int64_t je = min(e, jb + P.CH);
-    if (q == 0 && lane == 0) level[V] = L;
+    const int32_t V = it.x;
+    const int64_t jb = it.y, je = jb + (it.z & (kOrdFirst - 1));
+    if ((it.z & kOrdFirst) && lane == 0) level[V] = L;
     for (int64_t j0 = jb; j0 < je; j0 += 32 * kOrdPer) {
         bool take[kOrdPer];
         int32_t U[kOrdPer];
@@ -2491,7 +2655,7 @@ __device__ __forceinline__ void peel_item(const RoundParams &P, int32_t *res, in
             take[t] = j < je && static_cast<uint32_t>(U[t]) < static_cast<uint32_t>(P.n) && U[t] != V;
             if (j < je && !take[t]) set_error(P.err, GC_ERR_INVALID_GRAPH, V, j);
         }
-        ord_release<false, kOrdPer>(P, res, take, U, N, lane, k + 1);
+        ord_release<false, kOrdPer>(P, W, take, U, N, lane, static_cast<unsigned>(k) + 1u);
     }
 }
 
@@ -2500,12 +2664,12 @@ __device__ __forceinline__ void peel_item(const RoundParams &P, int32_t *res, in
 // previous one left (all vertices for the first), and its listing scan writes the ones it does not
 // list to the other of rlist0 / rlist1 (counts rcnt[0] / rcnt[1], zero at launch), so that the
 // scans shrink with the graph.
-__global__ void __launch_bounds__(kBlock, kWideBlocks) peel_kernel(RoundParams P, int32_t *res, int32_t *level,
+__global__ void __launch_bounds__(kBlock, kWideBlocks) peel_kernel(RoundParams P, unsigned long long *W, int32_t *level,
                                                                    unsigned *kw, int32_t *rlist0, int32_t *rlist1,
                                                                    unsigned *rcnt) {
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const unsigned nw = gridDim.x * (blockDim.x >> 5);
-    const unsigned gw = blockIdx.x * (blockDim.x >> 5) + wib;
+    const unsigned gw = static_cast<unsigned>(wib) * gridDim.x + blockIdx.x;
     const int64_t nthreads = static_cast<int64_t>(gridDim.x) * blockDim.x;
     const int64_t gtid = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     unsigned bar_target = 0;
@@ -2522,7 +2686,7 @@ __global__ void __launch_bounds__(kBlock, kWideBlocks) peel_kernel(RoundParams P
         unsigned m = 0x7fffffffu;
         for (int64_t i = gtid; i < nr; i += nthreads) {
             const int32_t v = f == 0 ? static_cast<int32_t>(i) : __ldcg(rcur + i);
-            if (__ldcg(level + v) == 0) m = min(m, static_cast<unsigned>(__ldcg(res + v)));
+            if (__ldcg(level + v) == 0) m = min(m, static_cast<unsigned>(__ldcg(W + v)) - static_cast<unsigned>(kOrdBias));
         }
         m = __reduce_min_sync(kFull, m);
         if (lane == 0 && m != 0x7fffffffu) atomicMin(kw + (f & 1), m);
@@ -2539,35 +2703,39 @@ __global__ void __launch_bounds__(kBlock, kWideBlocks) peel_kernel(RoundParams P
                 const int64_t i = base + lane;
                 int32_t v = 0;
                 bool present = false, now = false;
+                uint64_t w = 0;
                 if (i < nr) {
                     v = f == 0 ? static_cast<int32_t>(i) : __ldcg(rcur + i);
                     present = __ldcg(level + v) == 0;
-                    now = present && __ldcg(res + v) <= k;
+                    w = __ldcg(W + v);
+                    now = present && static_cast<int32_t>(static_cast<unsigned>(w) - static_cast<unsigned>(kOrdBias)) <= k;
                 }
                 warp_append(present && !now, v, rnext, rcnt + ((f + 1) & 1), lane);
                 const bool ready[1] = {now};
-                const int32_t Vs[1] = {v};
-                ord_list<false, 1>(P, ready, Vs, F, lane);
+                const int32_t Vs[1] = {v}, ds[1] = {ord_degree(w)};
+                ord_list<false, 1>(P, ready, Vs, ds, F, lane);
             }
         }
         if (!grid_sync(P.bar, bar_target, P.err, P.spin_ns)) break;
         for (;; ++pass) {
             const OrdLists C = ord_lists(P, pass), N = ord_lists(P, pass + 1);
-            const unsigned nsmall = __ldcg(C.cnt + kCntSmall), nmid = __ldcg(C.cnt + kCntMulti);
-            const unsigned nitems = __ldcg(C.cnt + kCntChunks);
+            const unsigned nsmall = __ldcg(C.cnt + kOrdPad * kCntSmall), nmid = __ldcg(C.cnt + kOrdPad * kCntMulti);
+            const unsigned nitems = __ldcg(C.cnt + kOrdPad * kCntChunks);
+            const int4 first = gw < P.ord_items ? __ldcg(C.items + gw) : make_int4(0, 0, 0, 0);
             if (nsmall + nmid + nitems == 0u) break;
-            if (blockIdx.x == 0 && threadIdx.x < kCnt) P.cnt[kCnt * ((pass + 2) % 3) + threadIdx.x] = 0u;
+            if (blockIdx.x == 0 && threadIdx.x < kCnt) P.ord_cnt[kOrdSet * ((pass + 2) % 3) + kOrdPad * threadIdx.x] = 0u;
             ++L;
-            for (unsigned i = gw; i < nitems; i += nw) peel_item(P, res, level, __ldcg(C.items + i), k, L, N, lane);
+            for (unsigned i = gw; i < nitems; i += nw)
+                peel_item(P, W, level, i == gw ? first : __ldcg(C.items + i), k, L, N, lane);
             const unsigned mid_groups = (nmid + 3u) / 4u;
             for (unsigned b = (gw + nw - nitems % nw) % nw; b < mid_groups; b += nw) {
                 const unsigned i = 4u * b + static_cast<unsigned>(lane >> 3);
-                peel_mid(P, res, level, i < nmid, i < nmid ? __ldcg(C.mid + i) : 0, k, L, N, lane);
+                peel_mid(P, W, level, i < nmid, i < nmid ? __ldcg(C.mid + i) : make_int4(0, 0, 0, 0), k, L, N, lane);
             }
             const unsigned skip = (nitems + mid_groups) % nw;
             for (unsigned base = ((gw + nw - skip) % nw) * 32u; base < nsmall; base += nw * 32u) {
                 const unsigned i = base + lane;
-                peel_small(P, res, level, i < nsmall, i < nsmall ? __ldcg(C.small + i) : 0, k, L, N, lane);
+                peel_small(P, W, level, i < nsmall, i < nsmall ? __ldcg(C.small + i) : make_int4(0, 0, 0, 0), k, L, N, lane);
             }
             if (!grid_sync(P.bar, bar_target, P.err, P.spin_ns)) {
                 ok = false;
@@ -2941,37 +3109,37 @@ cudaError_t ordered_kernel_occupancy(bool batch, int block, int *blocks_per_sm) 
         block, 0);
 }
 
-cudaError_t launch_ordered(const RoundParams &P, bool batch, int32_t *pend, int grid, int block, cudaStream_t s) {
+cudaError_t launch_ordered(const RoundParams &P, bool batch, unsigned long long *W, int grid, int block, cudaStream_t s) {
     if (block != kBlock) return cudaErrorInvalidValue;
     if (P.n <= 0) return cudaSuccess;
     const int cgrid = grid_for(static_cast<int64_t>(P.n) * 32, 256, sm_count() * 16);
     const bool hash = P.priority == GC_PRIORITY_HASH;
     if (batch) {
         if (hash)
-            ord_count_kernel<true, true><<<cgrid, 256, 0, s>>>(P, pend);
+            ord_count_kernel<true, true><<<cgrid, 256, 0, s>>>(P, W);
         else
-            ord_count_kernel<true, false><<<cgrid, 256, 0, s>>>(P, pend);
+            ord_count_kernel<true, false><<<cgrid, 256, 0, s>>>(P, W);
     } else {
         if (hash)
-            ord_count_kernel<false, true><<<cgrid, 256, 0, s>>>(P, pend);
+            ord_count_kernel<false, true><<<cgrid, 256, 0, s>>>(P, W);
         else
-            ord_count_kernel<false, false><<<cgrid, 256, 0, s>>>(P, pend);
+            ord_count_kernel<false, false><<<cgrid, 256, 0, s>>>(P, W);
     }
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemsetAsync(&P.bar->count, 0, sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
     RoundParams arg = P;
-    int32_t *parg = pend;
+    unsigned long long *parg = W;
     void *args[] = {&arg, &parg};
     return cudaLaunchCooperativeKernel(batch ? reinterpret_cast<const void *>(&ord_round_kernel<true>)
                                              : reinterpret_cast<const void *>(&ord_round_kernel<false>),
                                        dim3(grid), dim3(block), args, 0, s);
 }
 
-cudaError_t launch_peel_init(const RoundParams &P, int32_t *res, int32_t *level, unsigned *kw, unsigned *items,
+cudaError_t launch_peel_init(const RoundParams &P, unsigned long long *W, int32_t *level, unsigned *kw, unsigned *items,
                              cudaStream_t s) {
     const int grid = grid_for(P.n > 0 ? P.n : 1, 256, sm_count() * 16);
-    peel_init_kernel<<<grid, 256, 0, s>>>(P, res, level, kw, items);
+    peel_init_kernel<<<grid, 256, 0, s>>>(P, W, level, kw, items);
     return cudaGetLastError();
 }
 
@@ -2981,7 +3149,7 @@ cudaError_t peel_kernel_occupancy(int block, int *blocks_per_sm) {
                                                          block, 0);
 }
 
-cudaError_t launch_peel(const RoundParams &P, int32_t *res, int32_t *level, unsigned *kw, int32_t *rlist0,
+cudaError_t launch_peel(const RoundParams &P, unsigned long long *W, int32_t *level, unsigned *kw, int32_t *rlist0,
                         int32_t *rlist1, unsigned *rcnt, int grid, int block, cudaStream_t s) {
     if (block != kBlock) return cudaErrorInvalidValue;
     if (P.n <= 0) return cudaSuccess;
@@ -2989,7 +3157,8 @@ cudaError_t launch_peel(const RoundParams &P, int32_t *res, int32_t *level, unsi
     if (e == cudaSuccess) e = cudaMemsetAsync(rcnt, 0, 2 * sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
     RoundParams arg = P;
-    int32_t *ra = res, *la = level, *r0 = rlist0, *r1 = rlist1;
+    unsigned long long *ra = W;
+    int32_t *la = level, *r0 = rlist0, *r1 = rlist1;
     unsigned *ka = kw, *rc = rcnt;
     void *args[] = {&arg, &ra, &la, &ka, &r0, &r1, &rc};
     return cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(&peel_kernel), dim3(grid), dim3(block), args, 0,
