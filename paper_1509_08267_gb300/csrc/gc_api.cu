@@ -656,7 +656,12 @@ static int run(Context &C, const Problem &pb, int mode, uint64_t seed, const gc_
     // memory once at most core_M vertices with at most core_E list entries remain
     const int32_t core_opt = opt ? opt->core_vertices : 0;
     CoreParams Q{};
-    if (mode == GC_MODE_DETERMINISTIC && compact && core_opt >= 0 && pb.nnz > 0) {
+    // Without larger vertices (no row past T1) the default is no core phase: its warps then sweep rows of
+    // a few dozen entries one at a time (~200 instructions a row) and its set-up re-reads every row,
+    // while the round kernel takes a row per thread (ER n = 50,000 degree 24: 300 us against 508 with
+    // the core; stencil 60 x 50 x 40: 375 against 826; ER n = 10^6 degree 32: 1.45 ms against 1.68;
+    // with hubs the core wins: R-MAT n = 150,000 1.43 ms against 2.02).
+    if (mode == GC_MODE_DETERMINISTIC && compact && core_opt >= 0 && (core_opt > 0 || n_items > 0) && pb.nnz > 0) {
         if (C.core_max_v == 0) {
             const int32_t cm = core_max_vertices();
             C.core_max_v = cm > 0 ? cm : -1;
