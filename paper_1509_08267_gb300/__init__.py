@@ -180,12 +180,27 @@ def _on_cuda(x) -> bool:
     return _is_torch(x) and x.is_cuda
 
 
+_LEGACY_STREAM = 1  # cudaStreamLegacy: the default stream by its own handle
+
+
 def _current_stream(*arrays):
+    """The stream a call's work is queued on, behind what torch queued there.  torch's default stream
+    has the handle 0, which gc_options reads as "the library's own stream": that one does not wait for
+    torch, so the default stream is passed by its other handle."""
     for a in arrays:
         if _on_cuda(a):
             import torch
-            return ctypes.c_void_p(torch.cuda.current_stream(a.device).cuda_stream)
+            return ctypes.c_void_p(torch.cuda.current_stream(a.device).cuda_stream or _LEGACY_STREAM)
     return ctypes.c_void_p(0)
+
+
+def _finish_queued(*arrays):
+    """Waits for the current torch stream before a call that takes no stream, if an array is on the GPU."""
+    for a in arrays:
+        if _on_cuda(a):
+            import torch
+            torch.cuda.current_stream(a.device).synchronize()
+            return
 
 
 def _empty_like_home(ref, n: int, dtype=np.int32):
@@ -301,6 +316,7 @@ def det_round(rowptr, colidx, seed: int, colors_cur, worklist, colors_next=None,
         lost = _empty_like_home(worklist, nwork)
     pn, nk = _ptr(colors_next, np.int32)
     pl, lk = _ptr(lost, np.int32)
+    _finish_queued(rowptr, colidx, colors_cur, worklist, colors_next, lost)
     _check(lib.gc_det_round(n, prp, pci, seed & ((1 << 64) - 1), pcur, pw, nwork, pn, pl))
     return (nk if nk is not None else colors_next), (lk if lk is not None else lost)
 
@@ -340,7 +356,7 @@ def _color_one(rowptr, colidx, mode, seed, out, options, stats, round_cap, color
     if stats:
         opt = Options(**{**opt.__dict__, "flags": opt.flags | FLAG_STATS | FLAG_TIMING})
     want_stats = bool(opt.flags & (FLAG_STATS | FLAG_TIMING))
-    copt = opt._c(_current_stream(rowptr, colidx, out))
+    copt = opt._c(_current_stream(rowptr, colidx, out, colors_in))
     # the per-round arrays only when asked for: making and dropping 2 MB of them took half of a small
     # call's time (1,000 vertices: 114 us a call, 38 of them in the library)
     st, (wl, ds, rn, rr) = _stats_arrays(round_cap) if want_stats else (None, (None,) * 4)
@@ -399,6 +415,7 @@ def validate(rowptr, colidx, flags: int = VALIDATE_ALL) -> None:
     n = (rowptr.numel() if _is_torch(rowptr) else len(rowptr)) - 1
     prp, rk = _ptr(rowptr, np.int32)
     pci, ck = _ptr(colidx, np.int32)
+    _finish_queued(rowptr, colidx)
     _check(lib.gc_validate_graph(n, prp, pci, flags))
 
 
@@ -433,6 +450,7 @@ class Server:
         rid = ctypes.c_uint64(0)
         m = _mode(self._mode if mode is None else mode)
         sd = (self._seed if seed is None else seed) & ((1 << 64) - 1)
+        _finish_queued(rowptr, colidx)
         _check(load().gc_server_submit(self._h, n, prp, pci, m, sd, ctypes.byref(rid)))
         self._n[rid.value] = n
         return int(rid.value)
@@ -443,6 +461,7 @@ class Server:
         if out is None:
             out = np.empty(n, np.int32)
         pout, ok = _ptr(out, np.int32)
+        _finish_queued(out)
         nc = ctypes.c_int32(0)
         rd = ctypes.c_int32(0)
         st = load().gc_server_poll(self._h, req_id, timeout_ms, pout, ctypes.byref(nc), ctypes.byref(rd))
