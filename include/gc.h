@@ -118,8 +118,10 @@ typedef struct gc_options {
                                   80-register variant (3 blocks per SM) when most adjacency entries are
                                   in vertices of degree > small_max_degree, else the 64-register one (4);
                                   3 or 4: that variant; 1 or 2: the 64-register one, capped.  It also
-                                  sets the ordered mode's blocks per SM (default 1 on a single graph,
-                                  3 on a batch) and caps the smallest-last peeling kernels (3 per SM) */
+                                  sets the ordered mode's blocks per SM (default 2 on a single graph,
+                                  as many as fit on a batch) and the smallest-last peeling's (default
+                                  2).  Without any vertex of degree > small_max_degree the deterministic
+                                  mode's default is a variant without work-item code */
     int64_t spin_limit_ns;     /* grid-barrier wait limit in ns; 0 = 1e9.  A wait that runs out makes
                                   the call return GC_ERR_TIMEOUT with the device still usable */
     uint32_t flags;            /* GC_FLAG_* */

@@ -184,15 +184,15 @@ constexpr int kCoreCnt = 8;  // counter words per set
 #define GC_CORE_PIECE 2048
 #endif
 constexpr int kCorePiece = GC_CORE_PIECE;
-// Per core vertex, kCoreRecWords words: [0, 16) the round's window of neighbour colors 0..511,
-// kCoreFlag (some smaller-key neighbour has the vertex's color), kCoreDone (pieces of the vertex done
-// this round) -- the round part, used by vertices with several pieces --, [kAccFin, kAccFin + 16) the
-// window of final neighbours' colors, then the row's offset in the pool, degree, global id, row
-// length, graph, the hand-over list and the vertex's range of pieces.
+// Per core vertex, kCoreRecWords words: [0, 16) the window of neighbour colors 0..511 and kCoreFlag
+// (some smaller-key neighbour has the vertex's color), which the row build leaves for the core's first
+// round, [kAccFin, kAccFin + 16) the window of final neighbours' colors, then the row's offset in the
+// pool, degree, global id, row length, graph, the hand-over list's length and the vertex's range of
+// pieces.
 constexpr int kCoreRecWords = 64;
-constexpr int kCoreFlag = 16, kCoreDone = 17;
+constexpr int kCoreFlag = 16;
 constexpr int kCoreOffLo = 48, kCoreOffHi = 49, kCoreDeg = 50, kCoreGid = 51, kCoreFill = 52, kCoreG = 53;
-constexpr int kCoreListLo = 54, kCoreListHi = 55, kCoreListLen = 56, kCorePcBeg = 57, kCorePcEnd = 58;
+constexpr int kCoreListLen = 56, kCorePcBeg = 57, kCorePcEnd = 58;
 constexpr int kCoreTail = 59;  // the vertex's tail id (tail phase)
 // Tail phase (gc_tail.cu).  Once the core's worklist has at most tail_max vertices, one thread-block
 // cluster of tail_nc blocks runs the remaining rounds: the worklist vertices get tail ids 0..k-1 in
@@ -324,8 +324,8 @@ cudaError_t launch_det_round_block(int32_t n, const int32_t *rowptr, const int32
                                   const int32_t *cur, const int32_t *work, int32_t nwork, int32_t *next, int32_t *lost,
                                   int32_t *err, cudaStream_t s);
 // Core phase (after launch_rounds handed over, *P.core_go = 1; every kernel returns at once when
-// it did not): local ids and rows, the round kernel, and the final colors written back to col0 and
-// col1.  core_max_vertices: the largest M the shared memory of one block per SM allows.
+// it did not): local ids and rows, the round kernel, and the final colors written back to both buffers
+// of the vertex state.  core_max_vertices: the largest M the shared memory of one block per SM allows.
 int32_t core_max_vertices();
 cudaError_t launch_core(const RoundParams &P, const CoreParams &Q, bool batch, cudaStream_t s);
 // Tail phase: the largest cluster (16 or 8 blocks) the tail kernel can run as, 0 if none; the launch

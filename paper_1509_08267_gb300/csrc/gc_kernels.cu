@@ -353,7 +353,7 @@ __device__ __noinline__ bool det_small_exact(const RoundParams &P, const DetStat
 // places, so a row load costs 32 cache-line lookups whatever its width, and whole-sector loads make
 // the fewest of them.  A least-of-differences instead of a compare per entry and clamped shifts
 // instead of 64-bit windows keep the step at about nine instructions an entry.  256^3 stencil, whole
-// coloring: 8.5 ms, against 16.0 with 16-byte loads, 8-byte state gathers and a key test per entry of
+// coloring: 8.35 ms, against 16.0 with 16-byte loads, 8-byte state gathers and a key test per entry of
 // equal color; 4,096 graphs of 100..4,000 vertices: 5.4 against 7.4.  (Groups of 4 or 8 lanes per
 // row, rows in shared memory: 19.4 ms, three times the instructions.)
 template <int W>
