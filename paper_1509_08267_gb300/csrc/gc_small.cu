@@ -550,15 +550,16 @@ __global__ void __launch_bounds__(kOneThreads, 1) small_one_kernel(const __grid_
         __syncthreads();
     small_setup(P, g, S, st[1], list[1], cap, lo, hi, CLUSTER ? nullptr : st[0]);
     if (threadIdx.x == 0) S.stop = S.bad;
-    __syncthreads();
     if (CLUSTER) {
-        // the exchange buffers start with the block's own vertices' states
+        // the exchange buffers start with the block's own vertices' states; before the barrier, because
+        // round 1 writes them from whichever thread has the vertex on its list
         for (int32_t v = lo + static_cast<int32_t>(threadIdx.x); v < hi; v += kOneThreads) {
             const uint32_t w = st[1][v];
             __stcg(A.exchange + v, w);
             __stcg(A.exchange + cap + v, w);
         }
     }
+    __syncthreads();
     // this block's worklist; the cluster's size is known once the first round has run, and a round over
     // an empty list changes nothing
     unsigned left = 1u;
