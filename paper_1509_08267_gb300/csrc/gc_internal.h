@@ -55,6 +55,14 @@ constexpr int kOrdSingleChunk = 64;  // default work-item size of the ordered mo
 constexpr int kOrdSlotWords = 32;
 constexpr int kOrdPad = 32, kOrdSet = 4 * kOrdPad;  // words from one counter, or counter set, to the next
 
+// One row of a batch's offset tables: graph g's vertices [v0, v1) of n, entries [e0, e1) of nnz.  Every
+// row is checked against the totals by itself: a table that rises and falls again has rows that look
+// right next to each other and lie outside the arrays.
+inline __host__ __device__ bool batch_row_ok(int32_t g, int64_t v0, int64_t v1, int64_t e0, int64_t e1, int64_t n,
+                                             int64_t nnz) {
+    return 0 <= v0 && v0 <= v1 && v1 <= n && 0 <= e0 && e0 <= e1 && e1 <= nnz && (g != 0 || (v0 == 0 && e0 == 0));
+}
+
 // Worklist counters: three sets used round-robin (read / append / clear), kCnt words each.
 constexpr int kCnt = 4;
 //   kCntSmall   vertices of degree <= T1

@@ -1465,14 +1465,14 @@ __global__ void batch_tables_kernel(RoundParams P, const int64_t *vtx_off, const
     for (int32_t g = blockIdx.x; g < P.G; g += gridDim.x) {
         const int64_t v0 = vtx_off[g], v1 = vtx_off[g + 1];
         const int64_t e0 = edge_off[g], e1 = edge_off[g + 1];
-        const bool ok = v1 >= v0 && e1 >= e0 && v1 <= P.n && (g != 0 || (v0 == 0 && e0 == 0));
+        const bool ok = batch_row_ok(g, v0, v1, e0, e1, P.n, P.nnz);
         if (threadIdx.x == 0) {
             if (!ok) set_error(P.err, GC_ERR_INVALID_GRAPH, -1 - g, 0);
             g_vbase[g] = ok ? v0 : 0;
             g_n[g] = ok ? static_cast<int32_t>(v1 - v0) : 0;
-            g_ebase[g] = e0;
-            g_rbase[g] = v0 + g;
-            g_m[g] = e1 - e0;
+            g_ebase[g] = ok ? e0 : 0;
+            g_rbase[g] = ok ? v0 + g : 0;
+            g_m[g] = ok ? e1 - e0 : 0;
             P.graph_last[g] = (ok && v1 > v0) ? 1 : 0;
         }
         if (!ok) continue;

@@ -409,8 +409,8 @@ __global__ void __launch_bounds__(kBatchThreads, kBatchBlocks) small_batch_kerne
             }
             __syncthreads();
         }
-        // FINAL in both buffers of the batch's state (only if nothing is wrong; the color count and the
-        // copy to the caller's array read them)
+        // FINAL in both buffers of the batch's state; the color count and, if no error was posted, the copy
+        // to the caller's array read them
         const uint32_t *fin = st[pass & 1];
         for (int32_t v = static_cast<int32_t>(threadIdx.x); v < g.n; v += static_cast<int32_t>(blockDim.x)) {
             const int32_t c = static_cast<int32_t>(fin[v] >> 17);
@@ -432,6 +432,13 @@ constexpr int kQueueThreads = 1024;
 __global__ void __launch_bounds__(kQueueThreads) small_queue_kernel(RoundParams P, SmallBatch B, int64_t share) {
     __shared__ unsigned s_n[64], s_at[64];
     __shared__ unsigned long long s_left, s_small, s_all;
+    if (P.err[0] != 0) {  // the tables are wrong: the call ends with that error, nothing is colored
+        if (threadIdx.x == 0) {
+            *B.queued = *B.taken = 0u;
+            *B.left = 0ull;
+        }
+        return;
+    }
     if (threadIdx.x < 64) s_n[threadIdx.x] = 0u;
     if (threadIdx.x == 0) s_left = s_small = s_all = 0ull;
     __syncthreads();
