@@ -37,6 +37,7 @@
 #include <algorithm>
 #include <cstdio>
 #include <cstdlib>
+#include <mutex>
 
 #include "gc_device.cuh"
 
@@ -1077,15 +1078,23 @@ int core_static_smem(bool batch) {
 
 }  // namespace
 
+// Asked once per device.  The shared-memory limit of the round kernels is set to that size and never
+// lowered: it is one value per function and device, and calls of several threads (a call's, each
+// server's worker) launch the kernels with different sizes.
 int32_t core_max_vertices() {
+    static std::mutex mu;
+    static int32_t known[128];  // 0: not asked yet, -1: none
     int dev = 0, optin = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 128 ||
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
+    std::lock_guard<std::mutex> lk(mu);
+    if (known[dev] != 0) return std::max(known[dev], 0);
     const int st = std::max(core_static_smem(false), core_static_smem(true));
     if (st < 0) return 0;
+    known[dev] = -1;
     // the largest multiple of 64 vertices whose colors and FINAL bits leave one block resident per SM
     for (int64_t m = ((static_cast<int64_t>(optin) - st - 4) * 8 / 9) & ~int64_t{63}; m >= 64; m -= 1024) {
         const int smem = static_cast<int>(core_smem_bytes(m));
@@ -1098,10 +1107,13 @@ int32_t core_max_vertices() {
                  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, kCoreThreads, smem) == cudaSuccess &&
                  per_sm >= 1;
         }
-        if (ok) return static_cast<int32_t>(m);
+        if (ok) {
+            known[dev] = static_cast<int32_t>(m);
+            break;
+        }
         cudaGetLastError();
     }
-    return 0;
+    return std::max(known[dev], 0);
 }
 
 cudaError_t launch_core(const RoundParams &P, const CoreParams &Q, bool batch, cudaStream_t s) {
@@ -1112,12 +1124,7 @@ cudaError_t launch_core(const RoundParams &P, const CoreParams &Q, bool batch, c
     const size_t smem = core_smem_bytes(Q.max_v);
     const void *round_fn = batch ? reinterpret_cast<const void *>(&core_round_kernel<true>)
                                  : reinterpret_cast<const void *>(&core_round_kernel<false>);
-    e = cudaFuncSetAttribute(round_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, round_fn, kCoreThreads, smem);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
+    if (Q.max_v > core_max_vertices()) return cudaErrorInvalidConfiguration;
     const int grid = sms * 8;
     if (batch) {
         core_index_kernel<true><<<grid, 256, 0, s>>>(P, Q);
