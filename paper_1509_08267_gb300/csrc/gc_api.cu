@@ -546,6 +546,7 @@ static int run(Context &C, const Problem &pb, int mode, uint64_t seed, const gc_
     const bool timing = (flags & GC_FLAG_TIMING) != 0;
     Ctl h{};
     bool small = false;
+    int small_grid = 0;
     if (pb.batch) {
         GC_CUDA(launch_batch_tables(P, pb.vtx_off, pb.edge_off, C.g_vbase.as<int64_t>(), C.g_n.as<int32_t>(),
                                     C.g_ebase.as<int64_t>(), C.g_rbase.as<int64_t>(), C.g_m.as<int64_t>(), s));
@@ -557,7 +558,7 @@ static int run(Context &C, const Problem &pb, int mode, uint64_t seed, const gc_
             P.g_done = C.small_done.as<uint8_t>();
             const SmallBatch B{C.small_queue.as<int32_t>(), ctl->small_ctl, ctl->small_ctl + 1, &ctl->small_left,
                                C.small_done.as<uint8_t>()};
-            GC_CUDA(launch_small_batch(P, B, pb.nnz, s));
+            GC_CUDA(launch_small_batch(P, B, pb.nnz, s, &small_grid));
         }
         GC_CUDA(cudaMemcpyAsync(&h, ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
         GC_CUDA(cudaStreamSynchronize(s));
@@ -800,19 +801,22 @@ static int run(Context &C, const Problem &pb, int mode, uint64_t seed, const gc_
     GC_CUDA(cudaStreamSynchronize(s));
     if (stats) {
         int32_t total_colors = 0, maxc = -1;
+        int32_t most_rounds = rounds_single;
         if (pb.batch) {
+            // (the small graphs' rounds are not among the round kernel's)
             for (int32_t g = 0; g < G; ++g) {
                 total_colors += gcount_h[g];
                 if (gmax_h[g] > maxc) maxc = gmax_h[g];
+                if (glast_h[g] > most_rounds) most_rounds = glast_h[g];
             }
         } else {
             total_colors = h.gcount1;
             maxc = h.gmax1;
         }
-        stats->rounds = rounds_single;
+        stats->rounds = most_rounds;
         stats->ncolors = total_colors;
         stats->max_color = maxc;
-        stats->grid_blocks = static_cast<int32_t>(grid);
+        stats->grid_blocks = rest ? static_cast<int32_t>(grid) : small_grid;
         stats->block_size = block;
         stats->worklist_total = 0;
         stats->entries_scanned = 0;

@@ -261,8 +261,9 @@ struct SmallOne {
 // The cluster a single graph runs as (16 or 8 blocks, 0: none).
 int small_one_blocks();
 cudaError_t launch_small_one(const RoundParams &P, const SmallOne &A, int blocks, cudaStream_t s);
-// After launch_batch_tables: picks the small graphs and colors them (nnz: the batch's entries).
-cudaError_t launch_small_batch(const RoundParams &P, const SmallBatch &B, int64_t nnz, cudaStream_t s);
+// After launch_batch_tables: picks the small graphs and colors them (nnz: the batch's entries; *grid: the
+// blocks launched, of 256 threads).
+cudaError_t launch_small_batch(const RoundParams &P, const SmallBatch &B, int64_t nnz, cudaStream_t s, int *grid);
 
 // Launch wrappers (gc_kernels.cu).  All return the launch's cudaError_t.
 // gc_color_batch: graph table from the offset tables, graph id per vertex, graph_last = 1 (0 if empty).

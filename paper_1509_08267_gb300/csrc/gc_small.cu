@@ -701,7 +701,7 @@ cudaError_t launch_small_one(const RoundParams &P, const SmallOne &A, int blocks
                       : cudaLaunchKernelEx(&cfg, small_one_kernel<false>, P, A);
 }
 
-cudaError_t launch_small_batch(const RoundParams &P, const SmallBatch &B, int64_t nnz, cudaStream_t s) {
+cudaError_t launch_small_batch(const RoundParams &P, const SmallBatch &B, int64_t nnz, cudaStream_t s, int *grid) {
     int dev = 0, sms = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -713,7 +713,8 @@ cudaError_t launch_small_batch(const RoundParams &P, const SmallBatch &B, int64_
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, small_batch_kernel, kBatchThreads, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    small_batch_kernel<<<std::min(P.G, sms * per_sm), kBatchThreads, smem, s>>>(P, B);
+    *grid = std::min(P.G, sms * per_sm);
+    small_batch_kernel<<<*grid, kBatchThreads, smem, s>>>(P, B);
     return cudaGetLastError();
 }
 
