@@ -690,11 +690,12 @@ def main():
             # phase's four (index, fill, core rounds, write-back) and the tail phase's cluster launch in
             # deterministic mode when some vertex is past the thread bound; ordered mode and recoloring:
             # setup, counting pass, round kernel, color count (2) (smallest last adds the peeling's two:
-            # its set-up and the peeling kernel)
+            # its set-up and the peeling kernel, and deterministic mode's value keys their two digest passes)
             "gpu_launches": ((5 if mode in ("ordered", "recolor") else 7)
                              + (5 if mode == "det" and (g.max_degree > (opt.small_max_degree or 127)
                                                         or opt.core_vertices > 0) else 0)
-                             + (2 if args.priority == "sl" else 0)) * args.steps,
+                             + (2 if args.priority == "sl" else 0)
+                             + (2 if mode == "det" and args.priority != "hash" else 0)) * args.steps,
             "clocks": clk,
             **({"batched": batched} if batched is not None else {}),
             **({"served": served} if served is not None else {}),

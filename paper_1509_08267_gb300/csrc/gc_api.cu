@@ -92,6 +92,7 @@ struct Ctl {
     unsigned tail_ctl[4];  // tail phase: handed over, first round
     unsigned small_ctl[4];  // small graphs: a batch's queued and taken graphs; a cluster's losers per round
     unsigned long long small_left;  // vertices of the graphs that are not small
+    unsigned long long digest_cnt[kDigestBins];  // value keys: degrees per digest bin
     alignas(128) unsigned ord_cnt[3 * kOrdSet];  // ordered mode and peeling
     GridBar bar;
 };
@@ -639,6 +640,7 @@ static int run(Context &C, const Problem &pb, int mode, uint64_t seed, const gc_
         GC_CUDA(launch_ordered(P, pb.batch, C.col1.as<unsigned long long>(), static_cast<int>(grid), block, s));
     } else if (rest) {
     GC_CUDA(launch_setup(P, mode, pb.batch, 0, static_cast<int32_t>(n), -1, s));
+    if (mode == GC_MODE_DETERMINISTIC && priority != GC_PRIORITY_HASH) GC_CUDA(launch_digests(P, ctl->digest_cnt, s));
     GC_CUDA(launch_sort_small(P, pb.batch, 0, static_cast<int32_t>(n), s));
     GC_CUDA(cudaMemcpyAsync(&h, ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
     GC_CUDA(cudaStreamSynchronize(s));

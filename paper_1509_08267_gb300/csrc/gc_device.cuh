@@ -93,8 +93,7 @@ __device__ __forceinline__ uint32_t priority_bits(const RoundParams &P, uint32_t
         deg = c < 0 ? 0 : c;
     }
     if (P.priority != GC_PRIORITY_HASH) {
-        constexpr uint32_t kCap = (1u << 20) - 1u;
-        const uint32_t f = kCap - static_cast<uint32_t>(deg < kCap ? deg : kCap);
+        const uint32_t f = kKeyCap - static_cast<uint32_t>(deg < kKeyCap ? deg : kKeyCap);
         return (f << 11) | static_cast<uint32_t>(h >> 53);
     }
     return static_cast<uint32_t>(h >> 33);
@@ -196,15 +195,32 @@ __device__ __forceinline__ unsigned load_s16(const uint16_t *p) {
     return __ldca(reinterpret_cast<const unsigned short *>(p));
 }
 
-// 8 bits of the 31 priority bits, in their order (a <= b implies digest(a) <= digest(b)).  Hash key:
-// the top bits.  The other keys hold kCap - value (20 bits) over hash bits, with most values far
-// below the cap: a logarithmic code of the value (3 bits below the leading one), larger values first.
-__device__ __forceinline__ unsigned prio_digest(const RoundParams &P, uint32_t p31) {
-    if (P.priority == GC_PRIORITY_HASH) return p31 >> 23;
-    const uint32_t v = ((1u << 20) - 1u) - (p31 >> 11);
-    if (v < 8u) return 255u - v;
-    const int lead = 31 - __clz(static_cast<int>(v));  // 3..19
-    return 255u - (8u * static_cast<unsigned>(lead - 2) + ((v >> (lead - 3)) & 7u));
+// The table of the value keys' digests from the bins' counts (one warp; the counts and the table may
+// be shared memory).
+template <class Count>
+__device__ __forceinline__ void digest_table(const Count *cnt, DigestBin *bins, int lane) {
+    constexpr int kPer = (kDigestBins + 31) / 32;  // bins per lane, the largest values first
+    uint64_t c[kPer], sum = 0;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        const int b = kDigestBins - 1 - (lane * kPer + k);
+        c[k] = b >= 0 ? static_cast<uint64_t>(cnt[b]) : 0ull;
+        sum += c[k];
+    }
+    uint64_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint64_t y = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += y;
+    }
+    const uint64_t total = __shfl_sync(kFull, incl, 31);
+    uint64_t before = incl - sum;
+#pragma unroll 1
+    for (int k = 0; k < kPer; ++k) {
+        const int b = kDigestBins - 1 - (lane * kPer + k);
+        if (b >= 0) bins[b] = digest_range(before, c[k], total);
+        before += c[k];
+    }
 }
 
 // One parity's buffers: what a round reads, or what it writes.

@@ -1582,7 +1582,9 @@ __global__ void __launch_bounds__(256) setup_kernel(RoundParams P, int32_t v_beg
             // an isolated vertex takes color 0 in round 1 and never changes: it is final from the start
             if (MODE == GC_MODE_DETERMINISTIC) {
                 // C_1 = 0 everywhere: round 1's First Fit sees no colored neighbour
-                const uint16_t w = static_cast<uint16_t>(prio_digest(P, pv) << 1 | (d == 0 ? kFinal : 0u));
+                // (digest_store_kernel fills in a value key's digest)
+                const unsigned dig = P.priority == GC_PRIORITY_HASH ? pv >> 23 : 0u;
+                const uint16_t w = static_cast<uint16_t>(dig << 1 | (d == 0 ? kFinal : 0u));
                 P.s16a[V] = w;
                 P.s16b[V] = w;
                 P.prio[V] = pv;
@@ -1642,6 +1644,53 @@ __global__ void __launch_bounds__(256) setup_kernel(RoundParams P, int32_t v_beg
     flush_sum_u32(P.tmp + 1, st_chunks);
     if (P.list_total) flush_sum(P.list_total, st_list);
     if (P.ecnt) flush_sum(P.ecnt + pass % 3, st_ent);
+}
+
+// Value keys: the degrees of the vertices on the worklist, summed per digest bin, then their digests
+// into both state buffers.  Two passes of 6 to 8 bytes a vertex, bandwidth-bound (16M vertices: about
+// 50 us of an 8 ms coloring); a block's sums wrap at 2^32, which moves the bins' limits but not their order.
+__global__ void __launch_bounds__(256) digest_count_kernel(RoundParams P, unsigned long long *cnt) {
+    __shared__ unsigned s_cnt[kDigestBins];
+    for (int t = threadIdx.x; t < kDigestBins; t += blockDim.x) s_cnt[t] = 0u;
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    for (int64_t base = static_cast<int64_t>(blockIdx.x) * blockDim.x; base < P.n;
+         base += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        const int64_t V = base + threadIdx.x;
+        int bin = -1;
+        unsigned w = 0;
+        if (V < P.n && !(P.s16a[V] & kFinal)) {  // (isolated, malformed or already colored: FINAL)
+            const uint32_t value = kKeyCap - (P.prio[V] >> 11);
+            bin = digest_bin(value);
+            // (smallest last colors single graphs only; the other value is the degree)
+            w = P.priority == GC_PRIORITY_SMALLEST_LAST ? static_cast<unsigned>(P.rowptr[V + 1] - P.rowptr[V]) : value;
+        }
+        // one value in the whole warp (meshes): one atomic
+        int same = 0;
+        __match_all_sync(kFull, bin, &same);
+        if (same) {
+            w = __reduce_add_sync(kFull, w);
+            if (lane == 0 && bin >= 0) atomicAdd(&s_cnt[bin], w);
+        } else if (bin >= 0) {
+            atomicAdd(&s_cnt[bin], w);
+        }
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < kDigestBins; t += blockDim.x)
+        if (s_cnt[t]) atomicAdd(cnt + t, static_cast<unsigned long long>(s_cnt[t]));
+}
+
+__global__ void __launch_bounds__(256) digest_store_kernel(RoundParams P, const unsigned long long *cnt) {
+    __shared__ DigestBin s_bins[kDigestBins];
+    if (threadIdx.x < 32) digest_table(cnt, s_bins, static_cast<int>(threadIdx.x));
+    __syncthreads();
+    for (int64_t V = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; V < P.n;
+         V += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        if (P.s16a[V] & kFinal) continue;
+        const uint16_t w = static_cast<uint16_t>(key_digest24(s_bins, P.prio[V]) >> 16 << 1);  // color 0
+        P.s16a[V] = w;
+        P.s16b[V] = w;
+    }
 }
 
 // One block of kSortThreads threads: turns the (vertex block, degree) counts P.deg_hist[0, nbins)
@@ -2957,6 +3006,14 @@ cudaError_t launch_batch_tables(const RoundParams &P, const int64_t *vtx_off, co
                                 cudaStream_t s) {
     batch_tables_kernel<<<grid_for(P.G, 1, 65535), 256, 0, s>>>(P, vtx_off, edge_off, g_vbase, g_n, g_ebase, g_rbase,
                                                                 g_m);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_digests(const RoundParams &P, unsigned long long *cnt, cudaStream_t s) {
+    if (P.n <= 0) return cudaSuccess;
+    const int grid = grid_for(P.n, 256, sm_count() * 8);
+    digest_count_kernel<<<grid, 256, 0, s>>>(P, cnt);
+    digest_store_kernel<<<grid, 256, 0, s>>>(P, cnt);
     return cudaGetLastError();
 }
 

@@ -23,8 +23,8 @@
 // denser than kSmallOneRow entries a row is left to the core phase, whose 152 blocks then win.
 //
 // State word: color << 17 | 16-bit key digest << 1.  A neighbour's word minus (own color << 17) is below
-// twice the own digest exactly for an equal color and a smaller digest; equal digests (one pair in 65,536)
-// compare the full keys.
+// twice the own digest exactly for an equal color and a smaller digest; equal digests (hash key: one pair in
+// 65,536; value keys: hardly more than the pairs whose 31 priority bits are equal) compare the full keys.
 #include <algorithm>
 
 #include "gc_device.cuh"
@@ -54,8 +54,9 @@ struct SmallShared {
     unsigned at[kSmallRow + 1];  // set-up: vertices per degree, then their list positions
 };
 
-__device__ __forceinline__ uint32_t small_digest(const RoundParams &P, uint32_t p31) {
-    return P.priority == GC_PRIORITY_HASH ? p31 >> 15 : prio_digest(P, p31) << 8;
+// bins: the value keys' table, nullptr for the hash key.
+__device__ __forceinline__ uint32_t small_digest(const DigestBin *bins, uint32_t p31) {
+    return bins ? key_digest24(bins, p31) >> 8 : p31 >> 15;
 }
 
 // The full keys of two vertices of graph g: is u's smaller?
@@ -65,7 +66,7 @@ __device__ __noinline__ bool small_key_less(const RoundParams &P, const SmallGra
     for (int k = 0; k < 2; ++k) {
         const uint64_t h = vertex_hash(g.seed, static_cast<uint32_t>(x[k]));
         const int32_t d = __ldg(g.rp + x[k] + 1) - __ldg(g.rp + x[k]);
-        constexpr int32_t kCap = (1 << 20) - 1;
+        constexpr int32_t kCap = static_cast<int32_t>(kKeyCap);
         p[k] = P.priority == GC_PRIORITY_HASH
                    ? static_cast<uint32_t>(h >> 33)
                    : static_cast<uint32_t>(kCap - min(d, kCap)) << 11 | static_cast<uint32_t>(h >> 53);
@@ -94,30 +95,66 @@ __device__ __noinline__ bool small_exact(const RoundParams &P, const SmallGraph 
     return false;
 }
 
+// The same by a warp (longer rows).
+__device__ __noinline__ bool small_exact_warp(const RoundParams &P, const SmallGraph &g, SmallShared &S,
+                                              const uint32_t *cur, int32_t v, int lane) {
+    const int32_t b = __ldg(g.rp + v), e = __ldg(g.rp + v + 1);
+    bool lose = false;
+    for (int32_t j = b + lane; j < e; j += 32) {
+        const int32_t u = load_entry(P.colidx + g.e0 + j);
+        if (static_cast<uint32_t>(u) >= static_cast<uint32_t>(g.n) || u == v)
+            small_bad(P, S, g, v, j);
+        else if (cur[u] >> 17 == cur[v] >> 17)
+            lose |= small_key_less(P, g, u, v);
+    }
+    return __any_sync(kFull, lose);
+}
+
+// A row's degree, or -1 for a malformed one.
+__device__ __forceinline__ int32_t small_degree(const SmallGraph &g, int32_t v, int64_t &b) {
+    b = __ldg(g.rp + v);
+    const int64_t e = __ldg(g.rp + v + 1);
+    const bool ok = b >= 0 && b <= e && e <= g.m && (v != 0 || b == 0) && (v != g.n - 1 || e == g.m);
+    return ok ? static_cast<int32_t>(e - b) : -1;
+}
+
+// The value keys' digests of one graph (block-wide; both arrays kDigestBins long).
+__device__ void small_digests(const SmallGraph &g, DigestBin *bins, unsigned *cnt) {
+    for (int t = static_cast<int>(threadIdx.x); t < kDigestBins; t += static_cast<int>(blockDim.x)) cnt[t] = 0u;
+    __syncthreads();
+    for (int32_t v = static_cast<int32_t>(threadIdx.x); v < g.n; v += static_cast<int32_t>(blockDim.x)) {
+        int64_t b;
+        const int32_t d = small_degree(g, v, b);
+        if (d > 0) atomicAdd(&cnt[digest_bin(min(static_cast<uint32_t>(d), kKeyCap))], static_cast<unsigned>(d));
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) digest_table(cnt, bins, static_cast<int>(threadIdx.x));
+}
+
 // Set-up of one graph by the calling block: rows checked (every block of a cluster checks all of them
 // and comes to the same end), the states of all vertices, and the block's worklist: the vertices of
 // [lo, hi) with neighbours, rows up to kSmallRow at the list's front by increasing degree (a counting
 // sort: the 32 rows a warp sweeps side by side then have similar lengths), longer ones at its back.
-// Ends with a block barrier.
+// bins: room for the value keys' table and counts (key_room), or nullptr.  Ends with a block barrier.
 __device__ void small_setup(const RoundParams &P, const SmallGraph &g, SmallShared &S, uint32_t *st, uint16_t *list,
-                            int32_t cap, int32_t lo, int32_t hi, uint32_t *st2) {
+                            int32_t cap, int32_t lo, int32_t hi, uint32_t *st2, DigestBin *bins) {
     const int lane = threadIdx.x & 31;
+    if (bins) small_digests(g, bins, reinterpret_cast<unsigned *>(bins + kDigestBins));
     for (int t = static_cast<int>(threadIdx.x); t <= kSmallRow; t += static_cast<int>(blockDim.x)) S.at[t] = 0u;
     __syncthreads();
 #pragma unroll 4
     for (int32_t v = static_cast<int32_t>(threadIdx.x); v < g.n; v += static_cast<int32_t>(blockDim.x)) {
-        const int64_t b = __ldg(g.rp + v), e = __ldg(g.rp + v + 1);
-        int32_t d = 0;
-        if (!(b >= 0 && b <= e && e <= g.m && (v != 0 || b == 0) && (v != g.n - 1 || e == g.m)))
+        int64_t b;
+        int32_t d = small_degree(g, v, b);
+        if (d < 0) {
             small_bad(P, S, g, v, b);
-        else
-            d = static_cast<int32_t>(e - b);
+            d = 0;
+        }
         const uint64_t h = vertex_hash(g.seed, static_cast<uint32_t>(v));
-        constexpr int32_t kCap = (1 << 20) - 1;
-        const uint32_t p31 = P.priority == GC_PRIORITY_HASH
-                                 ? static_cast<uint32_t>(h >> 33)
-                                 : static_cast<uint32_t>(kCap - min(d, kCap)) << 11 | static_cast<uint32_t>(h >> 53);
-        const uint32_t w = small_digest(P, p31) << 1;
+        constexpr int32_t kCap = static_cast<int32_t>(kKeyCap);
+        const uint32_t p31 = bins ? static_cast<uint32_t>(kCap - min(d, kCap)) << 11 | static_cast<uint32_t>(h >> 53)
+                                  : static_cast<uint32_t>(h >> 33);
+        const uint32_t w = small_digest(bins, p31) << 1;
         st[v] = w;
         if (st2) st2[v] = w;
         if (v >= lo && v < hi && d > 0 && d <= kSmallRow) atomicAdd(&S.at[d], 1u);
@@ -291,7 +328,7 @@ __device__ __forceinline__ int32_t small_long_row(const RoundParams &P, const Sm
         if (base == 0) {
             least = __reduce_min_sync(kFull, least);
             bool lose = least < dig2;
-            if (least >> 1 == dig2 >> 1 || __any_sync(kFull, none != 0)) lose = small_exact(P, g, S, cur, v);
+            if (least >> 1 == dig2 >> 1 || __any_sync(kFull, none != 0)) lose = small_exact_warp(P, g, S, cur, v, lane);
             if (!lose) return -1;
         }
         __syncwarp();
@@ -351,10 +388,11 @@ __device__ void small_round(const RoundParams &P, const SmallGraph &g, SmallShar
 constexpr int kBatchThreads = 256;
 constexpr int kBatchBlocks = 3;  // per SM: 4 (64 registers) spill and leave little L1 for the rows, 2 idle
 
-// Dynamic shared memory: states [2][cap + 4], lists [2][cap], windows.
+// Dynamic shared memory: states [2][cap + 4], lists [2][cap], windows, a value key's table and counts.
+constexpr size_t key_room(bool value_key) { return value_key ? (sizeof(DigestBin) + 4) * kDigestBins : 0; }
 template <int THREADS>
-constexpr size_t small_smem(int32_t cap) {
-    return 12 * static_cast<size_t>(cap) + 32 + 4 * kWinWords * (THREADS / 32);
+constexpr size_t small_smem(int32_t cap, bool value_key) {
+    return 12 * static_cast<size_t>(cap) + 32 + 4 * kWinWords * (THREADS / 32) + key_room(value_key);
 }
 
 __global__ void __launch_bounds__(kBatchThreads, kBatchBlocks) small_batch_kernel(const __grid_constant__ RoundParams P,
@@ -368,6 +406,10 @@ __global__ void __launch_bounds__(kBatchThreads, kBatchBlocks) small_batch_kerne
     uint16_t *list[2] = {reinterpret_cast<uint16_t *>(st[1] + cap + 4),
                          reinterpret_cast<uint16_t *>(st[1] + cap + 4) + cap};
     unsigned *win = reinterpret_cast<unsigned *>(list[1] + cap) + kWinWords * wib;
+    DigestBin *bins = P.priority == GC_PRIORITY_HASH
+                          ? nullptr
+                          : reinterpret_cast<DigestBin *>(reinterpret_cast<unsigned *>(list[1] + cap) +
+                                                          kWinWords * (kBatchThreads / 32));
     const unsigned count = __ldcg(B.queued);
     if (threadIdx.x < 2) st[threadIdx.x][cap] = kNobody32;
     for (;;) {
@@ -388,7 +430,7 @@ __global__ void __launch_bounds__(kBatchThreads, kBatchBlocks) small_batch_kerne
         g.rp = P.rowptr + __ldg(P.g_rbase + g.g);
         g.seed = P.g_seed ? __ldg(P.g_seed + g.g) : P.seed;
         g.ci_len = P.ci_len;
-        small_setup(P, g, S, st[1], list[1], cap, 0, g.n, st[0]);
+        small_setup(P, g, S, st[1], list[1], cap, 0, g.n, st[0], bins);
         if (threadIdx.x == 0) S.stop = S.bad;
         __syncthreads();
         int pass = 1;
@@ -521,6 +563,10 @@ __global__ void __launch_bounds__(kOneThreads, 1) small_one_kernel(const __grid_
     uint16_t *list[2] = {reinterpret_cast<uint16_t *>(st[1] + cap + 4),
                          reinterpret_cast<uint16_t *>(st[1] + cap + 4) + cap};
     unsigned *win = reinterpret_cast<unsigned *>(list[1] + cap) + kWinWords * wib;
+    DigestBin *bins = P.priority == GC_PRIORITY_HASH
+                          ? nullptr
+                          : reinterpret_cast<DigestBin *>(reinterpret_cast<unsigned *>(list[1] + cap) +
+                                                          kWinWords * (kOneThreads / 32));
     SmallGraph g;
     g.g = 0;
     g.n = P.n;
@@ -555,7 +601,7 @@ __global__ void __launch_bounds__(kOneThreads, 1) small_one_kernel(const __grid_
         small_cluster_sync();
     else
         __syncthreads();
-    small_setup(P, g, S, st[1], list[1], cap, lo, hi, CLUSTER ? nullptr : st[0]);
+    small_setup(P, g, S, st[1], list[1], cap, lo, hi, CLUSTER ? nullptr : st[0], bins);
     if (threadIdx.x == 0) S.stop = S.bad;
     if (CLUSTER) {
         // the exchange buffers start with the block's own vertices' states; before the barrier, because
@@ -658,9 +704,9 @@ __global__ void __launch_bounds__(kOneThreads, 1) small_one_kernel(const __grid_
 }
 
 template <bool CLUSTER>
-cudaError_t one_config(int32_t cap, int blocks, cudaLaunchConfig_t &cfg, cudaLaunchAttribute *at) {
+cudaError_t one_config(int32_t cap, bool value_key, int blocks, cudaLaunchConfig_t &cfg, cudaLaunchAttribute *at) {
     const void *fn = reinterpret_cast<const void *>(&small_one_kernel<CLUSTER>);
-    const size_t smem = small_smem<kOneThreads>(cap);
+    const size_t smem = small_smem<kOneThreads>(cap, value_key);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e == cudaSuccess && blocks > 8) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     cfg = cudaLaunchConfig_t{};
@@ -683,7 +729,7 @@ int small_one_blocks() {
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute at[1];
         int n = 0;
-        if (one_config<true>(kSmallOneVertices, blocks, cfg, at) == cudaSuccess &&
+        if (one_config<true>(kSmallOneVertices, true, blocks, cfg, at) == cudaSuccess &&
             cudaOccupancyMaxActiveClusters(&n, small_one_kernel<true>, &cfg) == cudaSuccess && n >= 1)
             return blocks;
         cudaGetLastError();
@@ -694,7 +740,9 @@ int small_one_blocks() {
 cudaError_t launch_small_one(const RoundParams &P, const SmallOne &A, int blocks, cudaStream_t s) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at[1];
-    cudaError_t e = blocks > 1 ? one_config<true>(A.cap, blocks, cfg, at) : one_config<false>(A.cap, 1, cfg, at);
+    const bool value_key = P.priority != GC_PRIORITY_HASH;
+    cudaError_t e = blocks > 1 ? one_config<true>(A.cap, value_key, blocks, cfg, at)
+                               : one_config<false>(A.cap, value_key, 1, cfg, at);
     if (e != cudaSuccess) return e;
     cfg.stream = s;
     return blocks > 1 ? cudaLaunchKernelEx(&cfg, small_one_kernel<true>, P, A)
@@ -707,7 +755,7 @@ cudaError_t launch_small_batch(const RoundParams &P, const SmallBatch &B, int64_
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     small_queue_kernel<<<1, kQueueThreads, 0, s>>>(P, B, std::max<int64_t>(int64_t{1} << 14, 4 * nnz / sms));
-    const size_t smem = small_smem<kBatchThreads>(kSmallBatchVertices);
+    const size_t smem = small_smem<kBatchThreads>(kSmallBatchVertices, P.priority != GC_PRIORITY_HASH);
     e = cudaFuncSetAttribute(small_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, small_batch_kernel, kBatchThreads, smem);
