@@ -338,6 +338,41 @@ __device__ __noinline__ bool det_small_exact(const RoundParams &P, const DetStat
     return __any_sync(kFull, lose);
 }
 
+// The same by the vertex's own thread, four entries at a time: for rounds in which many rows of a warp
+// tie.  Smallest last ties by nature -- neighbours are removed in levels next to each other -- and a
+// warp that took its 32 rows one after another made such rounds three times as long (smallest last, whole
+// call: 2,000^2 grid 949 ms, 315 with this; 250^2 grid 11.1 and 3.5).
+template <bool BATCH>
+__device__ __noinline__ bool det_small_exact_lane(const RoundParams &P, const DetState &S, int32_t V) {
+    const Row r = load_row<BATCH>(P, V);
+    const unsigned own = load_s16(S.s16 + V);
+    const int32_t cv = det_color(S, V, own);
+    const uint32_t pv = __ldg(P.prio + V);
+    bool lose = false;
+    for (int64_t j = r.b; j < r.e && !lose; j += 4) {
+        int32_t ul[4], U[4];
+        bool same[4];
+        uint32_t p[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) ul[q] = j + q < r.e ? load_entry(P.colidx + j + q) : 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            U[q] = j + q < r.e ? neighbour(P, r, ul[q], j + q) : -1;
+            same[q] = U[q] >= 0 && color16(load_s16(S.s16 + U[q])) == color16(own);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (same[q] && color16(own) == kSat7) same[q] = det_color(S, U[q]) == cv;
+            p[q] = same[q] ? __ldca(P.prio + U[q]) : 0u;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (same[q])
+                lose |= key_less_in(p[q], pv, static_cast<uint32_t>(ul[q]), static_cast<uint32_t>(r.lv), P, V);
+    }
+    return lose;
+}
+
 // The row of a vertex of degree <= T1 <= 127, one thread: eight entries a step from the aligned
 // group of eight that holds the row's first entry (a whole 32-byte sector per load), the next step's
 // entries loaded before the current step's eight gathers are consumed.  W: words of the color window
@@ -449,10 +484,20 @@ __device__ __forceinline__ bool det_small(const RoundParams &P, const DetState &
             nc = min(first_free_words<4>(m), deg);
         }
     }
-    for (unsigned open = __ballot_sync(kFull, state == 2); open; open &= open - 1u) {
-        const int l = __ffs(static_cast<int>(open)) - 1;
-        const bool lost = det_small_exact<BATCH>(P, cur, __shfl_sync(kFull, V, l), lane);
-        if (lane == l) state = lost ? 1 : 0;
+    unsigned open = __ballot_sync(kFull, state == 2);
+    if (open != 0u) {
+        // all at once, a row's steps long, or one after another, a step or two each: whichever chain is the
+        // shorter (lanes already at half or a quarter as many rows: 40^3 stencil, hash key, 5% and 55% slower)
+        const unsigned longest = __reduce_max_sync(kFull, state == 2 ? static_cast<unsigned>(deg) : 0u);
+        if (static_cast<unsigned>(__popc(open)) > (longest + 3u) / 4u) {
+            if (state == 2) state = det_small_exact_lane<BATCH>(P, cur, V) ? 1 : 0;
+            open = 0u;
+        }
+        for (; open; open &= open - 1u) {
+            const int l = __ffs(static_cast<int>(open)) - 1;
+            const bool lost = det_small_exact<BATCH>(P, cur, __shfl_sync(kFull, V, l), lane);
+            if (lane == l) state = lost ? 1 : 0;
+        }
     }
     const bool lose = state == 1;
     if (in) {
