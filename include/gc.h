@@ -165,7 +165,9 @@ typedef struct gc_stats {
     int32_t block_size;        /* threads per block of the round kernel */
     int64_t *round_reads;      /* caller array or NULL: adjacency entries the round kernel read in each
                                   round (GC_FLAG_STATS); they sum to entries_scanned */
-    int32_t reserved[4];
+    int32_t core_round;        /* deterministic mode: first round of the shared-memory rounds (gc_options'
+                                  core_vertices), 0 if they did not run */
+    int32_t reserved[3];
 } gc_stats;
 
 /*
@@ -353,7 +355,9 @@ struct gc_server_stats {
     int32_t resident;            /* requests currently resident on the device */
     int32_t queued;              /* requests waiting for admission */
     int64_t failed;              /* requests that ended with a device error (their pool was reset) */
-    int32_t reserved[4];
+    int32_t core_handovers;      /* launches that handed the resident batch to the shared-memory rounds */
+    int32_t core_round;          /* the pool's round number at the latest of them */
+    int32_t reserved[2];
 };
 
 /* Creates the worker thread and the pool of cfg->mode. Errors: INVALID_ARG, OOM, CUDA. */

@@ -72,7 +72,7 @@ class _Stats(ctypes.Structure):
                 ("round_ns", ctypes.c_void_p),
                 ("worklist_total", ctypes.c_int64), ("entries_scanned", ctypes.c_int64), ("kernel_ms", ctypes.c_float),
                 ("setup_ms", ctypes.c_float), ("grid_blocks", ctypes.c_int32), ("block_size", ctypes.c_int32),
-                ("round_reads", ctypes.c_void_p), ("reserved", ctypes.c_int32 * 4)]
+                ("round_reads", ctypes.c_void_p), ("core_round", ctypes.c_int32), ("reserved", ctypes.c_int32 * 3)]
 
 
 class _ServerConfig(ctypes.Structure):
@@ -86,7 +86,8 @@ class _ServerStats(ctypes.Structure):
                 ("rounds_run", ctypes.c_int64), ("vertices_colored", ctypes.c_int64),
                 ("edges_colored", ctypes.c_int64), ("p50_ms", ctypes.c_double), ("p99_ms", ctypes.c_double),
                 ("busy_s", ctypes.c_double), ("wall_s", ctypes.c_double), ("resident", ctypes.c_int32),
-                ("queued", ctypes.c_int32), ("failed", ctypes.c_int64), ("reserved", ctypes.c_int32 * 4)]
+                ("queued", ctypes.c_int32), ("failed", ctypes.c_int64), ("core_handovers", ctypes.c_int32),
+                ("core_round", ctypes.c_int32), ("reserved", ctypes.c_int32 * 2)]
 
 
 _lib = None
@@ -259,6 +260,7 @@ class Stats:
     wl_degsum: np.ndarray = field(default_factory=lambda: np.zeros(0, np.int64))
     round_ns: np.ndarray = field(default_factory=lambda: np.zeros(0, np.int64))
     round_reads: np.ndarray = field(default_factory=lambda: np.zeros(0, np.int64))
+    core_round: int = 0  # first round of the shared-memory rounds, 0: they did not run
 
 
 def _stats_arrays(round_cap: int):
@@ -373,7 +375,7 @@ def _color_one(rowptr, colidx, mode, seed, out, options, stats, round_cap, color
         k = min(st.rounds, round_cap)
         s = Stats(st.rounds, st.ncolors, st.max_color, st.worklist_total, st.entries_scanned, st.kernel_ms,
                   st.setup_ms, st.grid_blocks, st.block_size, wl[:k].copy(), ds[:k].copy(), rn[:k].copy(),
-                  rr[:k].copy())
+                  rr[:k].copy(), st.core_round)
     return Result(out_k if out_k is not None else out, int(nc.value), int(rd.value), s)
 
 
@@ -405,7 +407,7 @@ def color_batch(vtx_off, edge_off, rowptr, colidx, mode="det", seed: int = 0, ou
         k = min(st.rounds, round_cap)
         res = res + (Stats(st.rounds, st.ncolors, st.max_color, st.worklist_total, st.entries_scanned, st.kernel_ms,
                            st.setup_ms, st.grid_blocks, st.block_size, wl[:k].copy(), ds[:k].copy(),
-                           rn[:k].copy(), rr[:k].copy()),)
+                           rn[:k].copy(), rr[:k].copy(), st.core_round),)
     return res
 
 

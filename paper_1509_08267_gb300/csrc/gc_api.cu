@@ -416,6 +416,7 @@ static int color_small(Context &C, int32_t n, const int32_t *rowptr, const int32
         stats->rounds = rounds;
         stats->ncolors = res[3];
         stats->max_color = res[4];
+        stats->core_round = 0;
         stats->grid_blocks = blocks;
         stats->block_size = 1024;
         stats->worklist_total = 0;
@@ -818,6 +819,7 @@ static int run(Context &C, const Problem &pb, int mode, uint64_t seed, const gc_
         stats->rounds = most_rounds;
         stats->ncolors = total_colors;
         stats->max_color = maxc;
+        stats->core_round = h.core_go ? static_cast<int32_t>(h.core_m[3]) : 0;
         stats->grid_blocks = rest ? static_cast<int32_t>(grid) : small_grid;
         stats->block_size = block;
         stats->worklist_total = 0;
@@ -982,6 +984,7 @@ static int color_batch(int32_t G, const int64_t *vtx_off, const int64_t *edge_of
     if (G == 0) {
         if (stats) {
             std::memset(stats, 0, offsetof(gc_stats, round_cap));
+            stats->core_round = 0;
             stats->max_color = -1;
         }
         return GC_OK;

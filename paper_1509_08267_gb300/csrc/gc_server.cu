@@ -192,6 +192,7 @@ struct gc_server {
     uint64_t next_id = 1;
     // statistics
     int64_t submitted = 0, completed = 0, rejected = 0, failed = 0, rounds_run = 0, v_done = 0, e_done = 0;
+    int32_t core_handovers = 0, core_round = 0;
     std::vector<double> latencies;
     double t_create = 0, busy = 0;
     int fatal = GC_OK;
@@ -636,6 +637,10 @@ bool engine_step(gc_server *s, Engine &E, std::vector<Request *> &adm, bool queu
     {
         std::lock_guard<std::mutex> lk(s->mu);
         s->rounds_run += ran;
+        if (core && h.core_go) {
+            s->core_handovers += 1;
+            s->core_round = static_cast<int32_t>(h.core_m[3]);
+        }
         for (auto it = E.resident.begin(); it != E.resident.end();) {
             if (E.h_glast[(*it)->slot] < E.next_pass) {
                 fin.push_back(*it);
@@ -1009,6 +1014,8 @@ int gc_server_stats(gc_server *s, struct gc_server_stats *out) {
     out->rejected = s->rejected;
     out->failed = s->failed;
     out->rounds_run = s->rounds_run;
+    out->core_handovers = s->core_handovers;
+    out->core_round = s->core_round;
     out->vertices_colored = s->v_done;
     out->edges_colored = s->e_done;
     if (!s->latencies.empty()) {
