@@ -688,12 +688,14 @@ def main():
             "e2e": e2e,
             # setup, degree sort (2), expand, round kernel, color count (2) per coloring, plus the core
             # phase's four (index, fill, core rounds, write-back) and the tail phase's cluster launch in
-            # deterministic mode when some vertex is past the thread bound; ordered mode and recoloring:
+            # deterministic mode when some vertex is past the thread bound (or the graph is small and
+            # dense); ordered mode and recoloring:
             # setup, counting pass, round kernel, color count (2) (smallest last adds the peeling's two:
             # its set-up and the peeling kernel, and deterministic mode's value keys their two digest passes)
             "gpu_launches": ((5 if mode in ("ordered", "recolor") else 7)
                              + (5 if mode == "det" and (g.max_degree > (opt.small_max_degree or 127)
-                                                        or opt.core_vertices > 0) else 0)
+                                                        or opt.core_vertices > 0
+                                                        or (g.n <= 16384 and g.nnz > 64 * g.n)) else 0)
                              + (2 if args.priority == "sl" else 0)
                              + (2 if mode == "det" and args.priority != "hash" else 0)) * args.steps,
             "clocks": clk,

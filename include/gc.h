@@ -133,7 +133,8 @@ typedef struct gc_options {
                                   remaining rounds run with every worklist vertex's color in shared memory
                                   (same results).  0 = the most one block's shared memory holds (about
                                   200k on GB300: one byte and one bit per vertex) if some vertex's degree is
-                                  past small_max_degree, else never; < 0 = never */
+                                  past small_max_degree or the call has at most 16,384 vertices with more
+                                  than 64 entries on average, else never; < 0 = never */
     int32_t core_entries;      /* deterministic mode: the most adjacency entries the shared-memory rounds take
                                   (their rows are rebuilt once, at the hand-over); 0 = min(nnz, 2^27).  Above
                                   2^27 it is clamped.  Only a graph with more entries than this counts its

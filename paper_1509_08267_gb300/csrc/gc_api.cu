@@ -664,8 +664,14 @@ static int run(Context &C, const Problem &pb, int mode, uint64_t seed, const gc_
     // a few dozen entries one at a time (~200 instructions a row) and its set-up re-reads every row,
     // while the round kernel takes a row per thread (ER n = 50,000 degree 24: 300 us against 508 with
     // the core; stencil 60 x 50 x 40: 375 against 826; ER n = 10^6 degree 32: 1.45 ms against 1.68;
-    // with hubs the core wins: R-MAT n = 150,000 1.43 ms against 2.02).
-    if (mode == GC_MODE_DETERMINISTIC && compact && core_opt >= 0 && (core_opt > 0 || n_items > 0) && pb.nnz > 0) {
+    // with hubs the core wins: R-MAT n = 150,000 1.43 ms against 2.02).  Small graphs of long rows (the
+    // small-graph kernels' vertices at most, denser than they take) have the core all the same: their rows
+    // keep few of the round kernel's threads busy, and each of those for long (20 cliques of 120: 0.98 ms
+    // against 1.93, 100 of them 1.59 and 2.25; ER degree about 90, n = 2,000 0.41 and 0.65, n = 8,000 0.50
+    // and 0.53, n = 16,000 0.59 and 0.53).
+    const bool core_dense = n <= kSmallOneVertices && pb.nnz > kSmallOneRow * n;
+    if (mode == GC_MODE_DETERMINISTIC && compact && core_opt >= 0 && pb.nnz > 0 &&
+        (core_opt > 0 || n_items > 0 || core_dense)) {
         if (C.core_max_v == 0) {
             const int32_t cm = core_max_vertices();
             C.core_max_v = cm > 0 ? cm : -1;

@@ -49,3 +49,11 @@ def test_a_servers_pool_hands_over_in_early_and_late_rounds(gclib):
             seen.append(st["core_round"])
     # the pool's round numbers go on from request to request: both sides of the fused first round's limit
     assert seen == sorted(set(seen)) and seen[0] <= 63 < seen[-1]
+
+
+@pytest.mark.parametrize("make, core", [(lambda: gg.er(2000, 90.0, 3), True), (lambda: gg.er(16384, 66.0, 3), True),
+                                        (lambda: gg.er(16385, 66.0, 3), False), (lambda: gg.er(16384, 60.0, 3), False)])
+def test_small_graphs_of_long_rows_take_it(gclib, make, core):
+    g = make()
+    assert g.max_degree <= 127
+    assert _core_round(gclib, g) == (1 if core else 0)
