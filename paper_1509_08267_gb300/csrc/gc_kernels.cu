@@ -252,32 +252,12 @@ __device__ __forceinline__ void det_write(const DetState &cur, const DetState &n
     if (!lose) det_store(cur, V, cv, dig, true);
 }
 
-// Least color >= start absent from the row's neighbours (warp-cooperative; mex <= deg(v) bounds it).
-template <bool BATCH>
-__device__ int32_t det_mex_from(const RoundParams &P, const DetState &S, const Row &r, unsigned *win, int lane,
-                                int32_t start) {
-    for (int32_t base = start;; base += 32 * kAccWords) {
-        if (lane < kAccWords) win[lane] = 0;
-        __syncwarp();
-        for (int64_t j = r.b + lane; j < r.e; j += 32) {
-            const int32_t ul = __ldg(P.colidx + j);
-            if (static_cast<uint32_t>(ul) >= static_cast<uint32_t>(r.ng)) continue;
-            const int32_t c = det_color(S, r.vbase + ul) - base;
-            if (static_cast<unsigned>(c) < 32u * kAccWords) atomicOr(&win[c >> 5], 1u << (c & 31));
-        }
-        __syncwarp();
-        int32_t res = -1;
-#pragma unroll 1
-        for (int w = 0; w < kAccWords; ++w) {
-            const unsigned x = win[w];
-            if (~x) {
-                res = base + 32 * w + __ffs(~x) - 1;
-                break;
-            }
-        }
-        __syncwarp();
-        if (res >= 0) return res;
-    }
+// The same in the deterministic mode's state (inlined, four entries a lane: a call, or eight, makes the
+// round kernel spill twice as much around its main loop).
+__device__ __forceinline__ int32_t det_mex_from(const int32_t *colidx, const DetState &S, const Row &r, unsigned *win,
+                                                int lane, int32_t start) {
+    return mex_rescan<4>(colidx, r, win, lane, start,
+                         [&](const int32_t (&U)[4], int32_t (&c)[4]) { det_colors<4>(S, U, c); });
 }
 
 // Does a neighbour (local id ul, global id U) of equal color have the smaller key?  pv: the
@@ -735,7 +715,7 @@ __device__ __forceinline__ void det_finish(const RoundParams &P, const DetState 
         const int l = __ffs(need) - 1;
         need &= need - 1;
         Row rl = load_row<BATCH>(P, __shfl_sync(kFull, V, l));
-        const int32_t x = det_mex_from<BATCH>(P, S, rl, win, lane, 32 * kAccWords);
+        const int32_t x = det_mex_from(P.colidx, S, rl, win, lane, 32 * kAccWords);
         if (lane == l) nc = x;
     }
     if (fin) {
@@ -878,7 +858,7 @@ __device__ void det_item(const RoundParams &P, const DetState &S, const DetState
     int32_t nc = cv;
     if (lose) {
         nc = first_free(lo0, lo1, win);
-        if (nc < 0) nc = det_mex_from<BATCH>(P, S, load_row<BATCH>(P, V), win, lane, 32 * kAccWords);
+        if (nc < 0) nc = det_mex_from(P.colidx, S, load_row<BATCH>(P, V), win, lane, 32 * kAccWords);
     }
     if (lane == 0) det_write(S, N, V, lose, cv, nc, dig);
     if (!lose) return;
@@ -2474,28 +2454,14 @@ __device__ __forceinline__ void ord_mid(const RoundParams &P, unsigned long long
     }
 }
 
-// Least color >= start absent from the row's colored neighbours (warp-cooperative).
-template <bool BATCH>
-__device__ int32_t ord_mex_from(const RoundParams &P, const unsigned long long *W, const Row &r, unsigned *win, int lane,
-                                int32_t start) {
-    for (int32_t base = start;; base += 32 * kAccWords) {
-        if (lane < kAccWords) win[lane] = 0;
-        __syncwarp();
-        for (int64_t j = r.b + lane; j < r.e; j += 32) {
-            const int32_t ul = __ldg(P.colidx + j);
-            if (static_cast<uint32_t>(ul) >= static_cast<uint32_t>(r.ng)) continue;
-            const int32_t x = ord_color(__ldcg(W + r.vbase + ul));
-            if (x >= base && x - base < 32 * kAccWords) atomicOr(&win[(x - base) >> 5], 1u << ((x - base) & 31));
-        }
-        __syncwarp();
-        const unsigned w = lane < kAccWords ? win[lane] : ~0u;
-        const unsigned open = __ballot_sync(kFull, ~w != 0u);
-        if (open) {
-            const int l = __ffs(static_cast<int>(open)) - 1;
-            return base + 32 * l + __ffs(static_cast<int>(~__shfl_sync(kFull, w, l))) - 1;
-        }
-        __syncwarp();
-    }
+// The same in the ordered mode's words (colored neighbours).
+template <int PER>
+__device__ __forceinline__ int32_t ord_mex_from(const int32_t *colidx, const unsigned long long *W, const Row &r,
+                                                unsigned *win, int lane, int32_t start) {
+    return mex_rescan<PER>(colidx, r, win, lane, start, [&](const int32_t (&U)[PER], int32_t (&c)[PER]) {
+#pragma unroll
+        for (int q = 0; q < PER; ++q) c[q] = U[q] >= 0 ? ord_color(__ldcg(W + U[q])) : -1;
+    });
 }
 
 // One work item of a larger ready vertex (one warp).  Colors of colored neighbours go into the window
@@ -2587,7 +2553,7 @@ __device__ void ord_item(const RoundParams &P, unsigned long long *W, int4 it, u
     int32_t nc = first_free(lo0, lo1, win);
     // every neighbour with a larger key is still uncolored, so the whole row's colors are the
     // smaller-key neighbours' colors
-    if (nc < 0) nc = ord_mex_from<BATCH>(P, W, load_row<BATCH>(P, V), win, lane, 32 * kAccWords);
+    if (nc < 0) nc = ord_mex_from<BATCH ? 4 : 8>(P.colidx, W, load_row<BATCH>(P, V), win, lane, 32 * kAccWords);
     if (lane == 0) {
         ord_paint(P, W, V, nc);
         if constexpr (BATCH) note_graph_round(P, r.g, pass);
