@@ -129,17 +129,11 @@ __device__ void core_init_vertex(const RoundParams &P, const CoreParams &Q, int3
     Q.cex[Q.max_v + local] = c;
     Q.c8[local] = static_cast<uint8_t>(sat8(c));
     Q.c8[Q.max_v + local] = static_cast<uint8_t>(sat8(c));
-    bool sat = sat8(c) == kSat8;
     const uint4 z = make_uint4(0, 0, 0, 0);
 #pragma unroll
     for (int w = 0; w < 32; w += 4) stcg4(rec + w, z);
 #pragma unroll
-    for (int w = 0; w < kAccWords; w += 4) {
-        const uint4 x = fin_src ? ldcg4(fin_src + w) : z;
-        stcg4(rec + kAccFin + w, x);
-        sat |= (w == 4 && x.w >> 31) || (w >= 8 && (x.x | x.y | x.z | x.w) != 0u);  // colors 255..511
-    }
-    if (sat) Q.tail[kTailSat] = 1u;
+    for (int w = 0; w < kAccWords; w += 4) stcg4(rec + kAccFin + w, fin_src ? ldcg4(fin_src + w) : z);
     const uint64_t lp = reinterpret_cast<uint64_t>(list);
     stcg4(rec + kCoreOffLo, make_uint4(static_cast<unsigned>(off), static_cast<unsigned>(off >> 32),
                                        static_cast<unsigned>(deg), static_cast<unsigned>(V)));
@@ -280,7 +274,6 @@ __global__ void __launch_bounds__(kFillThreads) core_fill_kernel(RoundParams P, 
                         flo |= 1ull << c;
                     else if (static_cast<unsigned>(c) < 32u * kAccWords)
                         atomicOr(&wfin[c >> 5], 1u << (c & 31));
-                    if (c >= static_cast<int32_t>(kSat8)) Q.tail[kTailSat] = 1u;
                 } else if (static_cast<unsigned>(loc[q]) < m) {
                     keepm |= 1u << q;
                     bool smaller;
@@ -512,43 +505,39 @@ __device__ __forceinline__ void consume_step(const Shared &S, const int32_t (&e)
     }
 }
 
-// Rounds past 255: the `cnt` entries of a piece with saturated neighbours looked at again for exactly
-// those: lane w returns word w of the window of their colors (255..511); the conflict.  Eight entries a
-// lane and step, their exact colors in flight together and marked in the warp's `seen` bytes (empty before
-// and after).  Entry by entry, with a vote and a shuffle each, a clique of 1,000 took 36.0 ms, 25.9 with
-// this; served 38.0 and 28.3.
-__device__ __noinline__ unsigned saturated_piece(const CoreParams &Q, const Shared &S, const Piece &p, int32_t cnt,
-                                                 const int32_t *cex_cur, int32_t cv, uint8_t *seen, int lane,
-                                                 bool &conflict) {
+// Rounds past 255: the `cnt` entries of a piece with saturated neighbours (row: its part of the pool, v: its
+// vertex, color cv) looked at again for exactly those: lane w returns word w of the window of their colors
+// (255..511), lane 0 whether one of them is a conflict.  Four entries a lane and step, their exact colors in
+// flight together and marked in the warp's `seen` bytes (empty before and after).  Entry by entry, with a
+// vote and a shuffle each, a clique of 1,000 took 36.0 ms, 16.5 with this; served 38.0 and 20.  Inlined, and
+// no more than four entries: a call, or eight, makes the rounds' own loop spill (R-MAT n = 2^20: 4.83 ms
+// with the old loop as a call, 4.70 with this, 5.0 with either).
+__device__ __forceinline__ unsigned saturated_piece(const int32_t *row, int32_t cnt, int32_t v, const int32_t *cex_cur,
+                                                 int32_t cv, uint8_t *seen) {
+    extern __shared__ __align__(16) unsigned char s_dyn[];  // the colors (core_round_kernel)
+    const int lane = threadIdx.x & 31;
     constexpr int kSat = static_cast<int>(kSat8);
     bool at255 = false, same = false;
-    for (int32_t j0 = 0; j0 < cnt; j0 += 256) {
-        int32_t e[8], c[8];
+    for (int32_t j0 = 0; j0 < cnt; j0 += 128) {
+        const int32_t j = j0 + 4 * lane;
+        int4 x = make_int4(v, v, v, v);
+        if (j < cnt) x = __ldcg(reinterpret_cast<const int4 *>(row + j));
+        const int32_t e[4] = {x.x, x.y, x.z, x.w};
+        int32_t c[4];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int32_t j = j0 + 128 * h + 4 * lane;
-            int4 x = make_int4(p.v, p.v, p.v, p.v);
-            if (j < cnt) x = __ldcg(reinterpret_cast<const int4 *>(Q.pool + p.off + j));
-            e[4 * h] = x.x;
-            e[4 * h + 1] = x.y;
-            e[4 * h + 2] = x.z;
-            e[4 * h + 3] = x.w;
-        }
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
+        for (int q = 0; q < 4; ++q) {
             const uint32_t id = static_cast<uint32_t>(e[q]) & ~kCoreSmaller;
-            c[q] = S.color8(id) == kSat8 ? __ldcg(cex_cur + id) : -1;
+            c[q] = s_dyn[id] == kSat8 ? __ldcg(cex_cur + id) : -1;
         }
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
+        for (int q = 0; q < 4; ++q) {
             same |= e[q] < 0 && c[q] == cv;
             at255 |= c[q] == kSat;
             if (c[q] > kSat && c[q] < 32 * kAccWords) seen[c[q] - kSat - 1] = 1;
         }
     }
-    conflict |= same;
     __syncwarp();
-    unsigned word = 0;
+    unsigned word = __any_sync(kFull, same) && lane == 0 ? 1u : 0u;
     for (int w = 0; w < kSeen / 32; ++w) {
         const unsigned b = __ballot_sync(kFull, seen[32 * w + lane] != 0);
         if (lane == kSeen / 32 + w) word = b;
@@ -596,7 +585,6 @@ __device__ __forceinline__ void flush_pending(const CoreParams &Q, const Pending
         if (m2) b2 = atomicAdd(cn + 4, static_cast<unsigned>(__popc(m2)));
     }
     const unsigned n8 = sat8(pd.color);
-    if (act && n8 == kSat8) Q.tail[kTailSat] = 1u;
     if (act) {
         Q.cex[nxt * Q.max_v + v] = pd.color;
         Q.c8[nxt * Q.max_v + v] = static_cast<uint8_t>(n8);
@@ -686,10 +674,7 @@ struct ManyShared {
 // with the register windows.  R-MAT-22 18.05 -> 15.9 ms with four entries per lane and step (eight:
 // the same there, 1-5% slower on smaller graphs), 2,048-entry pieces (1,024: 6% slower, 4,096: 1%
 // faster there, 3% slower on smaller graphs) and 24 warps (32: 2-6% slower).
-// SAT: some core vertex or final neighbour has a color of 255 or more (kTailSat), which the bytes do not
-// tell apart.  Without one -- nearly always -- neither those colors nor a full window can occur, and the
-// code for them is left out: calls in this loop make it spill (R-MAT n = 2^20: 4.85 -> 5.26 ms).
-template <bool BATCH, bool MANY, bool SAT>
+template <bool BATCH, bool MANY>
 __device__ void core_stream(const RoundParams &P, const CoreParams &Q, const Shared &S, const int32_t *cex_cur,
                             PieceCursor &cur, const int32_t *list, unsigned nact, unsigned nv, int pass,
                             const DetState &st_r0, unsigned *cn, unsigned nw, int lane, uint8_t *seen, unsigned *wfin,
@@ -731,7 +716,7 @@ __device__ void core_stream(const RoundParams &P, const CoreParams &Q, const Sha
         const unsigned own8 = S.color8(static_cast<uint32_t>(p.v));  // own color (never final on the worklist)
         // the conflict test's target: the key bit and the vertex's 8-bit color (never matched when it
         // is saturated; those are compared exactly)
-        const uint32_t tgt = kCoreSmaller | (SAT && own8 == kSat8 ? 0x1000u : own8);
+        const uint32_t tgt = kCoreSmaller | (own8 == kSat8 ? 0x1000u : own8);
         // a piece drops its FINAL neighbours in place once the worklist has lost half of its vertices
         // since the piece last did (its `flags` field records that worklist size): more often costs
         // more in writes than it saves in reads (a quarter: 1% slower on R-MAT-22; never: 25%)
@@ -795,13 +780,14 @@ __device__ void core_stream(const RoundParams &P, const CoreParams &Q, const Sha
                         reinterpret_cast<int2 *>(Q.pieces + pidx)[1] =
                             make_int2(static_cast<int32_t>(kept_total), static_cast<int32_t>(nv));
                 }
-                if constexpr (SAT) {
+                if (pass > static_cast<int>(kSat8)) {
                     const bool sat = __shfl_sync(kFull, rw, kSeen / 32 - 1) >> 31;
                     if (lane == kSeen / 32 - 1) rw &= 0x7fffffffu;
                     if (sat) {
-                        const int32_t cv = __ldcg(cex_cur + p.v);
-                        rw |= saturated_piece(Q, S, p, compact ? static_cast<int32_t>(kept_total) : p.cnt, cex_cur,
-                                              cv, seen, lane, conflict);
+                        const unsigned x = saturated_piece(Q.pool + p.off, compact ? static_cast<int32_t>(kept_total) : p.cnt,
+                                                           p.v, cex_cur, __ldcg(cex_cur + p.v), seen);
+                        conflict |= lane == 0 && x != 0u;
+                        rw |= lane == 0 ? 0u : x;
                     }
                 }
                 bool lose = __any_sync(kFull, conflict), finish = true;
@@ -833,7 +819,7 @@ __device__ void core_stream(const RoundParams &P, const CoreParams &Q, const Sha
                     int32_t nc;
                     if (lose) {
                         const unsigned fm = __ballot_sync(kFull, lane < kAccWords && ~tw != 0u);
-                        if (!SAT || fm) {
+                        if (fm) {
                             const int l = __ffs(fm) - 1;
                             nc = 32 * l + __ffs(~__shfl_sync(kFull, tw, l)) - 1;
                         } else {
@@ -844,7 +830,7 @@ __device__ void core_stream(const RoundParams &P, const CoreParams &Q, const Sha
                             *reinterpret_cast<uint2 *>(seen + 8 * lane) = make_uint2(0u, 0u);
                         }
                     } else {  // a winner keeps its color
-                        nc = SAT && own8 == kSat8 ? __ldcg(cex_cur + p.v) : static_cast<int32_t>(own8);
+                        nc = own8 == kSat8 ? __ldcg(cex_cur + p.v) : static_cast<int32_t>(own8);
                     }
                     if (P.stats) {
                         const unsigned deg = __shfl_sync(kFull, rx, kCoreDeg - 32);
@@ -882,7 +868,7 @@ __device__ void core_stream(const RoundParams &P, const CoreParams &Q, const Sha
 
 // A round: the block's share of the vertices of several pieces (every grid-th of the list, kMany at a
 // time), then the warp's share of the others.
-template <bool BATCH, bool SAT>
+template <bool BATCH>
 __device__ void core_round(const RoundParams &P, const CoreParams &Q, const Shared &S, const int32_t *cex_cur,
                            unsigned none, unsigned nmany, unsigned nv, int pass, const DetState &st_r0, unsigned *cn,
                            unsigned *grab, unsigned gw, unsigned nw, int lane, int wib, uint8_t *seen, unsigned *wfin,
@@ -926,10 +912,10 @@ __device__ void core_round(const RoundParams &P, const CoreParams &Q, const Shar
             }
         }
         __syncthreads();
-        core_stream<BATCH, true, SAT>(P, Q, S, cex_cur, cur, nullptr, 0u, nv, pass, st_r0, cn, nw, lane, seen, wfin, M, nmv,
+        core_stream<BATCH, true>(P, Q, S, cex_cur, cur, nullptr, 0u, nv, pass, st_r0, cn, nw, lane, seen, wfin, M, nmv,
                                  pd, npend, st_read, st_deg, st_cnt);
     }
-    core_stream<BATCH, false, SAT>(P, Q, S, cex_cur, cur, active_ones(Q, pass), none, nv, pass, st_r0, cn, nw, lane,
+    core_stream<BATCH, false>(P, Q, S, cex_cur, cur, active_ones(Q, pass), none, nv, pass, st_r0, cn, nw, lane,
                               seen, wfin, M, 0, pd, npend, st_read, st_deg, st_cnt);
     if (npend) flush_pending(Q, pd, npend, cn, pass, lane);
 }
@@ -964,7 +950,6 @@ __global__ void __launch_bounds__(kCoreThreads, 1) core_round_kernel(RoundParams
         Q.m[3] = static_cast<unsigned>(R0);
     }
     __shared__ ManyShared s_many;
-    __shared__ unsigned s_sat;
     *reinterpret_cast<uint2 *>(s_seen[wib] + 8 * lane) = make_uint2(0u, 0u);
     Shared S;
     S.col = s_dyn;
@@ -1063,19 +1048,15 @@ __global__ void __launch_bounds__(kCoreThreads, 1) core_round_kernel(RoundParams
                 else
                     apply_log(S, Q.log + static_cast<size_t>(pass & 1) * Q.max_v, nprev);
             }
-            if (threadIdx.x == 0) s_sat = __ldcg(Q.tail + kTailSat);  // (set for good, before the barrier)
             __syncthreads();
             CORE_PROF(1, atomicMax);
             unsigned st_deg = 0, st_cnt = 0, st_read = 0;
             // (word 3 of the counter set is the round's grab counter)
             if (pass == R0 && core_fused(R0))
                 core_first_round<BATCH>(P, Q, m, pass, cn, lane, st_read, st_deg, st_cnt);
-            else if (s_sat == 0u)
-                core_round<BATCH, false>(P, Q, S, cex_cur, cc.z, nmany, nv, pass, h.st, cn, cset + 3, gw, nw, lane,
-                                         wib, s_seen[wib], s_fin[wib], s_many, st_read, st_deg, st_cnt);
             else
-                core_round<BATCH, true>(P, Q, S, cex_cur, cc.z, nmany, nv, pass, h.st, cn, cset + 3, gw, nw, lane,
-                                        wib, s_seen[wib], s_fin[wib], s_many, st_read, st_deg, st_cnt);
+                core_round<BATCH>(P, Q, S, cex_cur, cc.z, nmany, nv, pass, h.st, cn, cset + 3, gw, nw, lane, wib,
+                                  s_seen[wib], s_fin[wib], s_many, st_read, st_deg, st_cnt);
 #ifdef GC_CORE_PROFILE
             __syncthreads();
             CORE_PROF(2, atomicMin);

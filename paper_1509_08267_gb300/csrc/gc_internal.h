@@ -257,7 +257,6 @@ constexpr int kCoreTail = 59;  // the vertex's tail id (tail phase)
 // from 1,024).
 constexpr int kTailOwned = 256;
 constexpr int kTailDefault = 384;
-constexpr int kTailSat = 2;
 struct CoreParams {
     int32_t max_v;        // vertex capacity M (shared memory holds M 8-bit colors and M FINAL bits; a
                           // multiple of 16)
@@ -278,8 +277,7 @@ struct CoreParams {
     unsigned *m;          // [4]: larger vertices numbered by the index kernel, m, pieces
     int32_t tail_max;     // tail phase once the worklist has at most this many vertices (0: never)
     int32_t tail_nc;      // blocks of the tail's cluster (tail_max <= kTailOwned * tail_nc)
-    unsigned *tail;       // [4]: 1 when the core handed over to the tail, the tail's first round, 1 once a core
-                          // vertex or one of its final neighbours has a color of 255 or more (kTailSat)
+    unsigned *tail;       // [4]: 1 when the core handed over to the tail, the tail's first round
 };
 
 // Small graphs (gc_small.cu).  A batch's graphs of at most kSmallBatchVertices vertices and
