@@ -92,9 +92,9 @@ struct Ctl {
     unsigned tail_ctl[4];  // tail phase: handed over, first round
     unsigned small_ctl[4];  // small graphs: a batch's queued and taken graphs; a cluster's losers per round
     unsigned long long small_left;  // vertices of the graphs that are not small
-    unsigned long long digest_cnt[kDigestBins];  // value keys: degrees per digest bin
     alignas(128) unsigned ord_cnt[3 * kOrdSet];  // ordered mode and peeling
     GridBar bar;
+    unsigned long long digest_cnt[kDigestBins];  // value keys: degrees per digest bin
 };
 static_assert(offsetof(Ctl, bar) % 128 == 0, "barrier alignment");
 static_assert(offsetof(Ctl, core_cnt) % 16 == 0, "core counter alignment");

@@ -252,12 +252,12 @@ __device__ __forceinline__ void det_write(const DetState &cur, const DetState &n
     if (!lose) det_store(cur, V, cv, dig, true);
 }
 
-// The same in the deterministic mode's state (inlined, four entries a lane: a call, or eight, makes the
-// round kernel spill twice as much around its main loop).
+// The same in the deterministic mode's state (inlined, two entries a lane: a call, or more, makes the round
+// kernel spill more around its main loop).
 __device__ __forceinline__ int32_t det_mex_from(const int32_t *colidx, const DetState &S, const Row &r, unsigned *win,
                                                 int lane, int32_t start) {
-    return mex_rescan<4>(colidx, r, win, lane, start,
-                         [&](const int32_t (&U)[4], int32_t (&c)[4]) { det_colors<4>(S, U, c); });
+    return mex_rescan<2>(colidx, r, win, lane, start,
+                         [&](const int32_t (&U)[2], int32_t (&c)[2]) { det_colors<2>(S, U, c); });
 }
 
 // Does a neighbour (local id ul, global id U) of equal color have the smaller key?  pv: the
@@ -547,6 +547,10 @@ __device__ __forceinline__ int32_t det_sweep_item(const RoundParams &P, const De
                 }
             }
         }
+        // exact colors in place of saturated ones, all in flight together (a color of 2^22 needs 2^43 entries)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (color16(b[q]) == kSat7) b[q] = static_cast<unsigned>(__ldca(S.cx + vbase + u[q])) << 9 | (b[q] & 511u);
         const bool more = j0 + kStep < le;
         if (more) item_quad(list, j0 + kStep + 4 * lane, lb, le, un, vn);
         unsigned keepm = valid, tie = 0;
@@ -555,8 +559,7 @@ __device__ __forceinline__ int32_t det_sweep_item(const RoundParams &P, const De
         for (int q = 0; q < 4; ++q) {
             if (!((valid >> q) & 1u)) continue;
             const bool fin = DROP && (b[q] & kFinal);
-            int32_t c = static_cast<int32_t>(color16(b[q]));
-            if (c == static_cast<int32_t>(kSat7)) c = __ldcg(S.cx + vbase + u[q]);
+            const int32_t c = static_cast<int32_t>(color16(b[q]));
             if (c < 32) {
                 lo0 |= 1u << c;
                 if (fin) f0 |= 1u << c;
