@@ -1015,7 +1015,14 @@ __global__ void __launch_bounds__(kCoreThreads, 1) core_round_kernel(RoundParams
             // of several pieces listed}
             unsigned *cset = Q.cnt + kCoreCnt * (pass % 3);
             const uint4 cc = ldcg4(cset);
-            const unsigned nmany = __ldcg(cset + 4);
+            unsigned nmany, leave = 0u;
+            if constexpr (BATCH) {  // (a server's pool: word 5, asked to leave)
+                const uint2 c2 = __ldcg(reinterpret_cast<const uint2 *>(cset + 4));
+                nmany = c2.x;
+                leave = c2.y;
+            } else {
+                nmany = __ldcg(cset + 4);
+            }
             unsigned *cn = Q.cnt + kCoreCnt * ((pass + 1) % 3);
             // |W_pass|: every core vertex in the first round, then the previous round's losers
             const unsigned nv = pass == R0 ? static_cast<unsigned>(m) : cc.y;
@@ -1025,6 +1032,14 @@ __global__ void __launch_bounds__(kCoreThreads, 1) core_round_kernel(RoundParams
                     set_error(P.err, GC_ERR_NO_CONVERGENCE, pass, 0);
                 break;
             }
+            // something waits for the GPU: the host puts what is left back on the worklist
+            if (BATCH && pass > R0 && leave != 0u) {
+                if (blockIdx.x == 0 && threadIdx.x == 0) Q.tail[2] = static_cast<unsigned>(pass);
+                break;
+            }
+            int ask = 0;  // (read while the round runs, seen by every block in the next one)
+            if (BATCH && Q.leave && blockIdx.x == 0 && threadIdx.x == 0)
+                ask = *reinterpret_cast<const volatile int *>(Q.leave);
             // few enough for the tail phase (one cluster runs the remaining rounds): every block
             // reads the same count, so all leave here
             if (pass > R0 && nv <= static_cast<unsigned>(Q.tail_max)) {
@@ -1063,6 +1078,7 @@ __global__ void __launch_bounds__(kCoreThreads, 1) core_round_kernel(RoundParams
             CORE_PROF(3, atomicMax);
 #endif
             if (P.stats) flush_stats(P, pass, st_deg, st_cnt, st_read);
+            if (BATCH && ask != 0) cn[5] = 1u;
             if (!grid_sync(P.bar, bar_target, P.err, P.spin_ns)) break;
         }
     }
@@ -1072,9 +1088,38 @@ __global__ void __launch_bounds__(kCoreThreads, 1) core_round_kernel(RoundParams
     }
 }
 
+// The worklist of round P.pass_begin after a core that left in it: one lane per core vertex.
+__global__ void core_return_kernel(RoundParams P, CoreParams Q) {
+    const int pass = P.pass_begin;
+    const int64_t m = __ldcg(Q.m + 1);
+    const int32_t *cex = Q.cex + static_cast<size_t>(pass & 1) * Q.max_v;
+    int32_t *small_cur = (pass & 1) ? P.small0 : P.small1;
+    const int lane = threadIdx.x & 31;
+    unsigned long long st_ent = 0;
+    for (int64_t base = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) & ~int64_t{31}; base < m;
+         base += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        const int64_t i = base + lane;
+        int32_t V = 0, deg = 0;
+        bool open = false;
+        if (i < m) {
+            V = static_cast<int32_t>(__ldcg(core_rec(Q, i) + kCoreGid));
+            deg = static_cast<int32_t>(__ldcg(core_rec(Q, i) + kCoreDeg));
+            open = !(__ldcg(Q.fbits + (i >> 5)) >> (i & 31) & 1u);
+            const int32_t c = __ldcg(cex + i);
+            const unsigned dig = digest16(load_s16(P.s16a + V));
+            det_store(DetState{P.s16a, P.cx0}, V, c, dig, !open);
+            det_store(DetState{P.s16b, P.cx1}, V, c, dig, !open);
+            if (open) st_ent += static_cast<unsigned long long>(deg);
+        }
+        warp_append(open && deg <= P.T1, V, small_cur, P.cnt + kCnt * (pass % 3) + kCntSmall, lane);
+        warp_append(open && deg > P.T1, V, P.items, P.tmp, lane);
+    }
+    if (P.ecnt) flush_sum(P.ecnt + pass % 3, st_ent);
+}
+
 // Final colors of the core into both state buffers (FINAL set), where the color count reads them.
 __global__ void core_writeback_kernel(RoundParams P, CoreParams Q) {
-    if (__ldcg(P.core_go) == 0) return;
+    if (__ldcg(P.core_go) == 0 || __ldcg(Q.tail + 2) != 0u) return;
     const int64_t m = __ldcg(Q.m + 1);  // the round kernel rewrote passes[0]; the core recorded m here
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < m;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
@@ -1186,6 +1231,11 @@ cudaError_t launch_core(const RoundParams &P, const CoreParams &Q, bool batch, c
     }
 #endif
     core_writeback_kernel<<<grid, 256, 0, s>>>(P, Q);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_core_return(const RoundParams &P, const CoreParams &Q, cudaStream_t s) {
+    core_return_kernel<<<static_cast<unsigned>((Q.max_v + 255) / 256), 256, 0, s>>>(P, Q);
     return cudaGetLastError();
 }
 

@@ -277,7 +277,9 @@ struct CoreParams {
     unsigned *m;          // [4]: larger vertices numbered by the index kernel, m, pieces
     int32_t tail_max;     // tail phase once the worklist has at most this many vertices (0: never)
     int32_t tail_nc;      // blocks of the tail's cluster (tail_max <= kTailOwned * tail_nc)
-    unsigned *tail;       // [4]: 1 when the core handed over to the tail, the tail's first round
+    unsigned *tail;       // [4]: 1 when the core handed over to the tail, the tail's first round, the round
+                          // the core left for the host's sake (0: it did not)
+    const int *leave;     // a host word that asks the rounds to stop when it is not 0, or nullptr
 };
 
 // Small graphs (gc_small.cu).  A batch's graphs of at most kSmallBatchVertices vertices and
@@ -385,6 +387,10 @@ cudaError_t launch_det_round_block(int32_t n, const int32_t *rowptr, const int32
 // of the vertex state.  core_max_vertices: the largest M the shared memory of one block per SM allows.
 int32_t core_max_vertices();
 cudaError_t launch_core(const RoundParams &P, const CoreParams &Q, bool batch, cudaStream_t s);
+// After a core that left (Q.tail[2] = P.pass_begin): the core vertices' colors back into both state
+// buffers and the unfinished ones onto the worklist of that round, the larger ones for launch_expand.  The
+// worklist counters and P.tmp must be zero.
+cudaError_t launch_core_return(const RoundParams &P, const CoreParams &Q, cudaStream_t s);
 // Tail phase: the largest cluster (16 or 8 blocks) the tail kernel can run as, 0 if none; the launch
 // (every block returns at once unless the core handed over).
 int32_t tail_cluster_size();

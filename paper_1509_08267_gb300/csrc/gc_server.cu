@@ -156,7 +156,7 @@ struct Engine {
     DevBuf c_rec, c_cex, c_c8, c_fbits, c_items, c_active, c_log, c_pool;
     CoreParams core{};
     int32_t core_max = 0;
-    int64_t left_vertices = 0;  // the next round's worklist, as of the last launch
+    int64_t left_vertices = 0, left_large = 0;  // the next round's worklist, as of the last launch
     std::vector<int64_t> h_vbase, h_ebase, h_rbase, h_m;
     std::vector<int32_t> h_n, h_glast;
     std::vector<uint64_t> h_seed;
@@ -197,6 +197,7 @@ struct gc_server {
     double t_create = 0, busy = 0;
     int fatal = GC_OK;
     std::string fatal_msg;
+    volatile int *waiting = nullptr;  // pinned: a request was submitted since the worker last looked
 };
 
 namespace gc {
@@ -218,7 +219,12 @@ int engine_index(int mode) { return mode == GC_MODE_INPLACE ? 1 : 0; }
 
 // The core phase's buffers for a deterministic pool (sizes as gc_color's); without them the pool's
 // rounds all run in the round kernel.
-void core_create(Engine &E) {
+void core_create(gc_server *s, Engine &E) {
+    void *waiting = nullptr;
+    if (cudaHostGetDevicePointer(&waiting, const_cast<int *>(s->waiting), 0) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
     const int32_t cm = core_max_vertices();
     const int64_t M = std::min<int64_t>({E.PV, static_cast<int64_t>(cm) - 16, (int64_t{1} << 18) - 32});
     if (M <= 0) return;
@@ -254,6 +260,7 @@ void core_create(Engine &E) {
     Q.cnt = c->core_cnt;
     Q.m = c->core_m;
     Q.tail = c->tail_ctl;
+    Q.leave = static_cast<const int *>(waiting);
     const int32_t nc = tail_cluster_size();
     if (nc > 0) {
         Q.tail_nc = nc;
@@ -304,7 +311,7 @@ int engine_create(gc_server *s, Engine &E, int mode) {
         return set_last_error(e == cudaErrorMemoryAllocation ? GC_ERR_OOM : GC_ERR_CUDA, "server pool: %s",
                               cudaGetErrorString(e));
     }
-    if (E.compact) core_create(E);
+    if (E.compact) core_create(s, E);
     int per_sm = 0, sms = 0;
     round_kernel_occupancy(mode, true, E.compact, 256, &per_sm);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->device);
@@ -534,7 +541,7 @@ int engine_reset(gc_server *s, Engine &E, int code) {
     SRV_CUDA(cudaMemsetAsync(E.ctl.p, 0, sizeof(Ctl), s->stream));
     SRV_CUDA(cudaStreamSynchronize(s->stream));
     E.next_pass = 1;
-    E.left_vertices = 0;
+    E.left_vertices = E.left_large = 0;
     return GC_OK;
 }
 
@@ -568,7 +575,8 @@ void fail_all(gc_server *s, int code, const std::string &msg) {
 
 // One pass of the worker over a pool: admission, a launch of a few rounds, retirement.  Returns
 // false after an error the server cannot recover from (a failed CUDA call).
-bool engine_step(gc_server *s, Engine &E, std::vector<Request *> &adm, bool queued) {
+// waiting: something else -- a queued request, one to be colored alone, the other pool -- waits for the GPU.
+bool engine_step(gc_server *s, Engine &E, std::vector<Request *> &adm, bool queued, bool waiting) {
     const double t0 = now_s();
     std::vector<Request *> bad;
     if (admit(s, E, adm, bad) != GC_OK) return false;
@@ -585,10 +593,14 @@ bool engine_step(gc_server *s, Engine &E, std::vector<Request *> &adm, bool queu
         if (E.resident.empty()) return true;
     }
     RoundParams P = params(s, E, queued ? kRoundsWhileQueued : kRoundsIdleQueue);
-    // Nothing waits, nothing joined and the worklist fits the core phase: it runs the batch to its end
-    // (about 10 us a round against 40-50 in the round kernel: 24 requests of up to 200,000 vertices
-    // took 7.9 ms without it).  A request that arrives meanwhile waits for that end, a millisecond or two.
-    const bool core = E.core_max > 0 && !queued && adm.empty() && E.left_vertices > 0 && E.left_vertices <= E.core_max;
+    // Nothing waits, nothing joined, the worklist fits the core phase and has vertices past the thread
+    // bound (as in gc_color's rule: without them the round kernel is the faster one): it runs the batch on
+    // (about 10 us a round against 40-50 in the round kernel: 24 requests of up to 200,000 vertices took
+    // 7.9 ms without it).  It ends with the batch, or one round after something was submitted (two when the
+    // read of the host's word is late; the tail phase, at most 384 vertices, is not interrupted): what is
+    // left then goes back on the worklist.
+    const bool core = E.core_max > 0 && !queued && !waiting && adm.empty() && E.left_large > 0 &&
+                      E.left_vertices <= E.core_max;
     cudaError_t e = cudaSuccess;
     Ctl *ctl = E.ctl.as<Ctl>();
     if (core) {
@@ -628,10 +640,23 @@ bool engine_step(gc_server *s, Engine &E, std::vector<Request *> &adm, bool queu
             srv_fail(s, GC_ERR_CUDA, "server round launch", e);
             return false;
         }
-        E.left_vertices = 0;
+        E.left_vertices = E.left_large = 0;
+        if (h.tail_ctl[2] != 0) {
+            RoundParams R = params(s, E);
+            e = cudaMemsetAsync(R.tmp, 0, 2 * sizeof(unsigned), s->stream);
+            if (e == cudaSuccess) e = launch_core_return(R, E.core, s->stream);
+            if (e == cudaSuccess) e = launch_expand(R, E.mode, true, E.compact, -1, s->stream);
+            if (e != cudaSuccess) {
+                srv_fail(s, GC_ERR_CUDA, "server round launch", e);
+                return false;
+            }
+            E.left_vertices = h.core_cnt[kCoreCnt * (E.next_pass % 3) + 1];
+            E.left_large = 1;  // (some, as far as known here)
+        }
     } else {
         const unsigned *c = h.cnt + kCnt * (E.next_pass % 3);
-        E.left_vertices = static_cast<int64_t>(c[kCntSmall]) + c[kCntItems];
+        E.left_large = c[kCntItems];
+        E.left_vertices = static_cast<int64_t>(c[kCntSmall]) + E.left_large;
     }
     std::vector<Request *> fin;
     {
@@ -705,6 +730,7 @@ void worker_main(gc_server *s) {
         std::vector<Request *> adm[2];
         bool active[2] = {false, false}, queued[2] = {false, false};
         Request *solo = nullptr;
+        bool solos = false;  // more of them wait
         {
             std::unique_lock<std::mutex> lk(s->mu);
             s->cv_work.wait(lk, [&] { return s->stop || !s->solo.empty() || s->eng[0].busy() || s->eng[1].busy(); });
@@ -714,6 +740,8 @@ void worker_main(gc_server *s) {
                 s->solo.pop_front();
                 solo->state = kResident;
             }
+            solos = !s->solo.empty();
+            *s->waiting = 0;  // everything submitted so far is in these lists
             for (int k = 0; k < 2; ++k) {
                 Engine &E = s->eng[k];
                 if (!E.busy()) continue;
@@ -744,7 +772,7 @@ void worker_main(gc_server *s) {
         }
         bool ok = true;
         for (int k = 0; k < 2 && ok; ++k)
-            if (active[k]) ok = engine_step(s, s->eng[k], adm[k], queued[k]);
+            if (active[k]) ok = engine_step(s, s->eng[k], adm[k], queued[k], solos || active[1 - k]);
         if (!ok) {
             fail_all(s, s->fatal, s->fatal_msg);
             break;
@@ -779,7 +807,11 @@ int gc_server_create(const gc_server_config *cfg, gc_server **out) {
     s->cfg = *cfg;
     s->device = dev;
     s->solo_min = cfg->solo_entries < 0 ? INT64_MAX : (cfg->solo_entries == 0 ? int64_t{1} << 24 : cfg->solo_entries);
-    cudaError_t e = cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking);
+    void *word = nullptr;
+    cudaError_t e = cudaHostAlloc(&word, 64, cudaHostAllocPortable | cudaHostAllocMapped);
+    s->waiting = static_cast<volatile int *>(word);
+    if (e == cudaSuccess) *s->waiting = 0;
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->copy_stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) {
         // the device copies of requests colored alone: memory freed by one stays for the next (a pool
@@ -806,6 +838,7 @@ int gc_server_create(const gc_server_config *cfg, gc_server **out) {
     }
     if (e != cudaSuccess) {
         cudaGetLastError();
+        if (word) cudaFreeHost(word);
         return set_last_error(GC_ERR_CUDA, "server streams: %s", cudaGetErrorString(e));
     }
     gc::Engine &E0 = s->eng[gc::engine_index(cfg->mode)];
@@ -815,6 +848,7 @@ int gc_server_create(const gc_server_config *cfg, gc_server **out) {
         cudaStreamDestroy(s->stream);
         cudaStreamDestroy(s->copy_stream);
         cudaMemPoolDestroy(s->solo_pool);
+        cudaFreeHost(word);
         return st;
     }
     s->t_create = gc::now_s();
@@ -953,6 +987,7 @@ int gc_server_submit(gc_server *s, int32_t n, const int32_t *rowptr, const int32
         s->solo.push_back(raw);
     else
         E.queue.push_back(raw);
+    *s->waiting = 1;
     s->cv_work.notify_one();
     return GC_OK;
 }
@@ -1048,6 +1083,7 @@ void gc_server_destroy(gc_server *s) {
     if (s->solo_pool) cudaMemPoolDestroy(s->solo_pool);
     if (s->stream) cudaStreamDestroy(s->stream);
     if (s->copy_stream) cudaStreamDestroy(s->copy_stream);
+    if (s->waiting) cudaFreeHost(const_cast<int *>(s->waiting));
     delete s;
 }
 
