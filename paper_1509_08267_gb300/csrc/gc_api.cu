@@ -294,8 +294,8 @@ static int peel_levels(Context &C, Ctl *ctl, RoundParams P, int32_t T1, int32_t 
     GC_TRY(ensure(C.col0, 8 * n, "vertex state"));
     GC_TRY(ensure(C.col1, 8 * n, "vertex state"));
     GC_TRY(ensure(C.items, 4 * n, "worklist"));
-    GC_TRY(ensure(C.mid0, 32 * n, "worklist"));
-    GC_TRY(ensure(C.mid1, 32 * n, "worklist"));
+    GC_TRY(ensure(C.mid0, 16 * n, "worklist"));
+    GC_TRY(ensure(C.mid1, 16 * n, "worklist"));
     P.T1 = T1 < kOrdSmall ? T1 : kOrdSmall;
     P.CH = CH < kOrdChunk ? CH : kOrdChunk;
     P.pass_begin = 1;
@@ -462,8 +462,13 @@ static int run(Context &C, const Problem &pb, int mode, uint64_t seed, const gc_
     GC_TRY(ensure(C.col0, 8 * n, "vertex state"));
     GC_TRY(ensure(C.col1, 8 * n + kDetPad, "vertex state"));
     GC_TRY(ensure(C.items, 4 * n, "worklist"));
-    GC_TRY(ensure(C.small0, 4 * n, "worklist"));
-    GC_TRY(ensure(C.small1, 4 * n, "worklist"));
+    if (mode == GC_MODE_ORDERED) {
+        GC_TRY(ensure(C.mid0, 16 * static_cast<size_t>(n), "worklist"));
+        GC_TRY(ensure(C.mid1, 16 * static_cast<size_t>(n), "worklist"));
+    } else {
+        GC_TRY(ensure(C.small0, 4 * n, "worklist"));
+        GC_TRY(ensure(C.small1, 4 * n, "worklist"));
+    }
     GC_TRY(ensure(C.ctl, sizeof(Ctl), "control"));
     GC_TRY(ensure(C.bitmap, 4 * (n / 32 + 2), "color bitmap"));
     const int32_t shift = sort_shift(n);
@@ -601,8 +606,10 @@ static int run(Context &C, const Problem &pb, int mode, uint64_t seed, const gc_
         // First Fit in key order: in-place set-up (vertices with neighbours uncolored, no worklist
         // sort; it also counts the larger vertices and their work items), pending counts of
         // smaller-key neighbours in the unused second state array, then rounds over the ready
-        // vertices only
+        // vertices only (the set-up's list of the others is not used; it goes where the ready lists will be)
         P.deg_hist = nullptr;
+        P.small0 = C.mid0.as<int32_t>();
+        P.small1 = C.mid1.as<int32_t>();
         P.T1 = T1 < kOrdSmall ? T1 : kOrdSmall;
         // a single graph's rounds are a chain of short latency-bound steps: 64-entry work items (32 and
         // 128: 0-32% slower on long chains or heavy rounds) and two blocks per SM (one: 1.5% faster where
@@ -620,8 +627,6 @@ static int run(Context &C, const Problem &pb, int mode, uint64_t seed, const gc_
         GC_TRY(ensure(C.chunk0, 16 * std::max<size_t>(n_items, 1), "work items"));
         GC_TRY(ensure(C.chunk1, 16 * std::max<size_t>(n_items, 1), "work items"));
         GC_TRY(ensure(C.acc, 4 * kOrdSlotWords * std::max<size_t>(slots, 1), "accumulators"));
-        GC_TRY(ensure(C.mid0, 32 * static_cast<size_t>(n), "worklist"));
-        GC_TRY(ensure(C.mid1, 32 * static_cast<size_t>(n), "worklist"));
         P.chunk0 = C.chunk0.as<int4>();
         P.chunk1 = C.chunk1.as<int4>();
         P.ord0 = C.mid0.as<int4>();

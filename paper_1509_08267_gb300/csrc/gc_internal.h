@@ -164,7 +164,8 @@ struct RoundParams {
     int64_t ci_len;  // entries of colidx that may be read (16-byte loads stay inside them)
     int32_t *small0, *small1;  // thread-per-vertex worklists (two parities)
     int4 *chunk0, *chunk1;     // warp work items, kItemBytes each (two parities)
-    int4 *ord0, *ord1;         // ordered mode: small, then medium-degree ready vertices, n each (two parities)
+    int4 *ord0, *ord1;         // ordered mode: the ready vertices, n entries (two parities): small ones from
+                               // the front, medium-degree ones from the back
     unsigned ord_items;        // ordered mode: entries chunk0 / chunk1 hold
     unsigned *ord_cnt;         // [3][kOrdSet] its counter sets, a counter per 128 bytes: every releasing warp adds
                                // to them, and atomics on one line queue
@@ -357,7 +358,7 @@ cudaError_t launch_count_colors(const RoundParams &P, bool batch, const int32_t 
 // Ordered mode (GC_MODE_ORDERED): after the in-place launch_setup (every vertex with neighbours
 // uncolored) with P.T1 <= kOrdSmall and P.CH <= kOrdChunk, with the counter sets and P.acc's slots
 // zeroed, counts each vertex's smaller-key neighbours into its word W[n], lists the first ready
-// vertices (P.ord0 / ord1 hold 2 n entries each, chunk0 / chunk1 P.ord_items work items) and runs the
+// vertices (P.ord0 / ord1 hold n entries each, chunk0 / chunk1 P.ord_items work items) and runs the
 // cooperative round kernel on `grid` blocks.
 cudaError_t ordered_kernel_occupancy(bool batch, int block, int *blocks_per_sm);
 // Smallest-last levels (single graph): launch_peel_init sets the words W to deg(v), level[v] = 0, the two

@@ -2093,7 +2093,8 @@ __device__ __forceinline__ int32_t ord_color(uint64_t w) { return ord_open(w) ? 
 // so that a round starts with its entries' loads.
 struct OrdLists {
     int4 *small;    // {V, first entry, degree}: degree <= P.T1    (count cnt[kCntSmall])
-    int4 *mid;      // the same: degree <= kOrdMid                  (count cnt[kCntMulti])
+    int4 *mid;      // the same: degree <= kOrdMid, from the array's end backwards (count cnt[kCntMulti]); a
+                    // vertex is listed once in the whole run, so the two fit into n entries
     int4 *items;    // work items {V, first entry, entries | kOrdFirst, slot}, a batch's first entry counted
                     // from the row's start                        (count cnt[kCntChunks]; slots cnt[kCntItems])
     unsigned *cnt;  // the round's counter set
@@ -2103,7 +2104,7 @@ constexpr int32_t kOrdFirst = 1 << 30;  // a vertex's first item
 __device__ __forceinline__ OrdLists ord_lists(const RoundParams &P, int pass) {
     const bool odd = (pass & 1) != 0;
     int4 *base = odd ? P.ord0 : P.ord1;
-    return OrdLists{base, base + P.n, odd ? P.chunk0 : P.chunk1, P.ord_cnt + kOrdSet * (pass % 3)};
+    return OrdLists{base, base + (P.n - 1), odd ? P.chunk0 : P.chunk1, P.ord_cnt + kOrdSet * (pass % 3)};
 }
 
 // Row of a small or medium list entry.
@@ -2191,7 +2192,7 @@ __device__ void ord_list(const RoundParams &P, const bool (&ready)[K], const int
         if (kind[k] == 0u) {
             L.small[b + __popc(m0 & lanemask_lt())] = make_int4(U[k], rb[k], deg[k], 0);
         } else if (kind[k] == 1u) {
-            L.mid[b + __popc(m1 & lanemask_lt())] = make_int4(U[k], rb[k], deg[k], 0);
+            L.mid[-static_cast<int64_t>(b + __popc(m1 & lanemask_lt()))] = make_int4(U[k], rb[k], deg[k], 0);
         } else if (kind[k] == 2u) {
             const unsigned nch = static_cast<unsigned>((deg[k] + P.CH - 1) / P.CH);
             const int32_t slot = nch > 1u ? static_cast<int32_t>(mb++) : -1;
@@ -2604,7 +2605,7 @@ __global__ void __launch_bounds__(kBlock, BATCH ? kWideBlocks : 2) ord_round_ker
         const unsigned mid_groups = (nmid + 3u) / 4u;
         for (unsigned b = (gw + nw - nitems % nw) % nw; b < mid_groups; b += nw) {
             const unsigned i = 4u * b + static_cast<unsigned>(lane >> 3);
-            ord_mid<BATCH>(P, W, i < nmid, i < nmid ? __ldcg(C.mid + i) : make_int4(0, 0, 0, 0), L, pass, lane, st_deg,
+            ord_mid<BATCH>(P, W, i < nmid, i < nmid ? __ldcg(C.mid - i) : make_int4(0, 0, 0, 0), L, pass, lane, st_deg,
                            st_cnt);
         }
         const unsigned skip = (nitems + mid_groups) % nw;
@@ -2793,7 +2794,7 @@ __global__ void __launch_bounds__(kBlock, kWideBlocks) peel_kernel(RoundParams P
             const unsigned mid_groups = (nmid + 3u) / 4u;
             for (unsigned b = (gw + nw - nitems % nw) % nw; b < mid_groups; b += nw) {
                 const unsigned i = 4u * b + static_cast<unsigned>(lane >> 3);
-                peel_mid(P, W, level, i < nmid, i < nmid ? __ldcg(C.mid + i) : make_int4(0, 0, 0, 0), k, L, N, lane);
+                peel_mid(P, W, level, i < nmid, i < nmid ? __ldcg(C.mid - i) : make_int4(0, 0, 0, 0), k, L, N, lane);
             }
             const unsigned skip = (nitems + mid_groups) % nw;
             for (unsigned base = ((gw + nw - skip) % nw) * 32u; base < nsmall; base += nw * 32u) {
