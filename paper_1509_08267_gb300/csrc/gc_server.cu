@@ -11,6 +11,7 @@
 // the GPU by itself (cfg.solo_entries) skips the pool: between launches the worker colors it alone
 // the way gc_color_ex does, with the core and tail phases that the batch's shared rounds cannot run.
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <climits>
 #include <condition_variable>
@@ -198,6 +199,7 @@ struct gc_server {
     int fatal = GC_OK;
     std::string fatal_msg;
     volatile int *waiting = nullptr;  // pinned: a request was submitted since the worker last looked
+    std::atomic<int> submitting{0};   // submits under way: their copies may have to wait for running kernels
 };
 
 namespace gc {
@@ -214,6 +216,18 @@ int srv_fail(gc_server *s, int code, const char *what, cudaError_t e) {
         cudaError_t e_ = (call);                                           \
         if (e_ != cudaSuccess) return srv_fail(s, GC_ERR_CUDA, #call, e_); \
     } while (0)
+
+// A submit under way: the core phase leaves its rounds for it and is not entered until it is done.
+struct Submitting {
+    gc_server *s;
+    explicit Submitting(gc_server *server) : s(server) {
+        s->submitting.fetch_add(1);
+        *s->waiting = 1;
+    }
+    ~Submitting() { s->submitting.fetch_sub(1); }
+    Submitting(const Submitting &) = delete;
+    Submitting &operator=(const Submitting &) = delete;
+};
 
 int engine_index(int mode) { return mode == GC_MODE_INPLACE ? 1 : 0; }
 
@@ -575,7 +589,8 @@ void fail_all(gc_server *s, int code, const std::string &msg) {
 
 // One pass of the worker over a pool: admission, a launch of a few rounds, retirement.  Returns
 // false after an error the server cannot recover from (a failed CUDA call).
-// waiting: something else -- a queued request, one to be colored alone, the other pool -- waits for the GPU.
+// waiting: something else -- a submit under way, a request to be colored alone, the other pool -- waits for
+// the GPU.
 bool engine_step(gc_server *s, Engine &E, std::vector<Request *> &adm, bool queued, bool waiting) {
     const double t0 = now_s();
     std::vector<Request *> bad;
@@ -596,9 +611,9 @@ bool engine_step(gc_server *s, Engine &E, std::vector<Request *> &adm, bool queu
     // Nothing waits, nothing joined, the worklist fits the core phase and has vertices past the thread
     // bound (as in gc_color's rule: without them the round kernel is the faster one): it runs the batch on
     // (about 10 us a round against 40-50 in the round kernel: 24 requests of up to 200,000 vertices took
-    // 7.9 ms without it).  It ends with the batch, or one round after something was submitted (two when the
-    // read of the host's word is late; the tail phase, at most 384 vertices, is not interrupted): what is
-    // left then goes back on the worklist.
+    // 7.9 ms without it).  It ends with the batch, or one round after a submit began (two when the read of the
+    // host's word is late; the tail phase, at most 384 vertices, is not interrupted): what is left then goes
+    // back on the worklist.
     const bool core = E.core_max > 0 && !queued && !waiting && adm.empty() && E.left_large > 0 &&
                       E.left_vertices <= E.core_max;
     cudaError_t e = cudaSuccess;
@@ -772,7 +787,8 @@ void worker_main(gc_server *s) {
         }
         bool ok = true;
         for (int k = 0; k < 2 && ok; ++k)
-            if (active[k]) ok = engine_step(s, s->eng[k], adm[k], queued[k], solos || active[1 - k]);
+            if (active[k]) ok = engine_step(s, s->eng[k], adm[k], queued[k],
+                                           solos || active[1 - k] || s->submitting.load() > 0);
         if (!ok) {
             fail_all(s, s->fatal, s->fatal_msg);
             break;
@@ -865,6 +881,7 @@ int gc_server_submit(gc_server *s, int32_t n, const int32_t *rowptr, const int32
         return set_last_error(GC_ERR_INVALID_ARG, "unknown mode %d (the server runs the deterministic and in-place "
                                                   "modes)", mode);
     if (n < 0 || (n > 0 && !rowptr)) return set_last_error(GC_ERR_INVALID_ARG, "bad n or NULL rowptr");
+    const gc::Submitting under_way(s);
     gc::Engine &E = s->eng[gc::engine_index(mode)];
     {
         // the first request of a mode allocates that mode's pool

@@ -47,6 +47,17 @@ def test_a_small_request_does_not_wait_for_the_batch(gclib, mode):
             assert st["core_handovers"] >= 2  # it left, and took over again
 
 
+def test_the_first_requests_do_not_wait_either(gclib):
+    # what a first submit sets up waits for running kernels
+    big, small = gg.complete(2500), gg.er(3000, 20.0, 1)
+    with gclib.Server(pool_vertices=8000, pool_entries=big.nnz + small.nnz + 64, mode="det", solo_entries=-1) as srv:
+        a = srv.submit(big.rowptr, big.colidx, seed=5)
+        time.sleep(0.05)
+        srv.poll(srv.submit(small.rowptr, small.colidx, seed=3))
+        assert srv.poll(a, timeout_ms=0) is None
+        np.testing.assert_array_equal(srv.poll(a)[0], _rank(big, 5))
+
+
 def test_many_arrivals(gclib):
     # power-law graphs (small and larger vertices, several work items) interrupted again and again
     gs = [gg.rmat(14, 16, 1), gg.rmat(13, 30, 2), gg.complete(400), gg.er(5000, 30.0, 3)]
