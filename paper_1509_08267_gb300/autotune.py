@@ -1,10 +1,11 @@
 """Autotuner for the round kernel's launch knobs.
 
-For each graph class it times the deterministic round kernel (CUDA events inside the library, on
-the launching stream) over a grid of knobs -- the largest degree handled by one thread
-(small_max_degree), the adjacency entries per warp work item (chunk), resident blocks per SM and
-the compact sweep -- and writes the fastest setting per class to a JSON table.  `options_for(graph)`
-returns the tuned gc_options for a graph from that table (library defaults when there is none).
+For each graph class it times whole deterministic calls over a grid of knobs -- the largest degree handled
+by one thread (small_max_degree), the adjacency entries per warp work item (chunk), resident blocks per SM
+and the compact sweep, 0 being the library's default -- and writes the fastest setting per class to a JSON
+table.  Whole calls, because a call that sets no knob may take the small-graph kernels instead of the round
+kernel.  `options_for(graph)` returns the tuned gc_options for a graph from that table (library defaults
+when there is none).
 
 Classes are decided from the degree sequence alone: "powerlaw" when the largest degree exceeds 50
 times the average, else "uniform"; each is split into "small" (< 100,000 vertices) and "large".
@@ -20,6 +21,7 @@ import itertools
 import json
 import os
 import statistics
+import time
 
 import numpy as np
 
@@ -29,8 +31,8 @@ from ._build import source_sha256
 TABLE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "tuning.json")
 
 GRID = {
-    "small_max_degree": [32, 63, 127],
-    "chunk": [256, 512, 1024],
+    "small_max_degree": [0, 32, 63, 127],
+    "chunk": [0, 256, 512, 1024],
     "blocks_per_sm": [0, 3],
     "compact": [False, True],
     "core_vertices": [0, -1],
@@ -51,19 +53,28 @@ def _options(cfg: dict, timing: bool = True) -> Options:
                    blocks_per_sm=cfg["blocks_per_sm"], flags=flags, core_vertices=cfg.get("core_vertices", 0))
 
 
-def time_config(rowptr, colidx, cfg: dict, repeats: int = 3, seed: int = 7) -> float:
-    """Median round-kernel milliseconds of deterministic coloring with the given knobs."""
-    color(rowptr, colidx, "det", seed, options=_options(cfg))  # warm-up
-    ms = [color(rowptr, colidx, "det", seed, options=_options(cfg)).stats.kernel_ms for _ in range(repeats)]
+def _median_ms(call, repeats: int) -> float:
+    """Median milliseconds of call(), which returns after its work is done."""
+    call()  # warm-up
+    ms = []
+    for _ in range(repeats):
+        t = time.perf_counter()
+        call()
+        ms.append((time.perf_counter() - t) * 1e3)
     return statistics.median(ms)
 
 
-def time_config_batch(args, cfg: dict, repeats: int = 3, seed: int = 7) -> float:
-    """Median round-kernel milliseconds of a deterministic batched coloring (args: the four packed
-    arrays on the device)."""
-    color_batch(*args, "det", seed, options=_options(cfg))
-    ms = [color_batch(*args, "det", seed, options=_options(cfg), stats=True)[3].kernel_ms for _ in range(repeats)]
-    return statistics.median(ms)
+def time_config(rowptr, colidx, cfg: dict, repeats: int = 5, seed: int = 7) -> float:
+    """Median milliseconds of a deterministic coloring with the given knobs."""
+    opt = _options(cfg, timing=False)
+    return _median_ms(lambda: color(rowptr, colidx, "det", seed, options=opt), repeats)
+
+
+def time_config_batch(args, cfg: dict, repeats: int = 5, seed: int = 7) -> float:
+    """Median milliseconds of a deterministic batched coloring (args: the four packed arrays on the
+    device)."""
+    opt = _options(cfg, timing=False)
+    return _median_ms(lambda: color_batch(*args, "det", seed, options=opt), repeats)
 
 
 def tune(samples: dict, grid: dict = GRID, repeats: int = 3, log=print) -> dict:
@@ -78,7 +89,7 @@ def tune(samples: dict, grid: dict = GRID, repeats: int = 3, log=print) -> dict:
             log(f"{cls:16s} {cfg} {ms:9.3f} ms")
             if best is None or ms < best[1]:
                 best = (cfg, ms)
-        table[cls] = {**best[0], "kernel_ms": best[1], "sources_sha256": source_sha256()}
+        table[cls] = {**best[0], "call_ms": best[1], "sources_sha256": source_sha256()}
     return table
 
 
@@ -134,7 +145,7 @@ def main():
     def on_device(g):
         return torch.from_numpy(g.rowptr).to(dev), torch.from_numpy(g.colidx).to(dev)
 
-    grid = GRID if not args.quick else {"small_max_degree": [63, 127], "chunk": [512, 1024], "blocks_per_sm": [0],
+    grid = GRID if not args.quick else {"small_max_degree": [0, 63, 127], "chunk": [0, 512, 1024], "blocks_per_sm": [0],
                                         "compact": [False, True], "core_vertices": [0, -1]}
     table = {}
     if args.only_batch:
