@@ -681,9 +681,8 @@ static int run(Context &C, const Problem &pb, int mode, uint64_t seed, const gc_
             const int32_t cm = core_max_vertices();
             C.core_max_v = cm > 0 ? cm : -1;
         }
-        // the shared colors hold the core and a sentinel entry after it, in a multiple of 16 entries
-        // (local ids stay below 2^18: a warp's batch of finished vertices packs them into 18 bits)
-        int64_t M = std::min<int64_t>({n, static_cast<int64_t>(C.core_max_v) - 16, (int64_t{1} << 18) - 32});
+        // (the shared colors are copied 16 at a time: room for a multiple of 16 that exceeds the core)
+        int64_t M = std::min<int64_t>(n, static_cast<int64_t>(C.core_max_v) - 16);
         if (core_opt > 0) M = std::min<int64_t>(M, core_opt);
         if (M > 0) {
             const int64_t E = core_E;

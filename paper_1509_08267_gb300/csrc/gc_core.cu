@@ -62,9 +62,8 @@ __device__ __forceinline__ unsigned sat8(int32_t c) {
     return c < static_cast<int32_t>(kSat8) ? static_cast<unsigned>(c) : kSat8;
 }
 
-// The core's colors as every block holds them in shared memory: an 8-bit color per vertex and a
-// FINAL bit per vertex; entry m is a sentinel (FINAL, color 255, and not saturated: it reads as no
-// color at all) that the padding slots of a step read.
+// The core's colors as every block holds them in shared memory: an 8-bit color and a FINAL bit per
+// vertex.
 struct Shared {
     uint8_t *col;   // [Mpad]
     unsigned *fin;  // [Mpad / 32 + 1]
@@ -330,7 +329,7 @@ __global__ void __launch_bounds__(kFillThreads) core_fill_kernel(RoundParams P, 
 
 
 // Shared copy of the colors and FINAL bits of [0, m) (16-byte loads; the buffers hold a multiple of
-// 16 that exceeds m), then the sentinel at m.  Ends with a block barrier.
+// 16 that exceeds m).  Ends with a block barrier.
 __device__ __forceinline__ void load_shared(const Shared &S, const CoreParams &Q, const uint8_t *c8, int32_t m) {
     const int32_t n16 = (m + 15) >> 4;
     const uint4 *s4 = reinterpret_cast<const uint4 *>(c8);
@@ -338,11 +337,6 @@ __device__ __forceinline__ void load_shared(const Shared &S, const CoreParams &Q
     for (int32_t i = threadIdx.x; i < n16; i += blockDim.x) d4[i] = __ldcg(s4 + i);
     const int32_t nw = (m >> 5) + 1;
     for (int32_t i = threadIdx.x; i < nw; i += blockDim.x) S.fin[i] = __ldcg(Q.fbits + i);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        S.col[m] = static_cast<uint8_t>(kSat8);
-        S.fin[m >> 5] |= 1u << (m & 31);
-    }
     __syncthreads();
 }
 
@@ -550,7 +544,7 @@ __device__ __forceinline__ unsigned saturated_piece(const int32_t *row, int32_t 
 }
 
 // The vertices a warp finished that are not yet in the round's lists: lane k holds the k-th (v |
-// kPendLose; the core never has 2^18 vertices), its C_{r+1}, its first piece and how many it has.
+// kPendLose), its C_{r+1}, its first piece and how many it has.
 constexpr unsigned kPendLose = 1u << 31;
 struct Pending {
     unsigned v;

@@ -3051,8 +3051,9 @@ cudaError_t launch_setup(const RoundParams &P, int mode, bool batch, int32_t v_b
 }
 
 int32_t sort_shift(int64_t n) {
-    // one block (a plain degree sort) while both state buffers (16 bytes a vertex) fit well inside
-    // L2; blocks of 2^17 ids beyond that
+    // one block (a plain degree sort) up to 6.3M vertices, blocks of 2^17 ids beyond that: measured with
+    // state words of 8 bytes a buffer (the in-place mode's), whose two buffers fit well inside L2 up to
+    // there; the deterministic mode's are 2 bytes and its line may lie higher
     return 16 * n <= (int64_t{96} << 20) ? 30 : 17;
 }
 

@@ -240,7 +240,7 @@ void core_create(gc_server *s, Engine &E) {
         return;
     }
     const int32_t cm = core_max_vertices();
-    const int64_t M = std::min<int64_t>({E.PV, static_cast<int64_t>(cm) - 16, (int64_t{1} << 18) - 32});
+    const int64_t M = std::min<int64_t>(E.PV, static_cast<int64_t>(cm) - 16);
     if (M <= 0) return;
     const size_t Mp = (static_cast<size_t>(M) + 16) & ~size_t{15};
     CoreParams Q{};
