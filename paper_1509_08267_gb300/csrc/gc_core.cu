@@ -4,7 +4,7 @@
 // in adjacency: the high-degree vertices keep conflicting with one another for hundreds of rounds
 // (on R-MAT scale 22, ~100k vertices remain after round 22 and still hold 54M adjacency entries
 // between them, 1.7G over the remaining ~330 rounds).  In the round kernel each of those entries is
-// a dependent gather of a neighbour's state word from L2.  Once the worklist has at most M vertices,
+// a dependent gather of a neighbour's state from L2.  Once the worklist has at most M vertices,
 // this phase numbers them 0..m-1 (the core) and rebuilds each one's row as the list of its
 // neighbours that are still on the worklist, in local ids; neighbours already final never change
 // again, so their colors go once into the vertex's window of final colors.  Every block then keeps
@@ -33,7 +33,8 @@
 // Kernels: core_index_kernel (local ids, records, initial colors), core_fill_kernel (the rows),
 // core_round_kernel (one persistent cooperative launch with one block per SM running the rounds
 // until the worklist is small enough for the tail phase, gc_tail.cu, or empty),
-// core_writeback_kernel (final colors back into the state words).
+// core_writeback_kernel (final colors back into the vertex state), core_return_kernel (a server's core
+// that left early: the unfinished vertices back on the worklist).
 #include <algorithm>
 #include <cstdio>
 #include <cstdlib>
@@ -597,7 +598,7 @@ __device__ __forceinline__ void flush_pending(const CoreParams &Q, const Pending
 // The first core round when the fill computed it (core_fused): a lane per vertex finishes it from
 // its record -- a loser takes the least color absent from the round window and the final window
 // (both below 64), a winner becomes FINAL -- and clears the record's round part; the warp flushes
-// its batch as core_round_warp does.
+// its batch as core_round does.
 template <bool BATCH>
 __device__ void core_first_round(const RoundParams &P, const CoreParams &Q, int32_t m, int pass, unsigned *cn,
                                  int lane, unsigned &st_read, unsigned &st_deg, unsigned &st_cnt) {

@@ -9,7 +9,7 @@
 // Deterministic mode.  Round r's phase 1 reads only C_{r-1}.  Because the conflict test of round
 // r and the First Fit of round r+1 both read C_r, one sweep over a worklist vertex's row does
 // both: it tells whether v lost in round r and, if so, v's color for round r+1.  Colors are
-// double-buffered (col0 / col1), so the result does not depend on the order of the sweep.
+// double-buffered, so the result does not depend on the order of the sweep.
 // In-place mode.  Phase 1 reads and writes one live color array, then a barrier, then phase 2.
 //
 // Work decomposition per round: vertices of degree <= T1 (<= 127) take one thread each (their First
@@ -364,12 +364,12 @@ __device__ __noinline__ bool det_small_exact_lane(const RoundParams &P, const De
 // Returns 1 if the vertex lost, 0 if not, 2 if its exact colors and keys have to tell; nread:
 // entries read.
 //
-// What bounds it: L1 wavefronts (65% busy on a 160^3 stencil; DRAM 38%): a warp's 32 rows lie in 32
+// What bounds it: L1 wavefronts (63% busy on a 160^3 stencil; DRAM 36%): a warp's 32 rows lie in 32
 // places, so a row load costs 32 cache-line lookups whatever its width, and whole-sector loads make
 // the fewest of them.  A least-of-differences instead of a compare per entry and clamped shifts
 // instead of 64-bit windows keep the step at about nine instructions an entry.  256^3 stencil, whole
 // coloring: 8.35 ms, against 16.0 with 16-byte loads, 8-byte state gathers and a key test per entry of
-// equal color; 4,096 graphs of 100..4,000 vertices: 5.4 against 7.4.  (Groups of 4 or 8 lanes per
+// equal color; 64 stencils of 30^3 in a batch: 1.6 against 2.4.  (Groups of 4 or 8 lanes per
 // row, rows in shared memory: 19.4 ms, three times the instructions.)
 template <int W>
 __device__ __forceinline__ int det_small_row(const RoundParams &P, const DetState &S, const Row &r, unsigned self,
@@ -2829,7 +2829,7 @@ __global__ void __launch_bounds__(256) count_mark_kernel(RoundParams P, const in
         if (threadIdx.x == 0) s_max = -1;
         __syncthreads();
     }
-    const bool det = colors_sel != nullptr;  // deterministic mode's byte state
+    const bool det = colors_sel != nullptr;  // deterministic mode's 16-bit state
     const DetState S = det ? det_state(P, *colors_sel + 1) : DetState{nullptr, nullptr};
     const bool copy = out != nullptr && P.err[0] == 0;
     const int64_t count = static_cast<int64_t>(v_end) - v_begin;

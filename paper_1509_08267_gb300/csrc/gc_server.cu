@@ -9,7 +9,8 @@
 // Because every graph's deterministic rounds read only its own previous colors, a request's
 // colors do not depend on which other requests share the launch.  A request large enough to fill
 // the GPU by itself (cfg.solo_entries) skips the pool: between launches the worker colors it alone
-// the way gc_color_ex does, with the core and tail phases that the batch's shared rounds cannot run.
+// the way gc_color_ex does.  The batch's own last rounds run in the core and tail phases while nothing
+// waits: the core leaves its rounds for a submit (engine_step).
 #include <algorithm>
 #include <atomic>
 #include <chrono>

@@ -17,8 +17,8 @@
 //
 // What bounds them: latency -- the row and entry loads of a round (L1 and L2 hits), its barriers, and for
 // the batch the L1 lookups of 32 rows in 32 places.  ER n = 1,000, degree 8 (9 rounds): 30 us of kernel,
-// 291 -> 131 us a call from Python; n = 10,000, degree 16 (12 rounds) on 16 blocks: 73 us, 402 -> 176;
-// 4,096 graphs of 100..4,000 vertices: 5.1 -> 2.46 ms (without the degree sort 5.8; a shared atomic
+// 290 -> 64 us a call from Python; n = 10,000, degree 16 (12 rounds) on 16 blocks: 73 us, 407 -> 123;
+// 4,096 graphs of 100..4,000 vertices: 5.1 -> 2.43 ms (without the degree sort 5.8; a shared atomic
 // per entry of a long row instead of register masks: 4.1).  A single graph past kSmallOneVertices or
 // denser than kSmallOneRow entries a row is left to the core phase, whose 152 blocks then win.
 //
