@@ -199,8 +199,8 @@ struct gc_server {
     double t_create = 0, busy = 0;
     int fatal = GC_OK;
     std::string fatal_msg;
-    volatile int *waiting = nullptr;  // pinned: a request was submitted since the worker last looked
-    std::atomic<int> submitting{0};   // submits under way: their copies may have to wait for running kernels
+    int *waiting = nullptr;          // pinned: a request was submitted since the worker last looked
+    std::atomic<int> submitting{0};  // submits under way: their copies may have to wait for running kernels
 };
 
 namespace gc {
@@ -218,12 +218,16 @@ int srv_fail(gc_server *s, int code, const char *what, cudaError_t e) {
         if (e_ != cudaSuccess) return srv_fail(s, GC_ERR_CUDA, #call, e_); \
     } while (0)
 
+// The word the core reads.  Sequentially consistent, like `submitting`: a worker that clears the word and then
+// sees no submit under way cannot have cleared a later submit's mark.
+void set_waiting(gc_server *s, int x) { __atomic_store_n(s->waiting, x, __ATOMIC_SEQ_CST); }
+
 // A submit under way: the core phase leaves its rounds for it and is not entered until it is done.
 struct Submitting {
     gc_server *s;
     explicit Submitting(gc_server *server) : s(server) {
         s->submitting.fetch_add(1);
-        *s->waiting = 1;
+        set_waiting(s, 1);
     }
     ~Submitting() { s->submitting.fetch_sub(1); }
     Submitting(const Submitting &) = delete;
@@ -236,7 +240,7 @@ int engine_index(int mode) { return mode == GC_MODE_INPLACE ? 1 : 0; }
 // rounds all run in the round kernel.
 void core_create(gc_server *s, Engine &E) {
     void *waiting = nullptr;
-    if (cudaHostGetDevicePointer(&waiting, const_cast<int *>(s->waiting), 0) != cudaSuccess) {
+    if (cudaHostGetDevicePointer(&waiting, s->waiting, 0) != cudaSuccess) {
         cudaGetLastError();
         return;
     }
@@ -757,7 +761,7 @@ void worker_main(gc_server *s) {
                 solo->state = kResident;
             }
             solos = !s->solo.empty();
-            *s->waiting = 0;  // everything submitted so far is in these lists
+            set_waiting(s, 0);  // everything submitted so far is in these lists
             for (int k = 0; k < 2; ++k) {
                 Engine &E = s->eng[k];
                 if (!E.busy()) continue;
@@ -826,7 +830,7 @@ int gc_server_create(const gc_server_config *cfg, gc_server **out) {
     s->solo_min = cfg->solo_entries < 0 ? INT64_MAX : (cfg->solo_entries == 0 ? int64_t{1} << 24 : cfg->solo_entries);
     void *word = nullptr;
     cudaError_t e = cudaHostAlloc(&word, 64, cudaHostAllocPortable | cudaHostAllocMapped);
-    s->waiting = static_cast<volatile int *>(word);
+    s->waiting = static_cast<int *>(word);
     if (e == cudaSuccess) *s->waiting = 0;
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->copy_stream, cudaStreamNonBlocking);
@@ -1005,7 +1009,7 @@ int gc_server_submit(gc_server *s, int32_t n, const int32_t *rowptr, const int32
         s->solo.push_back(raw);
     else
         E.queue.push_back(raw);
-    *s->waiting = 1;
+    gc::set_waiting(s, 1);
     s->cv_work.notify_one();
     return GC_OK;
 }
@@ -1101,7 +1105,7 @@ void gc_server_destroy(gc_server *s) {
     if (s->solo_pool) cudaMemPoolDestroy(s->solo_pool);
     if (s->stream) cudaStreamDestroy(s->stream);
     if (s->copy_stream) cudaStreamDestroy(s->copy_stream);
-    if (s->waiting) cudaFreeHost(const_cast<int *>(s->waiting));
+    if (s->waiting) cudaFreeHost(s->waiting);
     delete s;
 }
 
